@@ -1,5 +1,9 @@
 // Kernels shared by the engines: fixed-rank initial state (Sec. S1.A),
 // assignment-error epilogue (Sec. S3.A) and state precision conversion.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "lr_internal.cuh"
 
 namespace lr {
@@ -38,77 +42,182 @@ __device__ double block_sum(double v, double* sh) {
   return r;
 }
 
-// One block per trajectory: Gaussian padding columns, modified Gram-Schmidt
-// (two passes) against psi and each other, weights 1-(M-1)eps and eps.
-// Works in FP64 in `W` (layout of the state), writes the state as T2.
+// Fixed-rank initial state (Sec. S1.A): psi with weight 1 - (M-1) eps and M - 1
+// padding columns sqrt(eps) q_j, the q_j the Gram-Schmidt orthonormalisation of
+// Gaussian columns against psi and each other. psi is a basis state, so its
+// component is removed by zeroing one row; the rest is Cholesky QR: G = W^dag W
+// = L L^dag over the M - 1 Gaussian columns, Q = W L^-dag, which has the same q_j
+// (a QR factor with a positive diagonal is unique). Everything is FP64. A second
+// round brings the orthogonality from cond(W)^2 2^-53 to 2^-53; `rounds` is 1
+// where it cannot be seen (FP32 states with N >= 4 M: cond(W) < ~3).
+//
+// A cluster of CTAs per trajectory, each on N / C rows in tiles of ITR rows in
+// shared memory: draws and Gram sums of a tile in one sweep, the partial G of the
+// team added in rank order over distributed shared memory, the M x M factor in
+// every CTA, then Q tile by tile. Bound by the FP64 pipe (2 FMA/clk/SM): the draws
+// (~100 FP64 instructions a pair) and the 8 N M^2 FMAs of the two products. Column
+// by column Gram-Schmidt in one block per trajectory took a block sum and a sweep
+// of L2 per column pair: 512 trajectories of N = 2000, M = 20 took 31.5 ms, here
+// 6.3 ms; two trajectories 5.7 ms, here 0.3 ms.
+constexpr int ITR = 128;            // rows per tile
+constexpr int IM = LR_MAX_RANK - 1; // most padding columns
+
+__host__ __device__ inline int init_ldt(int m1) { return m1 | 1; }   // odd row stride: no bank conflicts down a column
+inline size_t init_smem(int m1) {
+  return sizeof(double2) * ((size_t)ITR * init_ldt(m1) + IT + 2 * (size_t)m1 * init_ldt(m1) + (size_t)m1 * (m1 + 1) / 2);
+}
+
 template <typename T2>
 __global__ void __launch_bounds__(IT) initial_state_kernel(const TrajDev* __restrict__ traj, double2* __restrict__ Wbase,
-                                                           T2* __restrict__ Zbase, unsigned long long seed, double eps) {
-  __shared__ double sh[33];
-  const int tj = blockIdx.x;
+                                                           T2* __restrict__ Zbase, unsigned long long seed, double eps,
+                                                           int max_m1, int two_rounds) {
+  extern __shared__ __align__(16) unsigned char init_sm[];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), q = (int)cluster.block_rank(), tj = blockIdx.x / C;
   const TrajDev d = traj[tj];
-  const int N = d.N, M = d.M, ld = d.ld;
+  const int N = d.N, M = d.M, ld = d.ld, M1 = M - 1, ldt = init_ldt(M1);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the layout of the batch's largest rank, the same in every CTA of a cluster
+  double2* tile = reinterpret_cast<double2*>(init_sm);                // [ITR][ldt]
+  double2* gred = tile + (size_t)ITR * init_ldt(max_m1);              // [groups][nep] partial sums
+  double2* L = gred + IT;                                             // [M1][ldt]
+  double2* Li = L + (size_t)max_m1 * init_ldt(max_m1);                // [M1][ldt]  L^-1
+  double2* gsum = Li + (size_t)max_m1 * init_ldt(max_m1);             // [M1 (M1 + 1) / 2]  G over the own rows
+  __shared__ double dinv[IM + 1];
   double2* W = Wbase + d.z_off;
   T2* Z = Zbase + d.z_off;
   const int psi = d.level0 * d.Nr * d.Nf;
+  const int r_lo = (int)((long long)N * q / C), r_hi = (int)((long long)N * (q + 1) / C);
   const unsigned long long ts = splitmix64(seed, (unsigned long long)tj);
-  for (int n = threadIdx.x; n < N; n += IT) {
-    W[(size_t)n * ld] = mk(n == psi ? 1.0 : 0.0, 0.0);
-    for (int j = 1; j < M; ++j) {
-      const unsigned long long pidx = (unsigned long long)(j - 1) * N + n;
-      const double u1 = uniform_open0(ts, 2ull * pidx), u2 = uniform_open0(ts, 2ull * pidx + 1ull);
-      const double r = sqrt(-2.0 * log(u1));
-      double sn, cs;
-      sincospi(2.0 * u2, &sn, &cs);
-      W[(size_t)n * ld + j] = mk(r * cs, r * sn);
+  const double w0 = sqrt(1.0 - M1 * eps), we = sqrt(eps);
+  // column 0, and the rank padding of the row
+  for (int n = r_lo + tid; n < r_hi; n += IT)
+    for (int j = 0; j < ld; ++j)
+      if (j == 0 || j >= M) Z[(size_t)n * ld + j] = mkc<T2>(j == 0 && n == psi ? w0 : 0.0, 0.0);
+  // Gram entry of this thread: pair (gi <= gj) number tid % nep of the upper
+  // triangle, over the rows r = group (mod groups) of every tile
+  const int ne = M1 * (M1 + 1) / 2, nep = (ne + 31) / 32 * 32, groups = nep ? IT / nep : 0;
+  const int ent = nep ? tid % nep : 0, group = nep ? tid / nep : 0;
+  int gj = 0;
+  while ((gj + 1) * (gj + 2) / 2 <= ent) ++gj;
+  const int gi = ent - gj * (gj + 1) / 2;
+  const bool mine = ent < ne && group < groups;
+  for (int round = 0; round < (M1 > 0 ? 1 + two_rounds : 0); ++round) {
+    double gr = 0.0, gim = 0.0;
+    for (int t0 = r_lo; t0 < r_hi; t0 += ITR) {
+      const int rows = min(ITR, r_hi - t0);
+      for (int e = tid; e < rows * M1; e += IT) {
+        const int r = e / M1, j = e - r * M1, n = t0 + r;
+        double2 w;
+        if (round == 0) {
+          const unsigned long long pidx = (unsigned long long)j * N + n;
+          const double u1 = uniform_open0(ts, 2ull * pidx), u2 = uniform_open0(ts, 2ull * pidx + 1ull);
+          const double rad = sqrt(-2.0 * log(u1));
+          double sn, cs;
+          sincospi(2.0 * u2, &sn, &cs);
+          w = n == psi ? mk(0.0, 0.0) : mk(rad * cs, rad * sn);
+          W[(size_t)n * ld + j + 1] = w;
+        } else {
+          w = W[(size_t)n * ld + j + 1];
+        }
+        tile[r * ldt + j] = w;
+      }
+      __syncthreads();
+      if (mine)
+        for (int r = group; r < rows; r += groups) {
+          const double2 a = tile[r * ldt + gi], b = tile[r * ldt + gj];   // conj(a) b
+          gr = fma(a.x, b.x, fma(a.y, b.y, gr));
+          gim = fma(a.x, b.y, fma(-a.y, b.x, gim));
+        }
+      __syncthreads();
     }
-  }
-  __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int j = 1; j < M; ++j) {
-      for (int i = 0; i < j; ++i) {
-        double re = 0.0, im = 0.0;
-        for (int n = threadIdx.x; n < N; n += IT) {
-          const double2 a = W[(size_t)n * ld + i], b = W[(size_t)n * ld + j];   // conj(a) b
-          re += a.x * b.x + a.y * b.y;
-          im += a.x * b.y - a.y * b.x;
-        }
-        re = block_sum<IT>(re, sh);
-        im = block_sum<IT>(im, sh);
-        for (int n = threadIdx.x; n < N; n += IT) {
-          const double2 a = W[(size_t)n * ld + i], b = W[(size_t)n * ld + j];
-          W[(size_t)n * ld + j] = mk(b.x - (re * a.x - im * a.y), b.y - (re * a.y + im * a.x));
-        }
-        __syncthreads();
+    if (mine) gred[group * nep + ent] = mk(gr, gim);
+    __syncthreads();
+    for (int e = tid; e < ne; e += IT) {
+      double2 s = gred[e];
+      for (int g = 1; g < groups; ++g) s = mk(s.x + gred[g * nep + e].x, s.y + gred[g * nep + e].y);
+      gsum[e] = s;
+    }
+    cluster.sync();
+    for (int e = tid; e < ne; e += IT) {   // the team's partials in rank order; lower triangle G_ji = conj(G_ij)
+      double2 s = mk(0.0, 0.0);
+      for (int r = 0; r < C; ++r) {
+        const double2 v = cluster.map_shared_rank(gsum, r)[e];
+        s = mk(s.x + v.x, s.y + v.y);
       }
-      double nn = 0.0;
-      for (int n = threadIdx.x; n < N; n += IT) {
-        const double2 b = W[(size_t)n * ld + j];
-        nn += b.x * b.x + b.y * b.y;
+      int j = 0;
+      while ((j + 1) * (j + 2) / 2 <= e) ++j;
+      L[j * ldt + e - j * (j + 1) / 2] = mk(s.x, -s.y);
+    }
+    cluster.sync();   // every rank has read the partials: they may be overwritten
+    for (int k = 0; k < M1; ++k) {   // right-looking Cholesky, warp 0 on the pivot column
+      if (warp == 0) {
+        const double inv = 1.0 / sqrt(L[k * ldt + k].x);
+        __syncwarp();
+        if (lane == 0) {
+          L[k * ldt + k].x *= inv;
+          dinv[k] = inv;
+        }
+        for (int i = k + 1 + lane; i < M1; i += 32) L[i * ldt + k] = mk(L[i * ldt + k].x * inv, L[i * ldt + k].y * inv);
       }
-      nn = block_sum<IT>(nn, sh);
-      const double inv = 1.0 / sqrt(nn);
-      for (int n = threadIdx.x; n < N; n += IT) {
-        const double2 b = W[(size_t)n * ld + j];
-        W[(size_t)n * ld + j] = mk(b.x * inv, b.y * inv);
+      __syncthreads();
+      const int w = M1 - k - 1;
+      for (int e = tid; e < w * w; e += IT) {
+        const int i = k + 1 + e / w, j = k + 1 + e % w;
+        if (j > i) continue;
+        const double2 a = L[i * ldt + k], c = L[j * ldt + k];   // L_ij -= L_ik conj(L_jk)
+        L[i * ldt + j] = mk(L[i * ldt + j].x - (a.x * c.x + a.y * c.y), L[i * ldt + j].y - (a.y * c.x - a.x * c.y));
       }
       __syncthreads();
     }
-  }
-  const double w0 = sqrt(1.0 - (M - 1) * eps), we = sqrt(eps);
-  for (int n = threadIdx.x; n < N; n += IT) {
-    for (int j = 0; j < ld; ++j) {
-      double2 v = mk(0.0, 0.0);
-      if (j < M) {
-        const double2 q = W[(size_t)n * ld + j];
-        const double s = j == 0 ? w0 : we;
-        v = mk(s * q.x, s * q.y);
+    for (int j = warp; j < M1; j += IT / 32) {   // column j of L^-1 by a warp, lane = row
+      double2 x = mk(lane == j ? 1.0 : 0.0, 0.0);
+      for (int k = j; k < M1; ++k) {
+        double2 xk = mk(__shfl_sync(0xffffffffu, x.x, k), __shfl_sync(0xffffffffu, x.y, k));
+        xk = mk(xk.x * dinv[k], xk.y * dinv[k]);
+        if (lane == k) {
+          x = xk;
+        } else if (lane > k && lane < M1) {
+          const double2 l = L[lane * ldt + k];
+          x = mk(x.x - (l.x * xk.x - l.y * xk.y), x.y - (l.x * xk.y + l.y * xk.x));
+        }
       }
-      if constexpr (sizeof(T2) == sizeof(double2)) {
-        Z[(size_t)n * ld + j] = v;
-      } else {
-        Z[(size_t)n * ld + j] = make_float2((float)v.x, (float)v.y);
+      if (lane >= j && lane < M1) Li[lane * ldt + j] = x;
+    }
+    __syncthreads();
+    // Q[n][j] = sum_{i <= j} W[n][i] conj(L^-1[j][i]): a warp takes 32 rows of a
+    // tile and the columns p and M1 - 1 - p (equal work for every p)
+    const bool last = round == two_rounds;
+    const int np = (M1 + 1) / 2;
+    for (int t0 = r_lo; t0 < r_hi; t0 += ITR) {
+      const int rows = min(ITR, r_hi - t0);
+      for (int e = tid; e < rows * M1; e += IT) {
+        const int r = e / M1, j = e - r * M1;
+        tile[r * ldt + j] = W[(size_t)(t0 + r) * ld + j + 1];
       }
+      __syncthreads();
+      for (int task = warp; task < (ITR / 32) * np; task += IT / 32) {
+        const int r = (task / np) * 32 + lane, p = task % np;
+        if (r >= rows) continue;
+        for (int h = 0; h < 2; ++h) {
+          const int j = h ? M1 - 1 - p : p;
+          if (h && j == p) break;
+          double xr = 0.0, xi = 0.0;
+          for (int i = 0; i <= j; ++i) {
+            const double2 a = tile[r * ldt + i], l = Li[j * ldt + i];   // a conj(l)
+            xr = fma(a.x, l.x, fma(a.y, l.y, xr));
+            xi = fma(a.y, l.x, fma(-a.x, l.y, xi));
+          }
+          const size_t o = (size_t)(t0 + r) * ld + j + 1;
+          if (last) {
+            Z[o] = mkc<T2>(we * xr, we * xi);
+          } else {
+            W[o] = mk(xr, xi);
+          }
+        }
+      }
+      __syncthreads();
     }
   }
 }
@@ -279,14 +388,38 @@ cudaError_t launch_grow(const DevPtrs& dst, const DevPtrs& src, int n_traj, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int /*max_N*/, int prec_fp32,
+template <typename T2>
+static cudaError_t launch_initial_t(const DevPtrs& p, const RunParams& rp, int max_N, int max_M, unsigned long long seed,
+                                    double eps, int two_rounds, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(initial_state_kernel<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)init_smem(IM));
+  if (e != cudaSuccess) return e;
+  // one CTA per SM in all: a team takes the SMs that the batch leaves over, at
+  // least a tile of rows per CTA, within the portable cluster size
+  const int C = std::max(1, std::min({8, sms / std::max(1, rp.n_traj), (max_N + ITR - 1) / ITR}));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C * rp.n_traj);
+  cfg.blockDim = dim3(IT);
+  cfg.dynamicSmemBytes = init_smem(std::max(1, max_M - 1));
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, initial_state_kernel<T2>, p.traj, reinterpret_cast<double2*>(p.Za),
+                            reinterpret_cast<T2*>(p.Zn), seed, eps, std::max(1, max_M - 1), two_rounds);
+}
+
+cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int min_N, int max_N, int max_M, int prec_fp32,
                                  uint64_t seed, double eps, cudaStream_t s) {
-  double2* W = reinterpret_cast<double2*>(p.Za);
-  if (prec_fp32)
-    initial_state_kernel<float2><<<rp.n_traj, IT, 0, s>>>(p.traj, W, reinterpret_cast<float2*>(p.Zn), seed, eps);
-  else
-    initial_state_kernel<double2><<<rp.n_traj, IT, 0, s>>>(p.traj, W, reinterpret_cast<double2*>(p.Zn), seed, eps);
-  return cudaGetLastError();
+  if (prec_fp32) return launch_initial_t<float2>(p, rp, max_N, max_M, seed, eps, min_N < 4 * max_M, s);
+  return launch_initial_t<double2>(p, rp, max_N, max_M, seed, eps, 1, s);
 }
 
 // One block per candidate: trapezoid of |beta_e - beta_g|^2 over the step grid,
