@@ -16,7 +16,7 @@ namespace lr {
 namespace {
 
 struct SmemLayout {
-  int o_zs, o_slot, slot_bytes, s_gp, s_tp, s_pop, o_gd, o_w, o_tred, o_trd, o_xs, o_misc, o_tab;
+  int o_zs, o_slot, slot_bytes, s_gp, s_tp, s_pop, o_gd, o_w, o_tred, o_xs, o_misc, o_tab;
   int o_ta, o_tb, npad, o_gs, total;
 };
 
@@ -41,8 +41,6 @@ SmemLayout layout(int R, int Mp, int zs_smem, size_t es, int tc, int gs) {
   o += al16(Mp * (Mp + 1) * (int)sizeof(double2));
   L.o_tred = o;
   o += al16(2 * Mp * Mp * (int)es);
-  L.o_trd = o;
-  o += al16(Mp * (int)sizeof(double));
   L.o_xs = o;
   o += al16(2 * Mp * Mp * (int)es);
   L.o_misc = o;
@@ -297,7 +295,6 @@ cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunPa
   a.o_gd = L.o_gd;
   a.o_w = L.o_w;
   a.o_tred = L.o_tred;
-  a.o_trd = L.o_trd;
   a.o_xs = L.o_xs;
   a.o_misc = L.o_misc;
   a.o_tab = L.o_tab;

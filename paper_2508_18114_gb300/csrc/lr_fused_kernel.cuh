@@ -7,9 +7,8 @@
 //               (+ level populations and readout photons at recording steps);
 //   B1          one cluster barrier: partials and the new Z_s are visible;
 //   R  (every CTA, redundantly) reduce the C partial slots in rank order,
-//               G = L D L^dag, L^-1, G^-1 = L^-dag D^-1 L^-1 and X_k = G^-1 T_k
-//               (FP64 for the FP64 state; double-word FP32, ~2^-48, for the FP32
-//               state), pre-scaled, conjugate-transposed and rounded to the bulk
+//               G^-1 by symmetric sweeps and X_k = G^-1 T_k (FP64 for the FP64
+//               state; double-word FP32, ~2^-48, for the FP32 state), pre-scaled, conjugate-transposed and rounded to the bulk
 //               precision: XT_r = kappa/2 X_r^dag, XT_b = gamma/2 X_b^dag;
 //   F  (local + DSMEM halo) F = -i H_eff Z_s + (rZ_s) XT_r + (bZ_s) XT_b and the
 //               RK4 stage update; the next stage input goes to the other Z_s
@@ -36,6 +35,7 @@
 #include <cstring>
 
 #include "lr_fused.cuh"
+#include "lr_mm.cuh"
 #include "lr_tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -57,7 +57,7 @@ struct Args {
   int zs_smem;
   // byte offsets in dynamic shared memory
   int o_zs, o_slot, slot_bytes, s_gp, s_tp, s_pop;   // s_*: offsets inside one slot
-  int o_gd, o_w, o_tred, o_trd, o_xs, o_misc, o_tab;
+  int o_gd, o_w, o_tred, o_xs, o_misc, o_tab;
   int o_ta, o_tb, npad;   // tensor-core operand tiles (TC > 0), B rows (2 Mp padded to 16)
   int o_gs;               // Gram on the tensor cores (GRAM_DW == 2): two slice buffers
   const int* order;
@@ -93,132 +93,6 @@ __device__ __forceinline__ Part part_of(const TrajDev& d, int C, int q) {
   P.st = P.nr * d.Nf;
   P.R = d.Nt * P.st;
   return P;
-}
-
-// ----------------------------------------------------------------- double-word accumulation
-// Exact FP32 products (p + e = a*b via FMA) accumulated in an unevaluated
-// sum of two floats (hi + lo): ~2^-48 relative, the FP64-class Gram matrix.
-struct DW {
-  float hi, lo;
-};
-__device__ __forceinline__ void dw_add_prod(DW& s, float a, float b) {
-  const float p = a * b;
-  const float e = fmaf(a, b, -p);
-  const float t = s.hi + p;
-  const float bp = t - s.hi;
-  const float err = (s.hi - (t - bp)) + (p - bp);
-  s.hi = t;
-  s.lo += err + e;
-}
-__device__ __forceinline__ void dw_add(DW& s, const DW& o) {
-  const float t = s.hi + o.hi;
-  const float bp = t - s.hi;
-  const float err = (s.hi - (t - bp)) + (o.hi - bp);
-  s.hi = t;
-  s.lo += err + o.lo;
-}
-__device__ __forceinline__ double dw_value(const DW& s) { return (double)s.hi + (double)s.lo; }
-__device__ __forceinline__ void dw_add_f(DW& s, float x) {   // s += x (Knuth's two-sum into hi)
-  const float t = s.hi + x;
-  const float bp = t - s.hi;
-  s.lo += (s.hi - (t - bp)) + (x - bp);
-  s.hi = t;
-}
-
-// Double-word arithmetic for the M x M phase (Dekker's product via FMA,
-// Knuth's two-sum; results normalised, ~2^-48 relative).
-__device__ __forceinline__ DW dw_make(double x) {
-  DW r;
-  r.hi = (float)x;
-  r.lo = (float)(x - (double)r.hi);
-  return r;
-}
-__device__ __forceinline__ DW dw_sum(DW a, DW b) {
-  const float s = a.hi + b.hi, bb = s - a.hi;
-  float e = (a.hi - (s - bb)) + (b.hi - bb);
-  e += a.lo + b.lo;
-  DW r;
-  r.hi = s + e;
-  r.lo = e - (r.hi - s);
-  return r;
-}
-__device__ __forceinline__ DW dw_neg(DW a) {
-  a.hi = -a.hi;
-  a.lo = -a.lo;
-  return a;
-}
-__device__ __forceinline__ DW dw_mul(DW a, DW b) {
-  const float p = a.hi * b.hi;
-  float e = fmaf(a.hi, b.hi, -p);
-  e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-  DW r;
-  r.hi = p + e;
-  r.lo = e - (r.hi - p);
-  return r;
-}
-// 1/p for p > 0: Newton's iteration r <- r + r (1 - p r) once, in double-word,
-// from the FP32 quotient (24 -> ~48 bits)
-__device__ __forceinline__ DW dw_recip(DW p) {
-  DW r0;
-  r0.hi = 1.0f / p.hi;
-  r0.lo = 0.0f;
-  DW one;
-  one.hi = 1.0f;
-  one.lo = 0.0f;
-  const DW e = dw_sum(one, dw_neg(dw_mul(p, r0)));
-  return dw_sum(r0, dw_mul(r0, e));
-}
-struct DWC {
-  DW re, im;
-};
-// x conj(y)
-__device__ __forceinline__ DWC dwc_mul_conj(const DWC& x, const DWC& y) {
-  DWC r;
-  r.re = dw_sum(dw_mul(x.re, y.re), dw_mul(x.im, y.im));
-  r.im = dw_sum(dw_mul(x.im, y.re), dw_neg(dw_mul(x.re, y.im)));
-  return r;
-}
-// x y
-__device__ __forceinline__ DWC dwc_mul(const DWC& x, const DWC& y) {
-  DWC r;
-  r.re = dw_sum(dw_mul(x.re, y.re), dw_neg(dw_mul(x.im, y.im)));
-  r.im = dw_sum(dw_mul(x.re, y.im), dw_mul(x.im, y.re));
-  return r;
-}
-__device__ __forceinline__ DWC dwc_sub(const DWC& a, const DWC& b) {
-  DWC r;
-  r.re = dw_sum(a.re, dw_neg(b.re));
-  r.im = dw_sum(a.im, dw_neg(b.im));
-  return r;
-}
-__device__ __forceinline__ DWC dwc_add(const DWC& a, const DWC& b) {
-  DWC r;
-  r.re = dw_sum(a.re, b.re);
-  r.im = dw_sum(a.im, b.im);
-  return r;
-}
-__device__ __forceinline__ DWC dwc_scale(const DWC& a, DW s) {
-  DWC r;
-  r.re = dw_mul(a.re, s);
-  r.im = dw_mul(a.im, s);
-  return r;
-}
-// double-word times float (the float exact as a double-word with lo = 0)
-__device__ __forceinline__ DW dw_mul_f(DW a, float b) {
-  const float p = a.hi * b;
-  float e = fmaf(a.hi, b, -p);
-  e = fmaf(a.lo, b, e);
-  DW r;
-  r.hi = p + e;
-  r.lo = e - (r.hi - p);
-  return r;
-}
-// g t for a double-word complex g and an FP32 complex t
-__device__ __forceinline__ DWC dwc_mul_f(const DWC& g, float tx, float ty) {
-  DWC r;
-  r.re = dw_sum(dw_mul_f(g.re, tx), dw_neg(dw_mul_f(g.im, ty)));
-  r.im = dw_sum(dw_mul_f(g.re, ty), dw_mul_f(g.im, tx));
-  return r;
 }
 
 // Reduce-scatter of NV = 2^p partial sums over a warp (recursive halving): at
@@ -343,14 +217,15 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
   const int lds = ZSM ? Mp + 1 : Mp;
   const long long zs_buf = (long long)a.R * lds;  // elements per smem Z_s buffer
 
-  double2* Gd = reinterpret_cast<double2*>(smem + a.o_gd);     // [Mp][Mp+1]  G -> L -> G^-1
-  double2* W = reinterpret_cast<double2*>(smem + a.o_w);       // [Mp][Mp+1]  L^-1
+  // arithmetic and 16-byte entries of the Gram matrix: FP64, or double-word FP32
+  using Ar = typename std::conditional<sizeof(T) == 4, DwArith, F64Arith>::type;
+  using GE = typename Ar::C;
+  GE* Gi = reinterpret_cast<GE*>(smem + a.o_gd);               // [Mp][Mp+1]  G^-1
+  double2* W = reinterpret_cast<double2*>(smem + a.o_w);       // [Mp][Mp+1]  sums of the tensor-core Gram
   T2* Tred = reinterpret_cast<T2*>(smem + a.o_tred);           // [2][Mp*Mp]
-  double* trd = reinterpret_cast<double*>(smem + a.o_trd);     // [Mp] diag of T_r (FP64)
   T2* XT = reinterpret_cast<T2*>(smem + a.o_xs);               // [2][Mp][Mp] (l, m)
-  // misc (FP64 scalars): [0] pulse coefficient, [1] not-PD flag, [8..24) photon
-  // partials per level, [32..64) Im diag T_r, [64..81) reduced populations and
-  // photons, [96..128) 1/L[k][k], [128..131) bulk-precision coefficient and
+  // misc (FP64 scalars): [0] pulse coefficient, [8..24) photon
+  // partials per level, [64..81) reduced populations and photons, [128..131) bulk-precision coefficient and
   // steps, [136..140) mbarriers of the tensor-core Gram, [140] phase-P task
   // counter, [141] tensor-core timeout flag, [142] tensor-core mbarrier, [143]
   // TMEM base address, [144..164) column maxima of the tensor-core Gram
@@ -369,6 +244,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
     }
     __syncthreads();
   }
+  __shared__ MmShared<Ar> mm;   // columns and pivots of the sweeps
   // row-ordered lower-triangle index table: entry e = i(i+1)/2 + j -> (i, j)
   __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
   for (int i = tid; i < LR_MAX_RANK; i += NT)
@@ -531,7 +407,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
         const int par = stage & 1;
         const bool record = stage == 0 && (step % pe) == 0;
         unsigned char* slot = smem + a.o_slot + par * a.slot_bytes;
-        double2* gp = reinterpret_cast<double2*>(slot + a.s_gp);
+        GE* gp = reinterpret_cast<GE*>(slot + a.s_gp);
         T2* tp = reinterpret_cast<T2*>(slot + a.s_tp);
         double* popp = reinterpret_cast<double*>(slot + a.s_pop);
 
@@ -763,8 +639,8 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                     v[k] = keep;
                   }
                 }
-                reinterpret_cast<double*>(gp)[2 * ((i0 + (lane >> 3)) * Mp + j0 + ((lane >> 1) & 3)) + (lane & 1)] =
-                    dw_value(v[0]);
+                reinterpret_cast<DW*>(gp)[2 * ((i0 + (lane >> 3)) * Mp + j0 + ((lane >> 1) & 3)) + (lane & 1)] =
+                    dw_norm(v[0]);
               } else {
                 T gr[TP][TP], gi[TP][TP];
 #pragma unroll
@@ -799,7 +675,11 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                 warp_reduce_scatter(v, lane);
                 if ((lane & ((1 << SH) - 1)) == 0) {
                   const int idx = lane >> SH, e2 = idx >> 1;
-                  reinterpret_cast<double*>(gp)[2 * ((i0 + e2 / TP) * Mp + j0 + e2 % TP) + (idx & 1)] = (double)v[0];
+                  const int o = 2 * ((i0 + e2 / TP) * Mp + j0 + e2 % TP) + (idx & 1);
+                  if constexpr (sizeof(T) == 4)
+                    reinterpret_cast<DW*>(gp)[o] = DW{v[0], 0.f};
+                  else
+                    reinterpret_cast<double*>(gp)[o] = v[0];
                 }
               }
             } else {
@@ -1061,75 +941,28 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
               int ei = 0, ej = 0;
               frexpf(__uint_as_float(gs_cmax[gs_par * 20 + i]), &ei);
               frexpf(__uint_as_float(gs_cmax[gs_par * 20 + j]), &ej);
-              const double sc = ldexp(1.0, ei + ej - 14);
+              const float si = ldexpf(1.0f, ei - 7), sj = ldexpf(1.0f, ej - 7);   // exact scalings
               DW re = Sb[e], im = Sb[420 + i * 20 + j];
               dw_add(re, Sb[210 + e]);
               const DW n2 = Sb[420 + j * 20 + i];
               dw_add(im, DW{-n2.hi, -n2.lo});
-              gp[i * Mp + j] = mk(dw_value(re) * sc, dw_value(im) * sc);
+              re = dw_norm(re);
+              im = dw_norm(im);
+              gp[i * Mp + j] = DWC{{re.hi * si * sj, re.lo * si * sj}, {im.hi * si * sj, im.lo * si * sj}};
             }
           }
         }
         // ================= B1
         cluster.sync();
 
-        // ================= R: reduce in rank order, FP64 Cholesky and inverse
+        // ================= R: reduce in rank order, inverse, X_k
         {
           const int MM = Mp * Mp, MMq = Mq * Mq;
-          for (int e = tid; e < 3 * MMq; e += NT) {
-            const int mat = e / MMq, iq = e - mat * MMq, i = iq / Mq, j = iq - i * Mq, ij = i * Mp + j;
-            if (mat == 0) {
-              if (i > j || j >= M) continue;
-              // issue the remote loads four at a time, then sum in rank order
-              double re = 0.0, im = 0.0;
-              for (int r0 = 0; r0 < C; r0 += 4) {
-                double2 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                  v[u] = r0 + u < C ? cluster.map_shared_rank(gp, r0 + u)[i * Mp + j] : mk(0.0, 0.0);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  re += v[u].x;
-                  im += v[u].y;
-                }
-              }
-              if (i == j) {
-                Gd[i * ldg + i] = mk(re, 0.0);
-              } else {
-                Gd[i * ldg + j] = mk(re, im);
-                Gd[j * ldg + i] = mk(re, -im);
-              }
-            } else {
-              T re = 0, im = 0;
-              for (int r0 = 0; r0 < C; r0 += 4) {
-                T2 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                  v[u] = r0 + u < C ? cluster.map_shared_rank(tp, r0 + u)[(mat - 1) * MM + ij] : cm<T2>(0, 0);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  re += v[u].x;
-                  im += v[u].y;
-                }
-              }
-              Tred[(mat - 1) * MM + ij] = cm<T2>(re, im);
-              if (mat == 1 && i == j) {
-                trd[i] = (double)re;
-                misc[32 + i] = (double)im;
-              }
-            }
-          }
-          if (record && tid < LR_MAX_NT + 1) {
-            double s = 0.0;
-            const bool use = tid < Nt || tid == LR_MAX_NT;
-            if (use)
-              for (int r = 0; r < C; ++r) s += cluster.map_shared_rank(popp, r)[tid];
-            misc[64 + tid] = s;
-          }
+          const int nw = mm_warps(M, NWARP);   // the warps that sweep G
           if (tid == 0) {
-            misc[1] = 0.0;   // not-PD flag
+            mm.bad = 0;
             *reinterpret_cast<int*>(misc + 140) = 0;   // phase-P task counter of the next stage
-            // bulk-precision copies: coefficient, step sizes split as hi + lo
+            // bulk-precision copies: step sizes split as hi + lo
             T* tb = reinterpret_cast<T*>(misc + 128);
             const double hs = stage == 2 ? dt : 0.5 * dt, h6 = dt / 6.0;
             tb[1] = (T)hs;
@@ -1137,220 +970,104 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
             tb[3] = (T)h6;
             tb[4] = (T)(h6 - (double)tb[3]);
           }
-          __syncthreads();
-          if (record && q == 0 && a.p.gsnap) {
-            // FP64 Gram matrix of this record step, for the diagnostics
-            double2* gs = a.p.gsnap + ((size_t)tj * a.rp.n_rec + step / pe) * a.rp.snap_m * a.rp.snap_m;
-            for (int e = tid; e < M * M; e += NT) gs[(e / M) * a.rp.snap_m + e % M] = Gd[(e / M) * ldg + e % M];
-            __syncthreads();   // the M x M phase below overwrites G in place
-          }
-          if (stage == 0 && q == 0 && tid == 0) {
-            double br = 0.0, bi = 0.0;
-            for (int i = 0; i < M; ++i) {
-              br += trd[i];
-              bi += misc[32 + i];
-            }
-            a.p.beta[(size_t)tj * (a.rp.max_steps + 1) + step] = mk(br, bi);
-            if (!isfinite(br) || !isfinite(bi)) set_error(a.p.err, DEV_NONFINITE);
-            if (record) {
-              const long rec = step / pe;
-              double trace = 0.0;
-              for (int lv = 0; lv < a.rp.nt_max; ++lv) {
-                const double v = lv < Nt ? misc[64 + lv] : 0.0;
-                a.p.pops[((size_t)tj * a.rp.n_rec + rec) * a.rp.nt_max + lv] = v;
-                trace += v;
+          if (nw == NWARP || warp >= nw) {
+            // T_k of the team, the partials added in rank order, by the warps that do
+            // not sweep; four remote loads in flight
+            const int n0 = nw == NWARP ? 0 : nw * 32;
+            for (int e = tid - n0; e < 2 * MMq; e += NT - n0) {
+              const int jump = e / MMq, iq = e - jump * MMq, i = iq / Mq, ij = jump * MM + i * Mp + iq - i * Mq;
+              T re = 0, im = 0;
+              for (int r0 = 0; r0 < C; r0 += 4) {
+                T2 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  v[u] = r0 + u < C ? cluster.map_shared_rank(tp, r0 + u)[ij] : cm<T2>(0, 0);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  re += v[u].x;
+                  im += v[u].y;
+                }
               }
-              a.p.nphot[(size_t)tj * a.rp.n_rec + rec] = misc[64 + LR_MAX_NT];
-              a.p.trace[(size_t)tj * a.rp.n_rec + rec] = trace;
+              Tred[ij] = cm<T2>(re, im);
+            }
+            if (record && tid >= NT - 32 && lane < LR_MAX_NT + 1) {
+              double s = 0.0;
+              if (lane < Nt || lane == LR_MAX_NT)
+                for (int r = 0; r < C; ++r) s += cluster.map_shared_rank(popp, r)[lane];
+              misc[64 + lane] = s;
+            }
+          }
+          if (warp < nw) {
+            // the warp's entries G_ij, i >= j, of the team: the partials hold the
+            // upper triangle
+            GE g[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int e = tid + u * NT;
+              g[u] = Ar::zero();
+              if (e < M * (M + 1) / 2) {
+                const int i = tri[e].x, j = tri[e].y, o = j * Mp + i;
+                for (int r0 = 0; r0 < C; r0 += 4) {
+                  GE v[4];
+#pragma unroll
+                  for (int w = 0; w < 4; ++w)
+                    v[w] = r0 + w < C ? cluster.map_shared_rank(gp, r0 + w)[o] : Ar::zero();
+#pragma unroll
+                  for (int w = 0; w < 4; ++w)
+                    if (r0 + w < C) g[u] = r0 + w == 0 ? v[w] : Ar::sum(g[u], v[w]);
+                }
+                g[u] = Ar::conj(g[u]);
+                if (record && q == 0 && a.p.gsnap) {
+                  // FP64 Gram matrix of this record step, for the diagnostics
+                  double2* gs = a.p.gsnap + ((size_t)tj * a.rp.n_rec + step / pe) * a.rp.snap_m * a.rp.snap_m;
+                  const double2 v = Ar::value(g[u]);
+                  gs[i * a.rp.snap_m + j] = mk(v.x, i == j ? 0.0 : v.y);
+                  if (i != j) gs[j * a.rp.snap_m + i] = mk(v.x, -v.y);
+                }
+              }
+            }
+            if (!last) {
+              asm volatile("bar.sync 2, %0;" ::"r"(nw * 32) : "memory");   // mm.bad is clear
+              mm_invert<Ar, NT>(g, Gi, ldg, mm, tri, M, tid);
+            }
+          }
+          __syncthreads();
+          if (tid == 0 && mm.bad) set_error(a.p.err, DEV_NOT_PD);
+          if (stage == 0 && q == 0 && warp == NWARP - 1) {
+            // beta = tr T_r, one lane per diagonal entry, summed over the warp in FP64
+            double br = lane < M ? (double)Tred[lane * Mp + lane].x : 0.0;
+            double bi = lane < M ? (double)Tred[lane * Mp + lane].y : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              br += __shfl_xor_sync(0xffffffffu, br, o);
+              bi += __shfl_xor_sync(0xffffffffu, bi, o);
+            }
+            if (lane == 0) {
+              a.p.beta[(size_t)tj * (a.rp.max_steps + 1) + step] = mk(br, bi);
+              if (!isfinite(br) || !isfinite(bi)) set_error(a.p.err, DEV_NONFINITE);
+              if (record) {
+                const long rec = step / pe;
+                double trace = 0.0;
+                for (int lv = 0; lv < a.rp.nt_max; ++lv) {
+                  const double v = lv < Nt ? misc[64 + lv] : 0.0;
+                  a.p.pops[((size_t)tj * a.rp.n_rec + rec) * a.rp.nt_max + lv] = v;
+                  trace += v;
+                }
+                a.p.nphot[(size_t)tj * a.rp.n_rec + rec] = misc[64 + LR_MAX_NT];
+                a.p.trace[(size_t)tj * a.rp.n_rec + rec] = trace;
+              }
             }
           }
           if (last) break;
-          T2* Gi = reinterpret_cast<T2*>(Gd);   // G^-1 reuses the storage of L once L is no longer needed
-          if constexpr (sizeof(T) == 4) {
-            // FP32 state: the same factorisation and inverse in double-word FP32
-            // (~2^-48 relative, FP64-class like the Gram matrix), on the FP32 pipes:
-            // on this GPU an FP64 warp instruction holds its SMSP's FP64 pipe for
-            // ~60 cycles, and G^-1 is rounded to FP32 at the end anyway. G, L and W
-            // use the storage of their FP64 counterparts (16 bytes per entry).
-            DWC* Gw = reinterpret_cast<DWC*>(Gd);
-            DWC* Ww = reinterpret_cast<DWC*>(W);
-            DW* dinv = reinterpret_cast<DW*>(misc + 96);   // [M] 1 / D[k]
-            float* diag0 = reinterpret_cast<float*>(W);    // W[k][0] slot: the diagonal of G
-            for (int e = tid; e < M * (M + 1) / 2; e += NT) {
-              const int i = tri[e].x, j = tri[e].y;
-              const double2 v = Gd[i * ldg + j];
-              DWC g;
-              g.re = dw_make(v.x);
-              g.im = dw_make(v.y);
-              if (i == j) diag0[i * ldg * 4] = (float)v.x;
-              Gw[i * ldg + j] = g;
-            }
-            // pivot k: breakdown check against the original diagonal, then 1 / D[k]
-            auto pivot = [&](int k) {
-              const DW piv = Gw[k * ldg + k].re;
-              if (!(piv.hi > 1e-13f * diag0[k * ldg * 4]) || !isfinite(piv.hi) || piv.hi < 1e-30f) {
-                misc[1] = 1.0;
-                dinv[k].hi = 1.0f;
-                dinv[k].lo = 0.0f;
-              } else {
-                dinv[k] = dw_recip(piv);
-              }
-            };
-            __syncthreads();
-            if (tid == 0) pivot(0);
-            __syncthreads();
-            for (int k = 0; k < M; ++k) {
-              const DW rk = dinv[k];
-              const int w = M - k - 1;
-              // trailing update G[i][j] -= G[i][k] conj(G[j][k]) / D[k], i >= j > k;
-              // entry 0 (the next pivot) belongs to thread 0, which then forms
-              // 1 / D[k+1] before the barrier: one barrier per elimination step
-              for (int e = tid; e < w * (w + 1) / 2; e += NT) {
-                const int i = k + 1 + tri[e].x, j = k + 1 + tri[e].y;
-                const DWC t = dwc_scale(dwc_mul_conj(Gw[i * ldg + k], Gw[j * ldg + k]), rk);
-                Gw[i * ldg + j] = dwc_sub(Gw[i * ldg + j], t);
-              }
-              if (tid == 0 && k + 1 < M) pivot(k + 1);
-              __syncthreads();
-            }
-            if (tid == 0 && misc[1] != 0.0) set_error(a.p.err, DEV_NOT_PD);
-            // W = L^-1 (unit lower, L[i][k] = G[i][k] / D[k]) by columns: column j
-            // by warp j mod NWARP, lane i = row i, forward substitution
-            // W[i][j] = delta_ij - sum_{j <= k < i} L[i][k] W[k][j] with W[k][j]
-            // broadcast from lane k (no block barrier)
-            for (int j = warp; j < M; j += NWARP) {
-              DWC wv;
-              wv.re.hi = lane == j ? 1.0f : 0.0f;
-              wv.re.lo = wv.im.hi = wv.im.lo = 0.0f;
-              for (int k = j; k < M - 1; ++k) {
-                DWC wk;
-                wk.re.hi = __shfl_sync(0xffffffffu, wv.re.hi, k);
-                wk.re.lo = __shfl_sync(0xffffffffu, wv.re.lo, k);
-                wk.im.hi = __shfl_sync(0xffffffffu, wv.im.hi, k);
-                wk.im.lo = __shfl_sync(0xffffffffu, wv.im.lo, k);
-                if (lane > k && lane < M) wv = dwc_sub(wv, dwc_mul(dwc_scale(Gw[lane * ldg + k], dinv[k]), wk));
-              }
-              if (lane < M) Ww[lane * ldg + j] = wv;
-            }
-            __syncthreads();
-            // G^-1 = W^dag D^-1 W (Hermitian): entry (i, j), i <= j, is
-            // sum_{k >= j} conj(W[k][i]) W[k][j] / D[k], kept in double-word (in the
-            // storage of G, no longer needed): X_k = G^-1 T_k is formed from it in
-            // double-word below, because G^-1 has entries up to 1 / p_M and a product
-            // rounded to FP32 first would lose the small columns to cancellation
-            for (int e = tid; e < M * M; e += NT) {
-              const int i = e / M, j = e - i * M;
-              if (i > j) continue;
-              DWC acc;
-              acc.re.hi = acc.re.lo = acc.im.hi = acc.im.lo = 0.0f;
-              for (int k = j; k < M; ++k)   // W[k][j] conj(W[k][i]) = conj of the term
-                acc = dwc_add(acc, dwc_scale(dwc_mul_conj(Ww[k * ldg + j], Ww[k * ldg + i]), dinv[k]));
-              Gw[i * ldg + j] = acc;
-              if (i != j) {
-                acc.im = dw_neg(acc.im);
-                Gw[j * ldg + i] = acc;
-              }
-            }
-            __syncthreads();
-          } else {
-            // FP64 G = L D L^dag (unit lower L, right-looking, in place in Gd), then
-            // W = L^-1 (unit lower) and G^-1 = W^dag D^-1 W. One FP64 reciprocal per
-            // pivot (formed once and shared: FP64 runs at 2 FMA/clk/SM here) and two
-            // block barriers per elimination step.
-            double* dinv = misc + 96;     // [M] 1 / D[k]
-            // keep the diagonal of G: a pivot below 1e-13 of it is a numerical breakdown
-            for (int k = tid; k < M; k += NT) W[k * ldg] = Gd[k * ldg + k];
-            __syncthreads();
-            for (int k = 0; k < M; ++k) {
-              if (tid == 0) {
-                const double piv = Gd[k * ldg + k].x;
-                if (!(piv > 1e-13 * W[k * ldg].x) || !isfinite(piv) || piv < 1e-30) {
-                  misc[1] = 1.0;
-                  dinv[k] = 1.0;
-                } else {
-                  // reciprocal by Newton-Raphson, r <- r (2 - piv r), from the FP32
-                  // estimate: 24 -> 48 -> 96 correct bits, two FP64 FMA pairs on the
-                  // serial path instead of a full FP64 division
-                  double r = (double)(1.0f / (float)piv);
-                  r = r * fma(-piv, r, 2.0);
-                  r = r * fma(-piv, r, 2.0);
-                  dinv[k] = r;
-                }
-              }
-              __syncthreads();
-              const double rk = dinv[k];
-              const int w = M - k - 1;
-              // trailing update G[i][j] -= G[i][k] conj(G[j][k]) / D[k], i >= j > k
-              for (int e = tid; e < w * (w + 1) / 2; e += NT) {
-                const int i = k + 1 + tri[e].x, j = k + 1 + tri[e].y;
-                const double2 x = Gd[i * ldg + k], y = Gd[j * ldg + k], g = Gd[i * ldg + j];
-                Gd[i * ldg + j] = mk(g.x - rk * (x.x * y.x + x.y * y.y), g.y - rk * (x.y * y.x - x.x * y.y));
-              }
-              __syncthreads();
-            }
-            if (tid == 0 && misc[1] != 0.0) set_error(a.p.err, DEV_NOT_PD);
-            // unit lower L[i][k] = G[i][k] / D[k]; W = L^-1 row by row (unit diagonal)
-            for (int e = tid; e < M * M; e += NT) {
-              const int i = e / M, j = e - i * M;
-              W[i * ldg + j] = mk(i == j ? 1.0 : 0.0, 0.0);
-              if (i > j) {
-                const double2 v = Gd[i * ldg + j];
-                Gd[i * ldg + j] = mk(v.x * dinv[j], v.y * dinv[j]);
-              }
-            }
-            __syncthreads();
-            for (int k = 0; k < M - 1; ++k) {
-              // rows i > k: W[i][j] -= L[i][k] W[k][j], j <= k (W[k] is final)
-              const int rows = M - k - 1;
-              for (int e = tid; e < rows * (k + 1); e += NT) {
-                const int i = k + 1 + e / (k + 1), j = e % (k + 1);
-                const double2 l = Gd[i * ldg + k], wv = W[k * ldg + j], o = W[i * ldg + j];
-                W[i * ldg + j] = mk(o.x - (l.x * wv.x - l.y * wv.y), o.y - (l.x * wv.y + l.y * wv.x));
-              }
-              __syncthreads();
-            }
-            // G^-1 = W^dag D^-1 W (Hermitian), rounded once to the bulk precision
-            for (int e = tid; e < M * M; e += NT) {
-              const int i = e / M, j = e - i * M;
-              if (i > j) continue;
-              double re = 0.0, im = 0.0;
-              for (int k = j; k < M; ++k) {          // W[k][i], W[k][j] nonzero for k >= max(i, j) = j
-                const double2 x = W[k * ldg + i], y = W[k * ldg + j];   // conj(x) y / D[k]
-                re += dinv[k] * (x.x * y.x + x.y * y.y);
-                im += dinv[k] * (x.x * y.y - x.y * y.x);
-              }
-              Gi[i * Mp + j] = cm<T2>((T)re, (T)im);
-              if (i != j) Gi[j * Mp + i] = cm<T2>((T)re, (T)-im);
-            }
-            __syncthreads();
-          }
           // XT_k[l][m] = s_k conj(X_k[m][l]), X_k = G^-1 T_k
           const double sk[2] = {0.5 * d.kappa, 0.5 * d.gamma};
           for (int e = tid; e < 2 * Mq * Mq; e += NT) {
             const int k = e / (Mq * Mq), lq = e - k * (Mq * Mq), l = lq / Mq, m = lq - l * Mq, lm = l * Mp + m;
             T xr = 0, xi = 0;
             if (l < M && m < M) {
-              const T2* Tk = Tred + k * MM;
-              if constexpr (sizeof(T) == 4) {
-                // FP32 state: double-word sums of G^-1 (double-word) times T_k (exact)
-                const DWC* Giw = reinterpret_cast<const DWC*>(Gd);
-                DWC acc;
-                acc.re.hi = acc.re.lo = acc.im.hi = acc.im.lo = 0.0f;
-                for (int j = 0; j < M; ++j) {
-                  const T2 t = Tk[j * Mp + l];
-                  acc = dwc_add(acc, dwc_mul_f(Giw[m * ldg + j], t.x, t.y));
-                }
-                xr = acc.re.hi + acc.re.lo;
-                xi = acc.im.hi + acc.im.lo;
-              } else {
-                for (int j = 0; j < M; ++j) {
-                  const T2 gv = Gi[m * Mp + j];
-                  const T gr = gv.x, gi = gv.y;
-                  const T2 t = Tk[j * Mp + l];
-                  xr = fma(gr, t.x, fma(-gi, t.y, xr));
-                  xi = fma(gr, t.y, fma(gi, t.x, xi));
-                }
-              }
+              const T2 x = mm_xk(Gi + m * ldg, Tred + k * MM + l, Mp, M);
+              xr = x.x;
+              xi = x.y;
             }
             const T s = (T)sk[k];
             XT[k * MM + lm] = cm<T2>(s * xr, -s * xi);

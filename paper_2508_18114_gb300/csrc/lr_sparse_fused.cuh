@@ -28,7 +28,7 @@
 //   P  warp tasks over 4 x 4 tiles: G = Z_s^dag Z_s (upper tiles, exact FP32
 //      products in double-word sums) and T_k = Z_s^dag Y_k (FP32), each tile
 //      summed over all rows and reduced over the warp by recursive halving;
-//   R  G = L D L^dag, L^-1, G^-1 and X_k = G^-1 T_k in double-word FP32
+//   R  G^-1 by symmetric sweeps and X_k = G^-1 T_k in double-word FP32
 //      (~2^-48 relative), XT_k[l][m] = 1/2 conj(X_k[m][l]) rounded to FP32;
 //   F  F = A(t) Z_s (A = -i H_eff: its static diagonal as hi + lo floats, the
 //      other entries by CSR gathers) + sum_k Y_k XT_k and the classical RK4
@@ -36,7 +36,7 @@
 //      Z_s buffer, the accumulator and Z_n are updated in place.
 #include <cooperative_groups.h>
 
-#include "lr_internal.cuh"
+#include "lr_mm.cuh"
 #include "lr_tc.cuh"
 
 namespace lr {
@@ -100,116 +100,6 @@ struct Args {
 };
 
 constexpr int SG_W = 10;   // slicing warps of the tensor-core Gram (warp SG_W issues the MMAs)
-
-struct DW {
-  float hi, lo;
-};
-__device__ __forceinline__ void dw_add_prod(DW& s, float a, float b) {
-  const float p = a * b;
-  const float e = fmaf(a, b, -p);
-  const float t = s.hi + p;
-  const float bp = t - s.hi;
-  const float err = (s.hi - (t - bp)) + (p - bp);
-  s.hi = t;
-  s.lo += err + e;
-}
-__device__ __forceinline__ void dw_add(DW& s, const DW& o) {
-  const float t = s.hi + o.hi;
-  const float bp = t - s.hi;
-  const float err = (s.hi - (t - bp)) + (o.hi - bp);
-  s.hi = t;
-  s.lo += err + o.lo;
-}
-__device__ __forceinline__ void dw_add_f(DW& s, float x) {   // s += x (Knuth's two-sum into hi)
-  const float t = s.hi + x;
-  const float bp = t - s.hi;
-  s.lo += (s.hi - (t - bp)) + (x - bp);
-  s.hi = t;
-}
-__device__ __forceinline__ DW dw_make(double x) {
-  DW r;
-  r.hi = (float)x;
-  r.lo = (float)(x - (double)r.hi);
-  return r;
-}
-__device__ __forceinline__ DW dw_sum(DW a, DW b) {
-  const float s = a.hi + b.hi, bb = s - a.hi;
-  float e = (a.hi - (s - bb)) + (b.hi - bb);
-  e += a.lo + b.lo;
-  DW r;
-  r.hi = s + e;
-  r.lo = e - (r.hi - s);
-  return r;
-}
-__device__ __forceinline__ DW dw_neg(DW a) {
-  a.hi = -a.hi;
-  a.lo = -a.lo;
-  return a;
-}
-__device__ __forceinline__ DW dw_mul(DW a, DW b) {
-  const float p = a.hi * b.hi;
-  float e = fmaf(a.hi, b.hi, -p);
-  e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-  DW r;
-  r.hi = p + e;
-  r.lo = e - (r.hi - p);
-  return r;
-}
-// 1/p for p > 0: one Newton step r + r (1 - p r) in double-word from the FP32 quotient
-__device__ __forceinline__ DW dw_recip(DW p) {
-  DW r0{1.0f / p.hi, 0.0f};
-  const DW one{1.0f, 0.0f};
-  const DW e = dw_sum(one, dw_neg(dw_mul(p, r0)));
-  return dw_sum(r0, dw_mul(r0, e));
-}
-struct DWC {
-  DW re, im;
-};
-__device__ __forceinline__ DWC dwc_mul_conj(const DWC& x, const DWC& y) {   // x conj(y)
-  DWC r;
-  r.re = dw_sum(dw_mul(x.re, y.re), dw_mul(x.im, y.im));
-  r.im = dw_sum(dw_mul(x.im, y.re), dw_neg(dw_mul(x.re, y.im)));
-  return r;
-}
-__device__ __forceinline__ DWC dwc_mul(const DWC& x, const DWC& y) {
-  DWC r;
-  r.re = dw_sum(dw_mul(x.re, y.re), dw_neg(dw_mul(x.im, y.im)));
-  r.im = dw_sum(dw_mul(x.re, y.im), dw_mul(x.im, y.re));
-  return r;
-}
-__device__ __forceinline__ DWC dwc_sub(const DWC& a, const DWC& b) {
-  DWC r;
-  r.re = dw_sum(a.re, dw_neg(b.re));
-  r.im = dw_sum(a.im, dw_neg(b.im));
-  return r;
-}
-__device__ __forceinline__ DWC dwc_add(const DWC& a, const DWC& b) {
-  DWC r;
-  r.re = dw_sum(a.re, b.re);
-  r.im = dw_sum(a.im, b.im);
-  return r;
-}
-__device__ __forceinline__ DWC dwc_scale(const DWC& a, DW s) {
-  DWC r;
-  r.re = dw_mul(a.re, s);
-  r.im = dw_mul(a.im, s);
-  return r;
-}
-__device__ __forceinline__ DW dw_mul_f(DW a, float b) {   // b exact as a double-word
-  const float p = a.hi * b;
-  float e = fmaf(a.hi, b, -p);
-  e = fmaf(a.lo, b, e);
-  DW r;
-  r.hi = p + e;
-  r.lo = e - (r.hi - p);
-  return r;
-}
-__device__ __forceinline__ DWC dwc_mul_f(const DWC& g, float tx, float ty) {
-  DWC r;
-  r.re = dw_sum(dw_mul_f(g.re, tx), dw_neg(dw_mul_f(g.im, ty)));
-  r.im = dw_sum(dw_mul_f(g.re, ty), dw_mul_f(g.im, tx));
-  return r;
-}
 
 __device__ __forceinline__ void load4(const float2* p, float2 (&v)[4]) {
   const float4 x = reinterpret_cast<const float4*>(p)[0], y = reinterpret_cast<const float4*>(p)[1];
@@ -390,6 +280,7 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
   __shared__ __align__(8) unsigned long long gbar_s[5];
   __shared__ uint32_t gslot;
   __shared__ uint32_t gcmax[2][20];
+  __shared__ MmShared<DwArith> mm;   // columns and pivots of the sweeps
   __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
   __shared__ float2 chi[NCH];
   __shared__ double red[NWARP * 4];
@@ -427,14 +318,13 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
     tc_fence_after();
     tmem = gslot;
   }
-  double2* Gd = reinterpret_cast<double2*>(smem + a.o_gd);   // [Mp][Mp+1]  G -> L -> G^-1
-  double2* W = reinterpret_cast<double2*>(smem + a.o_w);     // [Mp][Mp+1]  L^-1
+  DWC* Gi = reinterpret_cast<DWC*>(smem + a.o_gd);           // [Mp][Mp+1]  G^-1
+  double2* W = reinterpret_cast<double2*>(smem + a.o_w);     // [Mp][Mp+1]  sums of the tensor-core Gram
   float2* Tred = reinterpret_cast<float2*>(smem + a.o_tred);  // [K][Mp*Mp]  T_k over this CTA's rows
   float2* XT = reinterpret_cast<float2*>(smem + a.o_xt);      // [K][Mp][Mp] (l, m)
-  // [0] not-PD flag, [8..11) signal partials (Re, Im beta, photons), [32..64) 1/D,
-  // [64..96) population partials
+  // [8..11) signal partials (Re, Im beta, photons), [64..96) population partials
   double* misc = reinterpret_cast<double*>(smem + a.o_misc);
-  double2* gpart = reinterpret_cast<double2*>(smem + a.o_gpart);   // [Mp][Mp]  G over this CTA's rows
+  DWC* gpart = reinterpret_cast<DWC*>(smem + a.o_gpart);           // [Mp][Mp]  G (i <= j) over this CTA's rows
   float2* tsum = reinterpret_cast<float2*>(smem + a.o_tsum);       // [K][Mp*Mp]  T_k of the team
   cg::cluster_group cluster = cg::this_cluster();
   const int C = TEAM ? a.C : 1;
@@ -620,7 +510,7 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
       // G over the own rows from V: S[a][b] = V[a][b] + V[b][a] for the 820
       // entries G needs ([0, 210) (i, j), [210, 420) (20+i, 20+j), i <= j;
       // [420, 820) (i, 20+j)), then G_ij = 2^(e_i + e_j - 14) (S[i][j] +
-      // S[20+i][20+j] + i (S[i][20+j] - S[j][20+i])) into gpart, both triangles
+      // S[20+i][20+j] + i (S[i][20+j] - S[j][20+i])) into gpart
       DW* Sb = reinterpret_cast<DW*>(W);
       const int gt = tid;   // 0 .. SG_W * 32 - 1
       for (int e = gt; e < 820; e += SG_W * 32) {
@@ -643,14 +533,14 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
         int ei = 0, ej = 0;
         frexpf(__uint_as_float(gcmax[gpar][i]), &ei);
         frexpf(__uint_as_float(gcmax[gpar][j]), &ej);
-        const double sc = ldexp(1.0, ei + ej - 14);
+        const float si = ldexpf(1.0f, ei - 7), sj = ldexpf(1.0f, ej - 7);   // exact scalings
         DW re = Sb[e], im = Sb[420 + i * 20 + j];
         dw_add(re, Sb[210 + e]);
         const DW n2 = Sb[420 + j * 20 + i];
         dw_add(im, DW{-n2.hi, -n2.lo});
-        const double gr = ((double)re.hi + (double)re.lo) * sc, gi = ((double)im.hi + (double)im.lo) * sc;
-        gpart[i * Mp + j] = make_double2(gr, gi);
-        gpart[j * Mp + i] = make_double2(gr, -gi);
+        re = dw_norm(re);
+        im = dw_norm(im);
+        gpart[i * Mp + j] = DWC{{re.hi * si * sj, re.lo * si * sj}, {im.hi * si * sj, im.lo * si * sj}};
       }
     } else if (warp == SG_W) {
       // the issuing warp
@@ -883,17 +773,11 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
                 dw_add(keep, t);
               });
               const int i = i0 + (lane >> 3), j = j0 + ((lane >> 1) & 3), c = lane & 1;
-              const double val = (double)v[0].hi + (double)v[0].lo;
-              // G[i][j] and its conjugate G[j][i] over this CTA's rows (the diagonal's
-              // imaginary part is zero), summed over the row blocks in order
-              double* gp = reinterpret_cast<double*>(gpart);
-              if (i < j) {
-                const double lower = c ? -val : val;
-                gp[2 * (i * Mp + j) + c] = blk ? gp[2 * (i * Mp + j) + c] + val : val;
-                gp[2 * (j * Mp + i) + c] = blk ? gp[2 * (j * Mp + i) + c] + lower : lower;
-              } else if (i == j) {
-                const double d = c ? 0.0 : val;
-                gp[2 * (i * Mp + i) + c] = blk ? gp[2 * (i * Mp + i) + c] + d : d;
+              // G[i][j] over this CTA's rows, summed over the row blocks in order
+              if (i <= j) {
+                DW* gp = reinterpret_cast<DW*>(gpart) + 2 * (i * Mp + j) + c;
+                const DW val = i == j && c ? DW{0.f, 0.f} : dw_norm(v[0]);
+                *gp = blk ? dw_sum(*gp, val) : val;
               }
             } else {
               const int t2 = task - n_g, k = t2 / (nt_ * nt_), r2 = t2 - k * nt_ * nt_, ti = r2 / nt_,
@@ -942,110 +826,48 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
         // ================= B1: the team's partials are visible
         team_sync();
         if (stage == 0) publish(step, record);
-        // ================= R: G = L D L^dag, L^-1, G^-1 (double-word FP32), XT_k
+        // ================= R: G^-1 by symmetric sweeps (double-word FP32), XT_k
         {
-          DWC* Gw = reinterpret_cast<DWC*>(Gd);
-          DWC* Ww = reinterpret_cast<DWC*>(W);
-          DW* dinv = reinterpret_cast<DW*>(misc + 32);   // [M] 1 / D[k]
-          float* diag0 = reinterpret_cast<float*>(W);    // W[k][0] slot: the diagonal of G
-          if (tid == 0) misc[0] = 0.0;
-          // T_k of the team: the partials added in rank order (the same in every CTA)
-          for (int e = tid; e < K * MM; e += NT) {
-            float2 v = at_rank(Tred, 0)[e];
-            for (int r = 1; r < C; ++r) {
-              const float2 u = at_rank(Tred, r)[e];
-              v.x += u.x;
-              v.y += u.y;
+          const int nw = mm_warps(M, NWARP);   // the warps that sweep G
+          if (tid == 0) mm.bad = 0;
+          if (nw == NWARP || warp >= nw) {
+            // T_k of the team: the partials added in rank order (the same in every
+            // CTA), by the warps that do not sweep
+            const int n0 = nw == NWARP ? 0 : nw * 32;
+            for (int e = tid - n0; e < K * MM; e += NT - n0) {
+              float2 v = at_rank(Tred, 0)[e];
+              for (int r = 1; r < C; ++r) {
+                const float2 u = at_rank(Tred, r)[e];
+                v.x += u.x;
+                v.y += u.y;
+              }
+              tsum[e] = v;
             }
-            tsum[e] = v;
           }
-          for (int e = tid; e < M * (M + 1) / 2; e += NT) {
-            const int i = tri[e].x, j = tri[e].y;
-            double2 v = at_rank(gpart, 0)[i * Mp + j];
-            for (int r = 1; r < C; ++r) {
-              const double2 u = at_rank(gpart, r)[i * Mp + j];
-              v.x += u.x;
-              v.y += u.y;
+          if (warp < nw) {
+            DWC g[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int e = tid + u * NT;
+              g[u] = DwArith::zero();
+              if (e < M * (M + 1) / 2) {
+                const int i = tri[e].x, j = tri[e].y, o = j * Mp + i;
+                g[u] = at_rank(gpart, 0)[o];
+                for (int r = 1; r < C; ++r) g[u] = DwArith::sum(g[u], at_rank(gpart, r)[o]);
+                g[u] = DwArith::conj(g[u]);   // G_ij, i >= j
+              }
             }
-            DWC g;
-            g.re = dw_make(v.x);
-            g.im = dw_make(v.y);
-            if (i == j) diag0[i * ldg * 4] = (float)v.x;
-            Gw[i * ldg + j] = g;
-          }
-          auto pivot = [&](int k) {
-            const DW piv = Gw[k * ldg + k].re;
-            if (!(piv.hi > 1e-13f * diag0[k * ldg * 4]) || !isfinite(piv.hi) || piv.hi < 1e-30f) {
-              misc[0] = 1.0;
-              dinv[k] = DW{1.0f, 0.0f};
-            } else {
-              dinv[k] = dw_recip(piv);
-            }
-          };
-          __syncthreads();
-          if (tid == 0) pivot(0);
-          __syncthreads();
-          for (int k = 0; k < M; ++k) {
-            const DW rk = dinv[k];
-            const int w = M - k - 1;
-            for (int e = tid; e < w * (w + 1) / 2; e += NT) {
-              const int i = k + 1 + tri[e].x, j = k + 1 + tri[e].y;
-              const DWC t = dwc_scale(dwc_mul_conj(Gw[i * ldg + k], Gw[j * ldg + k]), rk);
-              Gw[i * ldg + j] = dwc_sub(Gw[i * ldg + j], t);
-            }
-            if (tid == 0 && k + 1 < M) pivot(k + 1);
-            __syncthreads();
-          }
-          if (tid == 0 && misc[0] != 0.0) set_error(a.err, DEV_NOT_PD);
-          // W = L^-1 by columns (warp j mod NWARP, lane i = row i)
-          for (int j = warp; j < M; j += NWARP) {
-            DWC wv;
-            wv.re.hi = lane == j ? 1.0f : 0.0f;
-            wv.re.lo = wv.im.hi = wv.im.lo = 0.0f;
-            for (int k = j; k < M - 1; ++k) {
-              DWC wk;
-              wk.re.hi = __shfl_sync(0xffffffffu, wv.re.hi, k);
-              wk.re.lo = __shfl_sync(0xffffffffu, wv.re.lo, k);
-              wk.im.hi = __shfl_sync(0xffffffffu, wv.im.hi, k);
-              wk.im.lo = __shfl_sync(0xffffffffu, wv.im.lo, k);
-              if (lane > k && lane < M) wv = dwc_sub(wv, dwc_mul(dwc_scale(Gw[lane * ldg + k], dinv[k]), wk));
-            }
-            if (lane < M) Ww[lane * ldg + j] = wv;
+            asm volatile("bar.sync 2, %0;" ::"r"(nw * 32) : "memory");   // mm.bad is clear
+            mm_invert<DwArith, NT>(g, Gi, ldg, mm, tri, M, tid);
           }
           __syncthreads();
-          // G^-1 = W^dag D^-1 W in double-word, into the storage of L (no longer needed)
-          for (int e = tid; e < M * M; e += NT) {
-            const int i = e / M, j = e - i * M;
-            if (i > j) continue;
-            DWC acc;
-            acc.re.hi = acc.re.lo = acc.im.hi = acc.im.lo = 0.0f;
-            for (int k = j; k < M; ++k)
-              acc = dwc_add(acc, dwc_scale(dwc_mul_conj(Ww[k * ldg + j], Ww[k * ldg + i]), dinv[k]));
-            Gw[i * ldg + j] = acc;
-            if (i != j) {
-              acc.im = dw_neg(acc.im);
-              Gw[j * ldg + i] = acc;
-            }
-          }
-          __syncthreads();
-          // XT_k[l][m] = 1/2 conj(X_k[m][l]), X_k = G^-1 T_k (the 1/2 of Eq. S5), in
-          // double-word sums: G^-1 has entries up to 1 / p_M, and a product rounded
-          // to FP32 first would lose the small columns to cancellation
+          if (tid == 0 && mm.bad) set_error(a.err, DEV_NOT_PD);
+          // XT_k[l][m] = 1/2 conj(X_k[m][l]), X_k = G^-1 T_k (the 1/2 of Eq. S5)
           for (int e = tid; e < K * Mq * Mq; e += NT) {
             const int k = e / (Mq * Mq), lq = e - k * (Mq * Mq), l = lq / Mq, m = lq - l * Mq;
-            float xr = 0.f, xi = 0.f;
-            if (l < M && m < M) {
-              const float2* Tk = tsum + k * MM;
-              DWC acc;
-              acc.re.hi = acc.re.lo = acc.im.hi = acc.im.lo = 0.0f;
-              for (int j = 0; j < M; ++j) {
-                const float2 t = Tk[j * Mp + l];
-                acc = dwc_add(acc, dwc_mul_f(Gw[m * ldg + j], t.x, t.y));
-              }
-              xr = acc.re.hi + acc.re.lo;
-              xi = acc.im.hi + acc.im.lo;
-            }
-            XT[k * MM + l * Mp + m] = make_float2(0.5f * xr, -0.5f * xi);
+            float2 x = make_float2(0.f, 0.f);
+            if (l < M && m < M) x = mm_xk(Gi + m * ldg, tsum + k * MM + l, Mp, M);
+            XT[k * MM + l * Mp + m] = make_float2(0.5f * x.x, -0.5f * x.y);
           }
           __syncthreads();
         }
