@@ -47,6 +47,7 @@ constexpr int NT = 384;       // threads of the tensor-core variants (12 warps: 
 constexpr int NWARP = NT / 32;
 constexpr int NT_CC = 512;    // threads of the CUDA-core variants (16 warps at <= 128 registers)
 __host__ __device__ constexpr int threads_for(int tc) { return tc > 0 ? NT : NT_CC; }
+constexpr int DRIVE_STEPS = 8;   // RK4 steps whose drive coefficients are formed at once (3 per step, <= 32 lanes)
 constexpr int TAB = 64;   // mode truncations handled by the fused engine: N_t, N_r, N_f < 64
 
 struct Args {
@@ -155,6 +156,16 @@ __device__ __forceinline__ void store4(T2* p, const T2 (&v)[4]) {
   }
 }
 
+// One or four consecutive complex values.
+template <int ZSM, typename T2>
+__device__ __forceinline__ void loadu(const T2* p, T2 (&v)[4]) { load4<ZSM>(p, v); }
+template <int ZSM, typename T2>
+__device__ __forceinline__ void loadu(const T2* p, T2 (&v)[1]) { v[0] = *p; }
+template <int ZSM, typename T2>
+__device__ __forceinline__ void storeu(T2* p, const T2 (&v)[4]) { store4<ZSM>(p, v); }
+template <int ZSM, typename T2>
+__device__ __forceinline__ void storeu(T2* p, const T2 (&v)[1]) { *p = v[0]; }
+
 // ----------------------------------------------------------------- tcgen05 helpers
 // Operand tiles are K-major without swizzle: 8-row x 16-byte core matrices,
 // rows of a core 16 bytes apart, cores of consecutive 8-row groups 128 bytes
@@ -188,7 +199,6 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
   static_assert(TC == 0 || (ZSM == 0 && sizeof(T2) == 8), "tensor-core projection: FP32 state in L2 only");
   using T = typename Real<T2>::t;
   constexpr int TP = sizeof(T) == 4 ? 4 : 2;     // phase-P tile edge
-  constexpr int TR = sizeof(T) == 4 ? 5 : 2;     // phase-F rows per thread tile
   // first step of this launch: the device step counter (so that a replayed
   // capture of the launch continues the pulse run), else the argument
   const long step0 = a.p.dstep ? (long)*a.p.dstep : a.step0;
@@ -224,9 +234,8 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
   double2* W = reinterpret_cast<double2*>(smem + a.o_w);       // [Mp][Mp+1]  sums of the tensor-core Gram
   T2* Tred = reinterpret_cast<T2*>(smem + a.o_tred);           // [2][Mp*Mp]
   T2* XT = reinterpret_cast<T2*>(smem + a.o_xs);               // [2][Mp][Mp] (l, m)
-  // misc (FP64 scalars): [0] pulse coefficient, [8..24) photon
-  // partials per level, [64..81) reduced populations and photons, [128..131) bulk-precision coefficient and
-  // steps, [136..140) mbarriers of the tensor-core Gram, [140] phase-P task
+  // misc (FP64 scalars): [8..24) photon partials per level, [64..81) reduced
+  // populations and photons, [128..131) bulk-precision step sizes, [136..140) mbarriers of the tensor-core Gram, [140] phase-P task
   // counter, [141] tensor-core timeout flag, [142] tensor-core mbarrier, [143]
   // TMEM base address, [144..164) column maxima of the tensor-core Gram
   double* misc = reinterpret_cast<double*>(smem + a.o_misc);
@@ -262,6 +271,18 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
 
   const double dt = a.rp.dt;
   const int pe = a.rp.pop_every;
+  // drive coefficient c(t) (rotating frame: complex weight) at t, t + dt/2 and
+  // t + dt of the next DRIVE_STEPS steps
+  __shared__ T2 drive[3 * DRIVE_STEPS];
+  if (tid == 0) {
+    // bulk-precision step sizes dt/2, dt, dt/6, split as hi + lo
+    T* tb = reinterpret_cast<T*>(misc + 128);
+    const double h[3] = {0.5 * dt, dt, dt / 6.0};
+    for (int k = 0; k < 3; ++k) {
+      tb[2 * k] = (T)h[k];
+      tb[2 * k + 1] = (T)(h[k] - (double)tb[2 * k]);
+    }
+  }
 
   // ---- tensor-core projection: operand tiles, D staging, TMEM and its mbarrier
   float* ta_big = reinterpret_cast<float*>(smem + a.o_ta);
@@ -401,7 +422,8 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
 
     int cur = 0;
     const long s_end = step0 + a.n_steps;
-    for (long step = step0;; ++step) {
+    int drive_step = 0;   // step within the drive table
+    for (long step = step0;; ++step, ++drive_step) {
       const bool last = step == s_end;
       for (int stage = 0; stage < 4; ++stage) {
         const int par = stage & 1;
@@ -419,22 +441,21 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
           // arithmetic is independent of which warp runs it, so results stay bitwise
           // reproducible
           int* task_ctr = reinterpret_cast<int*>(misc + 140);
-          if (tid == NT - 1) {
-            // drive coefficient of this stage (FP64 pulse shape), off the serial
-            // M x M phase: read by phase F after the barriers that follow
-            const double ts = (double)step * dt + (stage == 0 ? 0.0 : (stage == 3 ? dt : 0.5 * dt));
+          if (stage == 0 && drive_step == DRIVE_STEPS) drive_step = 0;
+          if (stage == 0 && drive_step == 0 && warp == NWARP - 1 && lane < 3 * DRIVE_STEPS) {
+            // drive coefficients of the next DRIVE_STEPS steps, one lane per stage time:
+            // the FP64 pulse shape takes ~12k cycles of one warp (64 cycles per FP64 warp
+            // instruction), whatever the number of lanes; read by phase F after the
+            // barriers that follow
+            const int k = lane % 3;
+            const double ts = (double)(step + lane / 3) * dt + (k == 0 ? 0.0 : (k == 2 ? dt : 0.5 * dt));
             if (FRAME) {
               // RWA drive w r + conj(w) r^dag, w = (Omega/2) e^{i phi}
               const double2 w = pulse_rwa_drive(pulse, a.rp.tau, ts);
-              misc[0] = w.x;
-              misc[2] = w.y;
+              drive[lane] = cm<T2>((T)w.x, (T)w.y);
             } else {
-              misc[0] = pulse_coefficient(pulse, a.rp.tau, ts);
-              misc[2] = 0.0;
+              drive[lane] = cm<T2>((T)pulse_coefficient(pulse, a.rp.tau, ts), 0);
             }
-            T* tb = reinterpret_cast<T*>(misc + 128);
-            tb[0] = (T)misc[0];
-            tb[5] = (T)misc[2];
           }
           if constexpr (GRAM_DW == 2) {
             // ---- Gram on the tensor cores. GS_W warps slice the chunks of GS_CH
@@ -962,13 +983,6 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
           if (tid == 0) {
             mm.bad = 0;
             *reinterpret_cast<int*>(misc + 140) = 0;   // phase-P task counter of the next stage
-            // bulk-precision copies: step sizes split as hi + lo
-            T* tb = reinterpret_cast<T*>(misc + 128);
-            const double hs = stage == 2 ? dt : 0.5 * dt, h6 = dt / 6.0;
-            tb[1] = (T)hs;
-            tb[2] = (T)(hs - (double)tb[1]);
-            tb[3] = (T)h6;
-            tb[4] = (T)(h6 - (double)tb[3]);
           }
           if (nw == NWARP || warp >= nw) {
             // T_k of the team, the partials added in rank order, by the warps that do
@@ -1096,13 +1110,14 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
         {
           // coefficient and split step sizes h = hi + lo (no systematic FP32 step error)
           const T* tb = reinterpret_cast<const T*>(misc + 128);
-          const T c = tb[0], hs_hi = tb[1], hs_lo = tb[2], h6_hi = tb[3], h6_lo = tb[4], ci = tb[5];
+          const T2 drv = drive[3 * drive_step + (stage == 0 ? 0 : (stage == 3 ? 2 : 1))];
+          const T c = drv.x, ci = drv.y;
+          const T hs_hi = tb[stage == 2 ? 2 : 0], hs_lo = tb[stage == 2 ? 3 : 1], h6_hi = tb[4], h6_lo = tb[5];
           constexpr bool rwa = FRAME != 0;
           // Z_n rows start on 16-byte boundaries for the paired FP32 accesses
           const bool zn_vec = sizeof(T2) == 8 && (M % 2) == 0 && (d.z_off % 2) == 0;
           const int nxt = cur ^ 1;
           const int mq = Mq / 4;
-          const int nrt_all = (P.R + TR - 1) / TR;
           const T g = (T)d.g, J = (T)d.J, ka = (T)d.kappa, ga = (T)d.gamma;
           const int MM = Mp * Mp;
           if constexpr (TC > 0) {
@@ -1373,17 +1388,19 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
               }
             }
           } else {
-          const int nrt = nrt_all;
-          const int row_lo = 0;
-          for (int tile = tid; tile < nrt * mq; tile += NT) {
-            const int rt = tile / mq, m0 = (tile - rt * mq) * 4;
+          // tiles of TR rows x TU columns, one per thread
+          auto tiles = [&](auto trc, auto tuc) {
+          constexpr int TR = decltype(trc)::value, TU = decltype(tuc)::value;
+          const int nrt = (P.R + TR - 1) / TR, ncol = TU == 4 ? mq : M;
+          for (int tile = tid; tile < nrt * ncol; tile += NT) {
+            const int rt = tile / ncol, m0 = (tile - rt * ncol) * TU;
             float cmx[4] = {0.f, 0.f, 0.f, 0.f};   // column maxima of the rows written (tensor-core Gram)
-            T fr[TR][4], fi[TR][4];
+            T fr[TR][TU], fi[TR][TU];
             T sr[TR], sb[TR];
             const T2* yrp[TR];
             const T2* ybp[TR];
             int nrow[TR];
-            const int l0 = row_lo + rt * TR;
+            const int l0 = rt * TR;
             int it = l0 / P.st, irl = (l0 - it * P.st) / Nf, iff = l0 - it * P.st - irl * Nf;
 #pragma unroll
             for (int r = 0; r < TR; ++r) {
@@ -1394,7 +1411,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
               ybp[r] = own(cur, 0);
               nrow[r] = -1;
 #pragma unroll
-              for (int u = 0; u < 4; ++u) fr[r][u] = fi[r][u] = 0;
+              for (int u = 0; u < TU; ++u) fr[r][u] = fi[r][u] = 0;
               if (l < P.R) {
                 const int ir = P.r_lo + irl;
                 const int iro = three ? iff : ir;
@@ -1413,29 +1430,29 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                   dl = er + dtab[(0 * TAB + it) * 2 + 1] + dtab[(1 * TAB + ir) * 2 + 1] + dtab[(2 * TAB + iff) * 2 + 1];
                 }
                 const T dim_ = (T)(-0.5) * (ka * (T)iro + ga * (T)it);
-                T2 z[4];
-                load4<ZSM>(own(cur, l) + m0, z);
-                T hr[4], hi[4];
+                T2 z[TU];
+                loadu<ZSM>(own(cur, l) + m0, z);
+                T hr[TU], hi[TU];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < TU; ++u) {
                   hr[u] = fma(dh, z[u].x, fma(dl, z[u].x, -dim_ * z[u].y));
                   hi[u] = fma(dh, z[u].y, fma(dl, z[u].y, dim_ * z[u].x));
                 }
                 auto add_row = [&](const T2* vp, T w) {
-                  T2 v[4];
-                  load4<ZSM>(vp, v);
+                  T2 v[TU];
+                  loadu<ZSM>(vp, v);
 #pragma unroll
-                  for (int u = 0; u < 4; ++u) {
+                  for (int u = 0; u < TU; ++u) {
                     hr[u] = fma(w, v[u].x, hr[u]);
                     hi[u] = fma(w, v[u].y, hi[u]);
                   }
                 };
                 // complex weight wr + i wi (the rotating-frame drive)
                 auto add_row_c = [&](const T2* vp, T wr, T wi) {
-                  T2 v[4];
-                  load4<ZSM>(vp, v);
+                  T2 v[TU];
+                  loadu<ZSM>(vp, v);
 #pragma unroll
-                  for (int u = 0; u < 4; ++u) {
+                  for (int u = 0; u < TU; ++u) {
                     hr[u] = fma(wr, v[u].x, fma(-wi, v[u].y, hr[u]));
                     hi[u] = fma(wr, v[u].y, fma(wi, v[u].x, hi[u]));
                   }
@@ -1508,7 +1525,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                 }
                 // F = -i H_eff z
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < TU; ++u) {
                   fr[r][u] = hi[u];
                   fi[r][u] = -hr[u];
                 }
@@ -1531,7 +1548,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
               }
             }
             // projection terms: + sr (rZ_s) XT_r + sb (bZ_s) XT_b
-            if constexpr (TC == 0 && ZSM == 0 && sizeof(T2) == 8) {
+            if constexpr (ZSM == 0 && sizeof(T2) == 8) {
               // FP32 state in L2: k in pairs with 16-byte loads of the Y rows
               // (Mp-wide, 32-byte aligned) and of XT; the padding columns and rows
               // up to Mp are zero, and every accumulator sees the same k order
@@ -1557,18 +1574,18 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                     const T y1x = kk ? yb2[r].z : yb2[r].x, y1y = kk ? yb2[r].w : yb2[r].y;
                     const T ar = sr[r] * y0x, ai = sr[r] * y0y, br = sb[r] * y1x, bi = sb[r] * y1y;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < TU; ++u) {
                       fr[r][u] = fma(ar, xr[u].x, fma(-ai, xr[u].y, fma(br, xb[u].x, fma(-bi, xb[u].y, fr[r][u]))));
                       fi[r][u] = fma(ar, xr[u].y, fma(ai, xr[u].x, fma(br, xb[u].y, fma(bi, xb[u].x, fi[r][u]))));
                     }
                   }
                 }
               }
-            } else if constexpr (TC == 0) {
+            } else {
             for (int k = 0; k < M; ++k) {
-              T2 xr[4], xb[4];
+              T2 xr[TU], xb[TU];
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
+              for (int u = 0; u < TU; ++u) {
                 xr[u] = XT[k * Mp + m0 + u];
                 xb[u] = XT[MM + k * Mp + m0 + u];
               }
@@ -1577,7 +1594,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                 const T2 y0 = yrp[r][k], y1 = ybp[r][k];
                 const T ar = sr[r] * y0.x, ai = sr[r] * y0.y, br = sb[r] * y1.x, bi = sb[r] * y1.y;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < TU; ++u) {
                   fr[r][u] = fma(ar, xr[u].x, fma(-ai, xr[u].y, fma(br, xb[u].x, fma(-bi, xb[u].y, fr[r][u]))));
                   fi[r][u] = fma(ar, xr[u].y, fma(ai, xr[u].x, fma(br, xb[u].y, fma(bi, xb[u].x, fi[r][u]))));
                 }
@@ -1589,7 +1606,7 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
             for (int r = 0; r < TR; ++r) {
               const int n = nrow[r];
               if (n < 0) continue;
-              T2 zo[4];
+              T2 zo[TU];
               if constexpr (sizeof(T2) == 8) {
                 // FP32 state: columns in pairs, 16-byte loads and stores (Z_n rows
                 // are 16-byte aligned when M and the trajectory offset are even;
@@ -1639,14 +1656,14 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                     }
                   }
                 }
-                store4<ZSM>(own(nxt, l0 + r) + m0, zo);
+                storeu<ZSM>(own(nxt, l0 + r) + m0, zo);
                 if constexpr (GRAM_DW == 2)   // column maxima of the next stage input
 #pragma unroll
-                  for (int u = 0; u < 4; ++u) cmx[u] = fmaxf(cmx[u], fmaxf(fabsf(zo[u].x), fabsf(zo[u].y)));
+                  for (int u = 0; u < TU; ++u) cmx[u] = fmaxf(cmx[u], fmaxf(fabsf(zo[u].x), fabsf(zo[u].y)));
                 continue;
               }
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
+              for (int u = 0; u < TU; ++u) {
                 const int m = m0 + u;
                 if (m >= M) {
                   zo[u] = cm<T2>(0, 0);
@@ -1671,12 +1688,33 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
                   zo[u] = z1;
                 }
               }
-              store4<ZSM>(own(nxt, l0 + r) + m0, zo);
+              storeu<ZSM>(own(nxt, l0 + r) + m0, zo);
             }
             if constexpr (GRAM_DW == 2)
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
+              for (int u = 0; u < TU; ++u)
                 if (m0 + u < 20) atomicMax(gs_cmax + (gs_par ^ 1) * 20 + m0 + u, __float_as_uint(cmx[u]));
+          }
+          };
+          using std::integral_constant;
+          if constexpr (sizeof(T) == 8) {
+            // FP64: 2 rows x 4 columns share the neighbours' weights; a batch with less
+            // than a tile per thread takes one element per thread (FP64 warp
+            // instructions take 64 cycles whatever the number of lanes: N = 40, M = 4 in
+            // one warp 42k cycles, over five warps 10.7k)
+            if ((P.R + 1) / 2 * mq < NT)
+              tiles(integral_constant<int, 1>(), integral_constant<int, 1>());
+            else
+              tiles(integral_constant<int, 2>(), integral_constant<int, 4>());
+          } else if constexpr (ZSM == 1) {
+            // FP32 in shared memory: 5 rows share every XT load; less than a tile per
+            // thread: 2 rows (200 rows, M = 20: 50k -> 33k cycles)
+            if ((P.R + 4) / 5 * mq < NT)
+              tiles(integral_constant<int, 2>(), integral_constant<int, 4>());
+            else
+              tiles(integral_constant<int, 5>(), integral_constant<int, 4>());
+          } else {
+            tiles(integral_constant<int, 5>(), integral_constant<int, 4>());
           }
           }
           cur = nxt;

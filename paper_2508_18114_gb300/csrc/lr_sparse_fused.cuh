@@ -20,7 +20,7 @@
 // the team's partials in rank order from distributed shared memory and runs
 // the M x M phase itself), B2 after the RK4 update (the new Z_s is visible).
 // The phases:
-//   C  channel factors Omega(t)^a e^{i q w_d t} of the stage time in FP32
+//   C  channel factors Omega(t)^a e^{i q w_d t} of eight steps' stage times in FP32
 //      (the stage time and the phase reduced to one cycle in FP64);
 //   Y  Y_k = L_k(t) Z_s by CSR gathers; at the first stage of every step also
 //      r(t) Z_s, the readout signal beta = tr(Z_s^dag r Z_s) and, at recording
@@ -48,7 +48,7 @@ constexpr int NT = 512;       // 16 warps at <= 128 registers
 constexpr int NWARP = NT / 32;
 constexpr int NCH = 10;   // time channels
 constexpr int TP = 4;     // phase-P tile edge
-constexpr int TR = 4;     // phase-F rows per thread tile
+constexpr int CHI_STEPS = 8;   // RK4 steps whose channel factors are formed at once
 constexpr int PB = 4;     // phase-P row blocks (at most)
 // bound of the wait for a head piece (~10 s at 2 GHz); the wait normally ends
 // at once, since the previous CTA runs that head first
@@ -282,11 +282,14 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
   __shared__ uint32_t gcmax[2][20];
   __shared__ MmShared<DwArith> mm;   // columns and pivots of the sweeps
   __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
-  __shared__ float2 chi[NCH];
+  __shared__ float2 chi_tab[CHI_STEPS * 3 * NCH];   // channel factors at t, t + dt/2 and t + dt
   __shared__ double red[NWARP * 4];
   __shared__ int task_ctr[2];   // phase-P task counters of alternate row blocks
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = a.N, M = a.M, Mp = a.Mp, K = a.K, MM = Mp * Mp;
+  // rows of a phase-F thread tile: 4 share every XT load; a team's CTA has few
+  // tiles, and 2 keep its threads busy (125 rows, M = 20: 51k -> 30k cycles)
+  constexpr int TR = TEAM ? 2 : 4;
   const int Mq = (M + 3) / 4 * 4;
   const int ldg = Mp + 1;
   for (int i = tid; i < LR_MAX_RANK; i += NT)
@@ -639,26 +642,34 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
       a.trace[(size_t)tj * a.n_rec + rec] = tr;
     };
     const long s_end = a.step0 + s_b;
-    for (long step = a.step0 + s_a;; ++step) {
+    int chi_step = 0;   // step within the table of channel factors
+    for (long step = a.step0 + s_a;; ++step, ++chi_step) {
       const bool last = step == s_end;
       if (last && head) break;
       for (int stage = 0; stage < 4; ++stage) {
         const bool record = stage == 0 && (step % pe) == 0;
         const float2* zc = zs0 + (size_t)cur * zsb;
-        // ================= C: channel factors of the stage time
-        if (tid < NCH) {
-          const double ts = (double)step * dt + (stage == 0 ? 0.0 : (stage == 3 ? dt : 0.5 * dt));
-          const int ach = tid / 5, q = tid % 5 - 2;
-          const float om = ach ? envelope_f(pulse, a.tau, ts) : 1.0f;
-          // e^{i q w_d t}: the phase in cycles, reduced to [-1/2, 1/2] in FP64, then
-          // sine and cosine of the reduced phase in FP32 (FP64 transcendentals hold
-          // the FP64 pipe for tens of cycles per warp instruction on this GPU)
-          const double cyc = (double)q * a.wd * ts * INV_2PI;
-          const float x = (float)(cyc - rint(cyc));
-          float sn, cs;
-          sincospif(2.0f * x, &sn, &cs);
-          chi[tid] = make_float2(om * cs, om * sn);
+        // ================= C: channel factors, of the next CHI_STEPS steps at once
+        if (stage == 0 && chi_step == CHI_STEPS) chi_step = 0;
+        if (stage == 0 && chi_step == 0) {
+          // one thread per (step, stage time, channel): a few thousand cycles of
+          // latency, whatever the number of threads
+          for (int e = tid; e < CHI_STEPS * 3 * NCH; e += NT) {
+            const int k = e / NCH % 3, ch = e % NCH;
+            const double ts = (double)(step + e / (3 * NCH)) * dt + (k == 0 ? 0.0 : (k == 2 ? dt : 0.5 * dt));
+            const int ach = ch / 5, q = ch % 5 - 2;
+            const float om = ach ? envelope_f(pulse, a.tau, ts) : 1.0f;
+            // e^{i q w_d t}: the phase in cycles, reduced to [-1/2, 1/2] in FP64, then
+            // sine and cosine of the reduced phase in FP32 (FP64 transcendentals hold
+            // the FP64 pipe for tens of cycles per warp instruction on this GPU)
+            const double cyc = (double)q * a.wd * ts * INV_2PI;
+            const float x = (float)(cyc - rint(cyc));
+            float sn, cs;
+            sincospif(2.0f * x, &sn, &cs);
+            chi_tab[e] = make_float2(om * cs, om * sn);
+          }
         }
+        const float2* chi = chi_tab + (3 * chi_step + (stage == 0 ? 0 : (stage == 3 ? 2 : 1))) * NCH;
         if (tid == 0) task_ctr[0] = task_ctr[1] = 0;
         __syncthreads();
         // ================= Y: operator images, readout signal
