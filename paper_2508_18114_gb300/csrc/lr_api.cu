@@ -586,7 +586,7 @@ lr_status lr_backward_workspace_size(const lr_ctx* c, int ckpt_every, size_t* by
   if (c->step < 1) return LR_ERR_STATE;
   size_t part = 0;
   for (const TrajDev& d : c->traj) part += (size_t)d.nblk * lr::plain_pstride(d.M);
-  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, c->nt_max, part, c->step, ckpt_every,
+  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, part, c->step, ckpt_every,
                                          c->opt.precision != LR_PREC_FP64);
   *bytes = L.total;
   return LR_OK;
@@ -608,15 +608,15 @@ lr_status lr_backward(lr_ctx* c, void* dev_ws, size_t ws_bytes, const double* d_
     if (!std::isfinite(d_eps_a[k])) return fail(c, LR_ERR_ARG, "non-finite cotangent");
   size_t part = 0;
   for (const TrajDev& d : c->traj) part += (size_t)d.nblk * lr::plain_pstride(d.M);
-  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, c->nt_max, part, c->step, ckpt_every,
+  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, part, c->step, ckpt_every,
                                          c->opt.precision != LR_PREC_FP64);
   if (!dev_ws || ws_bytes < L.total) return fail(c, LR_ERR_WORKSPACE, "backward workspace missing or too small");
   if (reinterpret_cast<uintptr_t>(dev_ws) % 256 != 0) return fail(c, LR_ERR_WORKSPACE, "backward workspace misaligned");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DevPtrs p = dev_ptrs(c);
   RunParams rp = run_params(c);
-  cudaError_t e = lr::backward_run(p, rp, static_cast<char*>(dev_ws), L, c->tot_elems, c->max_nblk, c->max_N, c->step,
-                                   c->ws + c->o_z0, c->opt.precision != LR_PREC_FP64, d_eps_a, d_theta, s);
+  cudaError_t e = lr::backward_run(p, rp, static_cast<char*>(dev_ws), L, c->tot_elems, c->max_nblk, c->max_N, c->max_M,
+                                   c->step, c->ws + c->o_z0, c->opt.precision != LR_PREC_FP64, d_eps_a, d_theta, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "backward");
   return check_device_error(c);
 }

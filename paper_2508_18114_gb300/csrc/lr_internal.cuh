@@ -147,6 +147,16 @@ __host__ __device__ inline size_t plain_pstride(int M) { return (size_t)6 * M * 
 
 // ------------------------------------------------------------------ stencil
 
+// sqrt(k) for k < SQ_N, a kernel parameter (constant bank). An FP64 sqrt on the
+// device takes ~10 instructions of a pipe that does 2 FMA/clk/SM; the ~16 of a
+// row's stencil cost as much as its projections at M = 20.
+constexpr int SQ_N = 128;
+struct SqTab {
+  double v[SQ_N];
+};
+const SqTab& sq_table();   // lr_plain.cu
+__device__ __forceinline__ double sq_of(const SqTab& t, int k) { return k < SQ_N ? t.v[k] : sqrt((double)k); }
+
 // Mode indices of a row.
 struct RowIdx {
   int it, ir, iff;
@@ -257,21 +267,29 @@ cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk,
 // single kernels of the plain engine (used by the adjoint's recomputation)
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s);
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s);
+// (coef: drive coefficients c(t), coef[cand * cstride], or null: plain_solve's; zout: the next
+// stage input, at stage 3 where Z_{n+1} goes, null for in place)
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const double2* zin, double2* zout, int stage,
-                      double t, cudaStream_t s);
+                      const double* coef, int cstride, cudaStream_t s);
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const float2* zin, float2* zout, int stage,
-                      double t, cudaStream_t s);
+                      const double* coef, int cstride, cudaStream_t s);
+// after plain_reduce; t: stage time of the drive coefficient (negative: not wanted); Gi
+// [n_traj][LR_MAX_RANK^2] or null
+void plain_solve_launch(const DevPtrs& p, const RunParams& rp, double2* Gi, long step, int stage, int record, int do_solve,
+                        double t, cudaStream_t s);
+// adds each trajectory's first n(M) = a M^2 + b doubles of its row blocks in block order into the first
+void plain_reduce_launch(const TrajDev* traj, int n_traj, int max_M, double* part, int a, int b, cudaStream_t s);
 
 // lr_adjoint.cu
 struct BwdLayout {
-  size_t ck, seg, cur, za, zb, acc, U, Ub, lam, lamn, X, part, Xs, Gi, EP, Xs32, EP32, bpart, beta, pops, nphot,
-      trace, gcoef, deps, thbar, total;
+  size_t ck, seg, cur, acc, U, Ub, Fb, lam, lamn, part, Xs, Gi, EP, Xs32, bpart, beta, coef, gcoef, deps, thbar, total;
   long n_seg, K;
-  int fp32;   // 1: FP32-bulk adjoint (complex64 states and cotangents)
+  long slots;   // steps whose stage inputs and M x M factors are kept: K, or 1 (recomputed step by step)
+  int fp32;     // 1: FP32-bulk adjoint (complex64 states and cotangents)
 };
-BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, int nt_max, size_t part_doubles, long S, int K, int fp32);
+BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles, long S, int K, int fp32);
 cudaError_t backward_run(const DevPtrs& main, const RunParams& rp, char* ws, const BwdLayout& L, long long tot,
-                         int max_nblk, int max_N, long S, const void* z0, int z0_fp32, const double* deps_host,
+                         int max_nblk, int max_N, int max_M, long S, const void* z0, int z0_fp32, const double* deps_host,
                          double* dtheta_host, cudaStream_t s);
 
 }  // namespace lr

@@ -1,12 +1,12 @@
 // PLAIN engine: straightforward FP64 kernels with the state in HBM.
 //
-// One RK4 stage of Eq. S5 is three launches:
+// One RK4 stage of Eq. S5 is four launches:
 //   plain_gram  - per row block, partial sums of G = Z^dag Z (upper triangle),
 //                 T_r = Z^dag r Z and T_b = Z^dag b Z, plus level populations
 //                 and readout photons at recording steps;
-//   plain_solve - one block per trajectory: reduce the partials in a fixed
-//                 order, record beta = tr(T_r) at stage 1 of each step, Cholesky
-//                 G = L L^dag, solve X_r = G^-1 T_r, X_b = G^-1 T_b;
+//   plain_reduce - the partials added in block order, one thread per entry;
+//   plain_solve - a few blocks per trajectory: record beta = tr(T_r) at stage 1 of
+//                 each step, G^-1 by symmetric sweeps, X_r = G^-1 T_r, X_b = G^-1 T_b;
 //   plain_rhs   - per element: F = -i H_eff Z + 1/2 kappa (rZ) X_r^dag
 //                 + 1/2 gamma (bZ) X_b^dag, then the RK4 stage update.
 // With Y_k = L_k Z the projection term of Eq. S5 is 1/2 sum_k Y_k (Z^+ Y_k)^dag
@@ -16,13 +16,25 @@
 // The state type is a template parameter: complex128 (the reference path), or
 // complex64 for the FP32-bulk recomputation inside the adjoint. With complex64
 // the Gram matrix is summed from the exact products of the FP32 entries in
-// double-word FP32 (FP64-class), the Cholesky factor and the solves are FP64,
+// double-word FP32 (FP64-class), G^-1 and X_k are FP64,
 // and the operator apply, T_k, the projection term and the RK4 update run in
 // FP32 (the diagonal energies and the step sizes split into hi + lo floats so
 // that FP32 does not round the mode frequencies or dt).
-#include "lr_internal.cuh"
+#include <algorithm>
+#include <cmath>
+
+#include "lr_mm.cuh"
 
 namespace lr {
+
+const SqTab& sq_table() {
+  static const SqTab t = [] {
+    SqTab x;
+    for (int k = 0; k < SQ_N; ++k) x.v[k] = std::sqrt((double)k);
+    return x;
+  }();
+  return t;
+}
 
 constexpr int PR = 16;        // rows per Gram block
 constexpr int PT = 256;       // threads per block
@@ -34,7 +46,8 @@ size_t plain_partial_doubles(int M) { return pstride(M); }
 
 template <typename T2>
 __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ traj, const T2* __restrict__ Zin,
-                                                 double* __restrict__ part, int with_obs) {
+                                                 double* __restrict__ part, int with_obs,
+                                                 const __grid_constant__ SqTab sq) {
   using T = typename real_of<T2>::type;
   const TrajDev d = traj[blockIdx.y];
   const int b = blockIdx.x;
@@ -56,12 +69,12 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
       const RowIdx ri = row_index(d, n);
       const int iro = readout_index(d, ri);
       if (iro + 1 < readout_dim(d)) {
-        const T c = (T)sqrt(iro + 1.0);
+        const T c = (T)sq_of(sq, iro + 1);
         const T2 v = Z[(size_t)(n + 1) * ld + m];
         zr = mkc<T2>(c * v.x, c * v.y);
       }
       if (ri.it + 1 < d.Nt) {
-        const T c = (T)sqrt(ri.it + 1.0);
+        const T c = (T)sq_of(sq, ri.it + 1);
         const T2 v = Z[(size_t)(n + st) * ld + m];
         zb = mkc<T2>(c * v.x, c * v.y);
       }
@@ -76,10 +89,24 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
   }
   __syncthreads();
   double* out = part + d.p_off + (size_t)b * pstride(M);
-  const int MM = M * M;
-  for (int e = threadIdx.x; e < 3 * MM; e += blockDim.x) {
-    const int mat = e / MM, ij = e - mat * MM, i = ij / M, j = ij - (ij / M) * M;
-    if (mat == 0 && i > j) continue;
+  const int MM = M * M, ne = M * (M + 1) / 2;
+  // entries in a row without the lower triangle: an FP64 instruction takes a warp's
+  // time however many of its lanes are in use
+  for (int e0 = threadIdx.x; e0 < ne + 2 * MM; e0 += blockDim.x) {
+    int mat = 0, i, j;
+    if (e0 < ne) {
+      j = (int)((sqrtf(8.f * e0 + 1.f) - 1.f) * 0.5f);
+      while (j * (j + 1) / 2 > e0) --j;
+      while ((j + 1) * (j + 2) / 2 <= e0) ++j;
+      i = e0 - j * (j + 1) / 2;   // i <= j
+    } else {
+      const int e1 = e0 - ne;
+      mat = 1 + e1 / MM;
+      const int ij = e1 - (mat - 1) * MM;
+      i = ij / M;
+      j = ij - i * M;
+    }
+    const int e = mat * MM + i * M + j;
     if (sizeof(T) == 4 && mat == 0) {
       // FP32 state: exact FP32 products (FMA TwoProduct) in double-word sums
       // (Knuth TwoSum), ~2^-48 relative: the FP64-class Gram on the FP32 pipes
@@ -145,311 +172,338 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
   }
 }
 
-__global__ void __launch_bounds__(PT) plain_solve(DevPtrs p, RunParams rp, long step, int stage, int record,
-                                                  int do_solve) {
-  const int tj = blockIdx.x;
+// Entry o < a M^2 + b of every trajectory: the row blocks' partial sums in block
+// order, into block 0's. One thread per entry over the whole chip: in the one block
+// per trajectory that solves, the 125 partials of N = 2000, M = 20 (3e5 FP64 adds)
+// took ~75 us of one SM.
+__global__ void __launch_bounds__(PT) plain_reduce(const TrajDev* __restrict__ traj, double* __restrict__ part, int a,
+                                                   int b) {
+  const TrajDev d = traj[blockIdx.y];
+  const int o = blockIdx.x * PT + threadIdx.x;
+  if (o >= a * d.M * d.M + b) return;
+  double* P = part + d.p_off + o;
+  const size_t ps = pstride(d.M);
+  double s = 0.0;
+  int k = 0;
+  for (; k + 8 <= d.nblk; k += 8) {   // eight loads in flight
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = P[(k + u) * ps];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  for (; k < d.nblk; ++k) s += P[k * ps];
+  P[0] = s;
+}
+
+void plain_reduce_launch(const TrajDev* traj, int n_traj, int max_M, double* part, int a, int b, cudaStream_t s) {
+  plain_reduce<<<dim3((a * max_M * max_M + b + PT - 1) / PT, n_traj), PT, 0, s>>>(traj, part, a, b);
+}
+
+// The FP64 entry arithmetic of the sweeps; a pivot counts as zero where it is lost in
+// the rounding of M updates of its diagonal entry (LR_MAX_RANK 2^-51 of it), so that a
+// rank-deficient state is told whatever the sign of that rounding.
+struct WidePivot : F64Arith {
+  static __device__ __forceinline__ double recip(double2 p) {
+    return p.x > 1e-30 && p.x < 1e30 ? F64Arith::recip(p) : 1.0 / p.x;
+  }
+  static __device__ __forceinline__ bool breakdown(double2 p, double d0) {
+    return !(p.x > LR_MAX_RANK * 0x1p-51 * d0) || !isfinite(p.x);
+  }
+};
+__device__ __forceinline__ double2 mac(double2 a, double2 b, double2 s) {   // s + a b
+  return mk(fma(a.x, b.x, fma(-a.y, b.y, s.x)), fma(a.x, b.y, fma(a.y, b.x, s.y)));
+}
+
+// Two doubles of the reduced sums carry the drive coefficient from plain_solve to
+// plain_rhs: the one after the populations, and the imaginary part of G_00.
+__device__ __forceinline__ double* drive_slot(double* P, int M, int c) { return P + (c ? 1 : 6 * M * M + LR_MAX_NT + 1); }
+
+constexpr int ST = 544;   // threads of plain_solve: one entry of the 32 x 32 triangle each
+
+// From the sums in the trajectory's first row block: G^-1 by symmetric sweeps and X_k
+// = G^-1 T_k (G^-1 to Gi unless null); at stage 0 the readout signal and the records;
+// the drive coefficient of the stage time t. Every block of a trajectory forms G^-1
+// (latency, ~1000 cycles a sweep in FP64) and its share of X_k, whose 8 M^3 FMAs
+// take one SM 31k cycles at M = 20. It replaces a Cholesky factorisation and two
+// triangular sweeps over 2 M columns in one block, ~70 barriers of FP64 latency.
+__global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, double2* __restrict__ Gi, long step, int stage,
+                                                  int record, int do_solve, double t) {
+  const int tj = blockIdx.y, g = blockIdx.x;
   const TrajDev d = p.traj[tj];
-  const int M = d.M, MM = M * M, tid = threadIdx.x;
-  __shared__ double2 L[LR_MAX_RANK][LR_MAX_RANK + 1];
-  __shared__ double2 B[LR_MAX_RANK][2 * LR_MAX_RANK + 1];
-  __shared__ int bad;
-  const double* P = p.part + d.p_off;
-  const size_t ps = pstride(M);
-  if (tid == 0) bad = 0;
-  for (int e = tid; e < 3 * MM; e += blockDim.x) {
-    const int mat = e / MM, ij = e - mat * MM, i = ij / M, j = ij - (ij / M) * M;
-    if (mat == 0 && i > j) continue;
-    double re = 0.0, im = 0.0;
-    for (int b = 0; b < d.nblk; ++b) {
-      re += P[b * ps + 2 * e];
-      im += P[b * ps + 2 * e + 1];
+  const int M = d.M, MM = M * M, tid = threadIdx.x, ldg = M | 1;
+  __shared__ double2 Gs[LR_MAX_RANK * (LR_MAX_RANK + 1)];
+  __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
+  __shared__ MmShared<WidePivot> mm;
+  double* Pd = p.part + d.p_off;
+  const double2* P = reinterpret_cast<const double2*>(Pd);   // p_off and the block size are even
+  if (g == 0 && stage == 0) {
+    if (tid == ST - 1) {
+      double2 b = mk(0.0, 0.0);
+      for (int i = 0; i < M; ++i) b = mk(b.x + P[MM + i * M + i].x, b.y + P[MM + i * M + i].y);
+      p.beta[(size_t)tj * (rp.max_steps + 1) + step] = b;
+      if (!isfinite(b.x) || !isfinite(b.y)) set_error(p.err, DEV_NONFINITE);
     }
-    if (mat == 0) {
-      if (i == j) {
-        L[i][i] = mk(re, 0.0);
-      } else {
-        L[i][j] = mk(re, im);
-        L[j][i] = mk(re, -im);
+    if (record) {
+      const long rec = step / rp.pop_every;
+      if (tid < LR_MAX_NT + 1) {
+        const double v = Pd[6 * MM + tid];
+        if (tid < rp.nt_max) p.pops[((size_t)tj * rp.n_rec + rec) * rp.nt_max + tid] = tid < d.Nt ? v : 0.0;
+        if (tid == LR_MAX_NT) p.nphot[(size_t)tj * rp.n_rec + rec] = v;
       }
-    } else {
-      B[i][(mat - 1) * M + j] = mk(re, im);
+      if (tid == 32) {
+        double tr = 0.0;
+        for (int i = 0; i < M; ++i) tr += P[i * M + i].x;
+        p.trace[(size_t)tj * rp.n_rec + rec] = tr;
+      }
+      if (p.gsnap) {
+        double2* gs = p.gsnap + ((size_t)tj * rp.n_rec + rec) * rp.snap_m * rp.snap_m;
+        for (int e = tid; e < MM; e += ST) {
+          const int i = e / M, j = e - i * M;
+          const double2 v = P[min(i, j) * M + max(i, j)];
+          gs[i * rp.snap_m + j] = mk(v.x, i == j ? 0.0 : (i < j ? v.y : -v.y));
+        }
+      }
     }
+  }
+  if (!do_solve) return;
+  if (g == (gridDim.x > 1 ? 1 : 0) && tid == ST - 33 && t >= 0.0) {
+    const PulseDev pulse = p.pulse[d.cand];
+    if (rp.frame) {
+      const double2 w = pulse_rwa_drive(pulse, rp.tau, t);
+      *drive_slot(Pd, M, 0) = w.x;
+      *drive_slot(Pd, M, 1) = w.y;
+    } else {
+      *drive_slot(Pd, M, 0) = pulse_coefficient(pulse, rp.tau, t);
+    }
+  }
+  if (tid == 0) mm.bad = 0;
+  for (int i = tid; i < M; i += ST)
+    for (int j = 0; j <= i; ++j) tri[i * (i + 1) / 2 + j] = make_short2((short)i, (short)j);
+  __syncthreads();
+  if (tid / 32 < mm_warps(M, ST / 32)) {
+    double2 e[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};   // the sums hold the upper triangle
+    if (tid < M * (M + 1) / 2) {
+      const int i = tri[tid].x, j = tri[tid].y;
+      const double2 v = P[j * M + i];
+      e[0] = mk(v.x, i == j ? 0.0 : -v.y);
+    }
+    mm_invert<WidePivot, ST>(e, Gs, ldg, mm, tri, M, tid);
   }
   __syncthreads();
-  if (stage == 0) {
-    if (tid == 0) {
-      double br = 0.0, bi = 0.0;
-      for (int i = 0; i < M; ++i) {
-        br += B[i][i].x;
-        bi += B[i][i].y;
-      }
-      p.beta[(size_t)tj * (rp.max_steps + 1) + step] = mk(br, bi);
-      if (!isfinite(br) || !isfinite(bi)) set_error(p.err, DEV_NONFINITE);
-    }
-    if (record && tid < LR_MAX_NT + 1) {
-      double acc = 0.0;
-      for (int b = 0; b < d.nblk; ++b) acc += P[b * ps + 6 * MM + tid];
-      const long rec = step / rp.pop_every;
-      if (tid < rp.nt_max) p.pops[((size_t)tj * rp.n_rec + rec) * rp.nt_max + tid] = tid < d.Nt ? acc : 0.0;
-      if (tid == LR_MAX_NT) p.nphot[(size_t)tj * rp.n_rec + rec] = acc;
-    }
-    if (record && tid == 32) {
-      double tr = 0.0;
-      for (int i = 0; i < M; ++i) tr += L[i][i].x;
-      p.trace[(size_t)tj * rp.n_rec + step / rp.pop_every] = tr;
-    }
-    if (record && p.gsnap) {
-      double2* gs = p.gsnap + ((size_t)tj * rp.n_rec + step / rp.pop_every) * rp.snap_m * rp.snap_m;
-      for (int e = tid; e < MM; e += blockDim.x) gs[(e / M) * rp.snap_m + e % M] = L[e / M][e % M];
-    }
-  }
-  __syncthreads();   // the trace above reads the diagonal before it is factorised
-  if (!do_solve) return;
-  // Cholesky G = L L^dag (right-looking, lower triangle in place).
-  for (int k = 0; k < M; ++k) {
-    if (tid == 0) {
-      double piv = L[k][k].x;
-      if (!(piv > 0.0) || !isfinite(piv)) {
-        bad = 1;
-        piv = 1.0;
-      }
-      L[k][k] = mk(sqrt(piv), 0.0);
-    }
-    __syncthreads();
-    const double inv = 1.0 / L[k][k].x;
-    for (int i = k + 1 + tid; i < M; i += blockDim.x) L[i][k] = mk(L[i][k].x * inv, L[i][k].y * inv);
-    __syncthreads();
-    const int w = M - k - 1;
-    for (int e = tid; e < w * w; e += blockDim.x) {
-      const int i = k + 1 + e / w, j = k + 1 + e % w;
-      if (j > i) continue;
-      const double2 a = L[i][k], c = L[j][k];   // L[i][j] -= a * conj(c)
-      L[i][j] = mk(L[i][j].x - (a.x * c.x + a.y * c.y), L[i][j].y - (a.y * c.x - a.x * c.y));
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && bad) set_error(p.err, DEV_NOT_PD);
-  const int nc = 2 * M;
-  // forward: L W = B
-  for (int k = 0; k < M; ++k) {
-    const double inv = 1.0 / L[k][k].x;
-    for (int c = tid; c < nc; c += blockDim.x) B[k][c] = mk(B[k][c].x * inv, B[k][c].y * inv);
-    __syncthreads();
-    for (int e = tid; e < (M - k - 1) * nc; e += blockDim.x) {
-      const int i = k + 1 + e / nc, c = e % nc;
-      const double2 a = L[i][k], w = B[k][c];
-      B[i][c] = mk(B[i][c].x - (a.x * w.x - a.y * w.y), B[i][c].y - (a.x * w.y + a.y * w.x));
-    }
-    __syncthreads();
-  }
-  // backward: L^dag X = W, (L^dag)[i][k] = conj(L[k][i])
-  for (int k = M - 1; k >= 0; --k) {
-    const double inv = 1.0 / L[k][k].x;
-    for (int c = tid; c < nc; c += blockDim.x) B[k][c] = mk(B[k][c].x * inv, B[k][c].y * inv);
-    __syncthreads();
-    for (int e = tid; e < k * nc; e += blockDim.x) {
-      const int i = e / nc, c = e % nc;
-      const double2 a = L[k][i], w = B[k][c];    // conj(a) * w
-      B[i][c] = mk(B[i][c].x - (a.x * w.x + a.y * w.y), B[i][c].y - (a.x * w.y - a.y * w.x));
-    }
-    __syncthreads();
+  if (g == 0) {
+    if (tid == 0 && mm.bad) set_error(p.err, DEV_NOT_PD);
+    if (Gi)
+      for (int e = tid; e < MM; e += ST) Gi[(size_t)tj * LR_MAX_RANK * LR_MAX_RANK + e] = Gs[(e / M) * ldg + e % M];
   }
   double2* X = p.X + (size_t)tj * 2 * LR_MAX_RANK * LR_MAX_RANK;
-  for (int e = tid; e < 2 * MM; e += blockDim.x) {
-    const int k = e / MM, ij = e - k * MM, i = ij / M, j = ij - (ij / M) * M;
-    X[k * LR_MAX_RANK * LR_MAX_RANK + ij] = B[i][k * M + j];
+  const int per = (2 * MM + gridDim.x - 1) / gridDim.x;
+  for (int e = g * per + tid; e < min(2 * MM, (g + 1) * per); e += ST) {
+    const int k = e / MM, ij = e - k * MM, i = ij / M, j = ij - i * M;
+    const double2* tk = P + (1 + k) * MM + j;
+    double2 s = mk(0.0, 0.0);
+    for (int l = 0; l < M; ++l) s = mac(Gs[i * ldg + l], tk[l * M], s);
+    X[k * LR_MAX_RANK * LR_MAX_RANK + ij] = s;
   }
 }
 
+void plain_solve_launch(const DevPtrs& p, const RunParams& rp, double2* Gi, long step, int stage, int record, int do_solve,
+                        double t, cudaStream_t s) {
+  // a trajectory's share of two blocks per SM, at most eight
+  const int blocks = do_solve ? std::max(1, std::min(8, 304 / rp.n_traj)) : 1;
+  plain_solve<<<dim3(blocks, rp.n_traj), ST, 0, s>>>(p, rp, Gi, step, stage, record, do_solve, t);
+}
+
+// Thread: one row, the columns m and m + 1. Bound by the FP64 pipe for the
+// complex128 state: 8 FMAs per column and l of the two projections, ~45 others.
+constexpr int RT = 128;   // threads per block
+
 template <typename T2>
-__global__ void __launch_bounds__(PT) plain_rhs(DevPtrs p, RunParams rp, const T2* __restrict__ Zin,
-                                                T2* __restrict__ Zout, int stage, double t) {
+__global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T2* __restrict__ Zin,
+                                                T2* __restrict__ Zout, int stage,
+                                                const double* __restrict__ ctab, int cstride,
+                                                const __grid_constant__ SqTab sq) {
   using T = typename real_of<T2>::type;
   constexpr bool f32 = sizeof(T) == 4;
   const int tj = blockIdx.y;
   const TrajDev d = p.traj[tj];
+  const int M = d.M, MM = M * M, ld = d.ld, np = (M + 1) / 2;
+  const long total = (long)d.N * np;
+  if ((long)blockIdx.x * RT >= total) return;
   __shared__ T2 sX[2][LR_MAX_RANK * LR_MAX_RANK];
   __shared__ double coef, coef_i, wfr;
-  const int M = d.M, MM = M * M, ld = d.ld;
   const double2* X = p.X + (size_t)tj * 2 * LR_MAX_RANK * LR_MAX_RANK;
   // transposed in shared memory, sX[k][l * M + m] = X_k[m][l]: the threads of a
   // warp (consecutive m) then read consecutive words (no bank conflicts)
-  for (int e = threadIdx.x; e < 2 * MM; e += blockDim.x) {
+  for (int e = threadIdx.x; e < 2 * MM; e += RT) {
     const int k = e / MM, ij = e - k * MM, i = ij / M, j = ij - i * M;
     const double2 x = X[k * LR_MAX_RANK * LR_MAX_RANK + ij];
     sX[k][j * M + i] = mkc<T2>((T)x.x, (T)x.y);
   }
   if (threadIdx.x == 0) {
-    const PulseDev P = p.pulse[d.cand];
-    if (rp.frame) {
-      const double2 w = pulse_rwa_drive(P, rp.tau, t);
-      coef = w.x;
-      coef_i = w.y;
-      wfr = pulse_drive_frequency(P);
-    } else {
-      coef = pulse_coefficient(P, rp.tau, t);
-      coef_i = 0.0;
-      wfr = 0.0;
-    }
+    double* P = p.part + d.p_off;
+    coef = ctab ? ctab[(size_t)d.cand * cstride] : *drive_slot(P, M, 0);
+    coef_i = rp.frame ? *drive_slot(P, M, 1) : 0.0;
+    wfr = rp.frame ? pulse_drive_frequency(p.pulse[d.cand]) : 0.0;
   }
   __syncthreads();
+  const long idx = (long)blockIdx.x * RT + threadIdx.x;
+  if (idx >= total) return;
   const T2* Z = Zin + d.z_off;
   T2* Zn = reinterpret_cast<T2*>(p.Zn) + d.z_off;
   T2* acc = reinterpret_cast<T2*>(p.acc) + d.z_off;
-  T2* Zo = Zout ? Zout + d.z_off : nullptr;
+  T2* Zo = Zout ? Zout + d.z_off : Zn;
   const int st = d.Nr * d.Nf, sr = d.Nf;
   const T c = (T)coef, ci = (T)coef_i;
   const double dt = rp.dt;
-  // FP32 state: step sizes as hi + lo floats
+  // step sizes as hi + lo (FP32 state; lo = 0 in FP64)
   const double hsd = stage == 2 ? dt : 0.5 * dt, h6d = dt / 6.0;
   const T hs_hi = (T)hsd, hs_lo = (T)(hsd - (double)hs_hi), h6_hi = (T)h6d, h6_lo = (T)(h6d - (double)h6_hi);
   const bool rwa = rp.frame != 0;
-  const long total = (long)d.N * M;
-  for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-    const int n = (int)(idx / M), m = (int)(idx - (long)n * M);
-    const RowIdx ri = row_index(d, n);
-    double dre, dim_;
-    heff_diag(d, ri, wfr, dre, dim_);
-    const T2 z = Z[(size_t)n * ld + m];
-    T hr, hi;
-    if constexpr (f32) {
-      // diagonal energy as hi + lo floats: FP32 does not round the mode frequencies
-      const T dh = (T)dre, dl = (T)(dre - (double)dh), di = (T)dim_;
-      hr = fma(dh, z.x, fma(dl, z.x, -di * z.y));
-      hi = fma(dh, z.y, fma(dl, z.y, di * z.x));
-    } else {
-      hr = dre * z.x - dim_ * z.y;
-      hi = dre * z.y + dim_ * z.x;
+  const int n = (int)(idx / np), m = 2 * (int)(idx - (long)n * np);
+  const bool two = m + 1 < M;
+  const int m1 = two ? m + 1 : m;
+  const RowIdx ri = row_index(d, n);
+  double dre, dim_;
+  heff_diag(d, ri, wfr, dre, dim_);
+  const T2* zrow = Z + (size_t)n * ld;
+  T hr[2], hi[2];
+  {
+    // diagonal energy as hi + lo floats: FP32 does not round the mode frequencies
+    const T dh = (T)dre, dl = (T)(dre - (double)dh), di = (T)dim_;
+    const T2 z[2] = {zrow[m], zrow[m1]};
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if constexpr (f32) {
+        hr[u] = fma(dh, z[u].x, fma(dl, z[u].x, -di * z[u].y));
+        hi[u] = fma(dh, z[u].y, fma(dl, z[u].y, di * z[u].x));
+      } else {
+        hr[u] = fma(dh, z[u].x, -di * z[u].y);
+        hi[u] = fma(dh, z[u].y, di * z[u].x);
+      }
     }
-    // g (b + b^dag)(a + a^dag)
+  }
+  auto add_row = [&](int off, T w) {
+    const T2* v = zrow + (long)off * ld;
+    const T2 v0 = v[m], v1 = v[m1];
+    hr[0] = fma(w, v0.x, hr[0]);
+    hi[0] = fma(w, v0.y, hi[0]);
+    hr[1] = fma(w, v1.x, hr[1]);
+    hi[1] = fma(w, v1.y, hi[1]);
+  };
+  // g (b + b^dag)(a + a^dag)
+#pragma unroll
+  for (int a = -1; a <= 1; a += 2) {
+    const int it2 = ri.it + a;
+    if (it2 < 0 || it2 >= d.Nt) continue;
+    const double ct = sq_of(sq, max(ri.it, it2));
+#pragma unroll
+    for (int bb = -1; bb <= 1; bb += 2) {
+      const int ir2 = ri.ir + bb;
+      if (ir2 < 0 || ir2 >= d.Nr) continue;
+      if (rwa && a == bb) continue;   // RWA keeps g (b^dag a + b a^dag) only
+      add_row(a * st + bb * sr, (T)(d.g * ct * sq_of(sq, max(ri.ir, ir2))));
+    }
+  }
+  if (d.n_modes == 3) {
+    // J (a + a^dag)(f + f^dag)
+#pragma unroll
     for (int a = -1; a <= 1; a += 2) {
-      const int it2 = ri.it + a;
-      if (it2 < 0 || it2 >= d.Nt) continue;
-      const double ct = sqrt((double)max(ri.it, it2));
+      const int ir2 = ri.ir + a;
+      if (ir2 < 0 || ir2 >= d.Nr) continue;
+      const double cr = sq_of(sq, max(ri.ir, ir2));
+#pragma unroll
       for (int bb = -1; bb <= 1; bb += 2) {
-        const int ir2 = ri.ir + bb;
-        if (ir2 < 0 || ir2 >= d.Nr) continue;
-        if (rwa && a == bb) continue;   // RWA keeps g (b^dag a + b a^dag) only
-        const T w = (T)(d.g * ct * sqrt((double)max(ri.ir, ir2)));
-        const T2 v = Z[(size_t)(n + a * st + bb * sr) * ld + m];
-        hr += w * v.x;
-        hi += w * v.y;
+        const int if2 = ri.iff + bb;
+        if (if2 < 0 || if2 >= d.Nf) continue;
+        if (rwa && a == bb) continue;   // RWA keeps J (a^dag f + a f^dag) only
+        add_row(a * sr + bb, (T)(d.J * cr * sq_of(sq, max(ri.iff, if2))));
       }
     }
-    if (d.n_modes == 3) {
-      // J (a + a^dag)(f + f^dag)
-      for (int a = -1; a <= 1; a += 2) {
-        const int ir2 = ri.ir + a;
-        if (ir2 < 0 || ir2 >= d.Nr) continue;
-        const double cr = sqrt((double)max(ri.ir, ir2));
-        for (int bb = -1; bb <= 1; bb += 2) {
-          const int if2 = ri.iff + bb;
-          if (if2 < 0 || if2 >= d.Nf) continue;
-          if (rwa && a == bb) continue;   // RWA keeps J (a^dag f + a f^dag) only
-          const T w = (T)(d.J * cr * sqrt((double)max(ri.iff, if2)));
-          const T2 v = Z[(size_t)(n + a * sr + bb) * ld + m];
-          hr += w * v.x;
-          hi += w * v.y;
-        }
-      }
+  }
+  // drive on the readout mode (stride 1): lab frame c(t) (r + r^dag); RWA
+  // w r + conj(w) r^dag with w = c + i ci (row n gets r from n+1, r^dag from n-1)
+  const int iro = readout_index(d, ri), dro = readout_dim(d);
+#pragma unroll
+  for (int a = -1; a <= 1; a += 2) {
+    const int i2 = iro + a;
+    if (i2 < 0 || i2 >= dro) continue;
+    const T s = (T)sq_of(sq, max(iro, i2));
+    add_row(a, c * s);
+    if (rwa) {
+      const T wi = (a > 0 ? ci : -ci) * s;
+      const T2* v = zrow + (long)a * ld;
+      const T2 v0 = v[m], v1 = v[m1];
+      hr[0] = fma(-wi, v0.y, hr[0]);
+      hi[0] = fma(wi, v0.x, hi[0]);
+      hr[1] = fma(-wi, v1.y, hr[1]);
+      hi[1] = fma(wi, v1.x, hi[1]);
     }
-    // drive on the readout mode (stride 1): lab frame c(t) (r + r^dag); RWA
-    // w r + conj(w) r^dag with w = c + i ci (row n gets r from n+1, r^dag from n-1)
-    const int iro = readout_index(d, ri), dro = readout_dim(d);
-    for (int a = -1; a <= 1; a += 2) {
-      const int i2 = iro + a;
-      if (i2 < 0 || i2 >= dro) continue;
-      const T s = (T)sqrt((double)max(iro, i2));
-      const T wr = c * s, wi = (a > 0 ? ci : -ci) * s;
-      const T2 v = Z[(size_t)(n + a) * ld + m];
-      hr += wr * v.x - wi * v.y;
-      hi += wr * v.y + wi * v.x;
+  }
+  // F = -i H_eff Z
+  T fr[2] = {hi[0], hi[1]}, fi[2] = {-hr[0], -hr[1]};
+  // + 1/2 kappa (rZ) X_r^dag + 1/2 gamma (bZ) X_b^dag
+  auto project = [&](const T2* y, const T2* x, T s) {
+    T pr[2] = {0, 0}, pi[2] = {0, 0};
+    for (int l = 0; l < M; ++l) {
+      const T2 v = y[l], x0 = x[l * M + m], x1 = x[l * M + m1];   // v conj(x)
+      pr[0] = fma(v.x, x0.x, fma(v.y, x0.y, pr[0]));
+      pi[0] = fma(v.y, x0.x, fma(-v.x, x0.y, pi[0]));
+      pr[1] = fma(v.x, x1.x, fma(v.y, x1.y, pr[1]));
+      pi[1] = fma(v.y, x1.x, fma(-v.x, x1.y, pi[1]));
     }
-    // F = -i H_eff Z
-    T fr = hi, fi = -hr;
-    // + 1/2 kappa (rZ) X_r^dag + 1/2 gamma (bZ) X_b^dag
-    if (iro + 1 < dro) {
-      const T s = (T)(0.5 * d.kappa * sqrt(iro + 1.0));
-      const T2* zr = Z + (size_t)(n + 1) * ld;
-      T sr_ = 0, si_ = 0;
-      for (int l = 0; l < M; ++l) {
-        const T2 y = zr[l], x = sX[0][l * M + m];   // y * conj(x)
-        sr_ += y.x * x.x + y.y * x.y;
-        si_ += y.y * x.x - y.x * x.y;
-      }
-      fr += s * sr_;
-      fi += s * si_;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      fr[u] = fma(s, pr[u], fr[u]);
+      fi[u] = fma(s, pi[u], fi[u]);
     }
-    if (ri.it + 1 < d.Nt) {
-      const T s = (T)(0.5 * d.gamma * sqrt(ri.it + 1.0));
-      const T2* zb = Z + (size_t)(n + st) * ld;
-      T sr_ = 0, si_ = 0;
-      for (int l = 0; l < M; ++l) {
-        const T2 y = zb[l], x = sX[1][l * M + m];
-        sr_ += y.x * x.x + y.y * x.y;
-        si_ += y.y * x.x - y.x * x.y;
-      }
-      fr += s * sr_;
-      fi += s * si_;
-    }
-    // RK4 (weights 1/6, 1/3, 1/3, 1/6)
-    const size_t o = (size_t)n * ld + m;
+  };
+  if (iro + 1 < dro) project(zrow + ld, sX[0], (T)(0.5 * d.kappa * sq_of(sq, iro + 1)));
+  if (ri.it + 1 < d.Nt) project(zrow + (size_t)st * ld, sX[1], (T)(0.5 * d.gamma * sq_of(sq, ri.it + 1)));
+  // RK4 (weights 1/6, 1/3, 1/3, 1/6)
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (u == 1 && !two) break;
+    const size_t o = (size_t)n * ld + m + u;
     const T2 zn = Zn[o];
-    if constexpr (f32) {
-      if (stage < 3) {
-        if (stage == 0) {
-          acc[o] = mkc<T2>(fr, fi);
-        } else {
-          const T2 a = acc[o];
-          acc[o] = mkc<T2>(fma((T)2, fr, a.x), fma((T)2, fi, a.y));
-        }
-        Zo[o] = mkc<T2>(zn.x + fma(hs_lo, fr, hs_hi * fr), zn.y + fma(hs_lo, fi, hs_hi * fi));
-      } else {
-        const T2 a = acc[o];
-        const T s_r = a.x + fr, s_i = a.y + fi;
-        Zn[o] = mkc<T2>(zn.x + fma(h6_lo, s_r, h6_hi * s_r), zn.y + fma(h6_lo, s_i, h6_hi * s_i));
-      }
+    T sx = fr[u], sy = fi[u];
+    if (stage > 0) {
+      const T2 a = acc[o];
+      const T w = stage < 3 ? (T)2 : (T)1;
+      sx = fma(w, sx, a.x);
+      sy = fma(w, sy, a.y);
+    }
+    if (stage < 3) {
+      acc[o] = mkc<T2>(sx, sy);
+      Zo[o] = f32 ? mkc<T2>(zn.x + fma(hs_lo, fr[u], hs_hi * fr[u]), zn.y + fma(hs_lo, fi[u], hs_hi * fi[u]))
+                  : mkc<T2>(fma(hs_hi, fr[u], zn.x), fma(hs_hi, fi[u], zn.y));
     } else {
-      if (stage == 0) {
-        acc[o] = mkc<T2>(fr, fi);
-        Zo[o] = mkc<T2>(zn.x + 0.5 * dt * fr, zn.y + 0.5 * dt * fi);
-      } else if (stage == 1) {
-        const T2 a = acc[o];
-        acc[o] = mkc<T2>(a.x + 2.0 * fr, a.y + 2.0 * fi);
-        Zo[o] = mkc<T2>(zn.x + 0.5 * dt * fr, zn.y + 0.5 * dt * fi);
-      } else if (stage == 2) {
-        const T2 a = acc[o];
-        acc[o] = mkc<T2>(a.x + 2.0 * fr, a.y + 2.0 * fi);
-        Zo[o] = mkc<T2>(zn.x + dt * fr, zn.y + dt * fi);
-      } else {
-        const T2 a = acc[o];
-        const double h = dt / 6.0;
-        Zn[o] = mkc<T2>(zn.x + h * (a.x + fr), zn.y + h * (a.y + fi));
-      }
+      Zo[o] = f32 ? mkc<T2>(zn.x + fma(h6_lo, sx, h6_hi * sx), zn.y + fma(h6_lo, sy, h6_hi * sy))
+                  : mkc<T2>(fma(h6_hi, sx, zn.x), fma(h6_hi, sy, zn.y));
     }
   }
 }
 
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s) {
-  plain_gram<double2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0);
+  plain_gram<double2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, sq_table());
 }
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s) {
-  plain_gram<float2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0);
+  plain_gram<float2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, sq_table());
 }
 
 template <typename T2>
-void rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const T2* zin, T2* zout, int stage, double t,
-                cudaStream_t s) {
-  const int rhs_blocks = (int)((long)max_N * LR_MAX_RANK / PT / 2 + 1);
-  plain_rhs<T2><<<dim3(rhs_blocks, rp.n_traj), PT, 0, s>>>(p, rp, zin, zout, stage, t);
+void rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const T2* zin, T2* zout, int stage,
+                const double* coef, int cstride, cudaStream_t s) {
+  const int blocks = (int)(((long)max_N * (LR_MAX_RANK / 2) + RT - 1) / RT);   // those past a trajectory's rank leave at once
+  plain_rhs<T2><<<dim3(blocks, rp.n_traj), RT, 0, s>>>(p, rp, zin, zout, stage, coef, cstride, sq_table());
 }
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const double2* zin, double2* zout, int stage,
-                      double t, cudaStream_t s) {
-  rhs_launch(p, rp, max_N, zin, zout, stage, t, s);
+                      const double* coef, int cstride, cudaStream_t s) {
+  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, s);
 }
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const float2* zin, float2* zout, int stage,
-                      double t, cudaStream_t s) {
-  rhs_launch(p, rp, max_N, zin, zout, stage, t, s);
+                      const double* coef, int cstride, cudaStream_t s) {
+  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, s);
 }
 
 template <typename T2>
@@ -459,8 +513,6 @@ cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int
   T2* Za = reinterpret_cast<T2*>(p.Za);
   T2* Zb = reinterpret_cast<T2*>(p.Zb);
   const dim3 ggrid(max_nblk, rp.n_traj);
-  const int rhs_blocks = (int)((long)max_N * LR_MAX_RANK / PT / 2 + 1);
-  const dim3 rgrid(rhs_blocks < 1 ? 1 : rhs_blocks, rp.n_traj);
   for (long st = step0; st < step0 + n_steps; ++st) {
     const double tn = (double)st * rp.dt;
     const int record = (st % rp.pop_every) == 0;
@@ -468,9 +520,10 @@ cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int
       const T2* zin = stage == 0 ? Zn : (stage == 2 ? Zb : Za);
       T2* zout = stage == 1 ? Zb : (stage == 3 ? nullptr : Za);
       const double ts = tn + (stage == 0 ? 0.0 : (stage == 3 ? rp.dt : 0.5 * rp.dt));
-      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, zin, p.part, stage == 0 && record);
-      plain_solve<<<rp.n_traj, PT, 0, s>>>(p, rp, st, stage, stage == 0 && record, 1);
-      plain_rhs<T2><<<rgrid, PT, 0, s>>>(p, rp, zin, zout, stage, ts);
+      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, zin, p.part, stage == 0 && record, sq_table());
+      plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 && record ? LR_MAX_NT + 1 : 0, s);
+      plain_solve_launch(p, rp, nullptr, st, stage, stage == 0 && record, 1, ts, s);
+      rhs_launch(p, rp, max_N, zin, zout, stage, nullptr, 0, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -478,8 +531,9 @@ cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int
   // observables of the final state
   const long se = step0 + n_steps;
   const int record = (se % rp.pop_every) == 0;
-  plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Zn, p.part, record);
-  plain_solve<<<rp.n_traj, PT, 0, s>>>(p, rp, se, 0, record, 0);
+  plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Zn, p.part, record, sq_table());
+  plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, record ? LR_MAX_NT + 1 : 0, s);
+  plain_solve_launch(p, rp, nullptr, se, 0, record, 0, 0.0, s);
   return cudaGetLastError();
 }
 
