@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(AT) adj_bsolve(Ptrs a, int stage, double t_sta
 
 // Ubar_s for the cotangent Fbar (Fb). Thread: one row, the columns m and m + 1, with
 // the M x M factors in shared memory (rows of M | 1 entries: no bank conflicts along
-// a column either): 28 FMAs per column and l on the FP64 pipe, 75 us a stage at its
-// peak for 12 trajectories of N = 2000, M = 20, which with ~60 others is its bound.
+// a column either): 28 FMAs per column and l on the FP64 pipe, 448 us a stage at its
+// rate for 12 trajectories of N = 2000, M = 20; 522 us with the ~60 others (ncu).
 constexpr int VT = 128;
 template <typename T2>
 __global__ void __launch_bounds__(VT) adj_vjp(Ptrs a, const T2* __restrict__ U, const T2* __restrict__ Fb, int stage,

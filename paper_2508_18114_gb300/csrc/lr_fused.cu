@@ -104,6 +104,52 @@ int rows_per_cta(const TrajDev& d, int C) {
   return d.Nt * ((d.Nr + C - 1) / C) * d.Nf;
 }
 
+// The wide schedule (four launches per RK4 stage, each over the whole chip) against the
+// teams: a team holds a trajectory on at most min(16, N_r) SMs, so a batch of one or
+// two candidates leaves most of the chip idle. Estimates in us per stage, fitted on
+// GB300 to 1 to 16 candidates of 13 models (M = 4 .. 32, N = 40 .. 9600):
+//   teams: 2.05 M (1.5 M on one CTA; the M x M phase and the barrier) + rows per CTA x
+//          M (M + 11) x 1.7e-4 (stage state in L2: 2.3e-4; two modes, shared memory: 1e-4),
+//          for every wave of teams;
+//   wide:  20 + 1.1 M (launches and the M x M phase) + 4.6e-6 x sum N M (M + 11).
+// Measured, teams / wide: N = 2000, M = 20, 1 candidate 62 / 47, 2 candidates 62 / 61;
+// N = 480, M = 32 (two modes) 202 / 62, 8 candidates 203 / 114; N = 8000, M = 32 269 /
+// 148; N = 2000, M = 10 32 / 35; N = 40, M = 4 10 / 28. The line lies at 0.9, where no
+// measured batch lost more than 1%.
+bool wide_is_faster(const std::vector<TrajDev>& traj, const FusedPlan& plan) {
+  double team = 0.0, wide = 0.0;
+  for (const TrajDev& d : traj) {
+    const double w = d.M * (d.M + 11.0);
+    const double slope = !plan.zs_smem ? 2.3e-4 : (d.n_modes == 2 ? 1.0e-4 : 1.7e-4);
+    team = std::max(team, (plan.C > 1 ? 2.05 : 1.5) * d.M + slope * w * rows_per_cta(d, plan.C));
+    wide = std::max(wide, 20.0 + 1.1 * d.M);
+  }
+  for (const TrajDev& d : traj) wide += 4.6e-6 * d.N * d.M * (d.M + 11.0);
+  const int waves = ((int)traj.size() + plan.n_clusters - 1) / plan.n_clusters;
+  return wide < 0.9 * waves * team;
+}
+
+// Wide schedule: two stage buffers and the accumulator, X_k, partial sums, from `off`.
+struct WideLayout {
+  size_t za, zb, acc, x, part, total;
+};
+WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  WideLayout L{};
+  L.za = take(sizeof(float2) * plan.tot);
+  L.zb = take(sizeof(float2) * plan.tot);
+  L.acc = take(sizeof(float2) * plan.tot);
+  L.x = take(sizeof(double2) * 2 * LR_MAX_RANK * LR_MAX_RANK * n_traj);
+  L.part = take(sizeof(double) * plan.part);
+  L.total = off;
+  return L;
+}
+size_t order_bytes(int n_traj) { return ((sizeof(int) * n_traj + 255) / 256) * 256; }
+
 }  // namespace
 
 bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, FusedPlan* plan) {
@@ -131,7 +177,8 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
   }
   const int Mp = (Mmax + 3) / 4 * 4;
   // Variants (stage state placement, tensor-core passes of the projection).
-  // Overrides for tuning and tests: LR_FUSED_C = cluster size, LR_FUSED_ZS =
+  // Overrides for tuning and tests: LR_FUSED_WIDE = 0 / 1 (teams / wide schedule, FP32_G64),
+  // LR_FUSED_C = cluster size, LR_FUSED_ZS =
   // "global" keeps the stage state in L2, LR_FUSED_TC = 0 keeps the FP32_G64
   // projection on the CUDA cores (3: only the tensor-core variant).
   int force_c = 0, force_global = 0, force_tc = -1, gram_dw = 0;
@@ -241,6 +288,14 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
     }
   }
   if (!plan->ok) return false;
+  for (const TrajDev& d : traj) {
+    plan->max_nblk = std::max(plan->max_nblk, d.nblk);
+    plan->tot += (long long)d.N * d.M;
+    plan->part += (long long)d.nblk * (long long)plain_pstride(d.M);
+  }
+  plan->wide = prec == LR_PREC_FP32_G64 && !force_c && !force_global && force_tc < 0 && !gram_dw &&
+               wide_is_faster(traj, *plan);
+  if (const char* e = getenv("LR_FUSED_WIDE")) plan->wide = prec == LR_PREC_FP32_G64 && atoi(e);
   // largest work first, round-robin over the teams
   std::vector<std::pair<double, int>> w;
   for (size_t j = 0; j < traj.size(); ++j)
@@ -252,7 +307,8 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
 
 size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj) {
   // order list, then global stage buffers (only without smem residency) and accumulators per team
-  size_t b = ((sizeof(int) * n_traj + 255) / 256) * 256;
+  size_t b = order_bytes(n_traj);
+  if (plan.wide) return wide_layout(plan, n_traj, b).total;
   const size_t es = plan.es;
   if (!plan.zs_smem)
     b += ((2 * (size_t)plan.R * (plan.Mp + 1) * es * plan.C * plan.n_clusters + 255) / 256) * 256;
@@ -263,6 +319,7 @@ size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj) {
 cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratch, int n_traj) {
   cudaError_t e = cudaMemcpy(scratch, plan.order.data(), sizeof(int) * n_traj, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
+  if (plan.wide) return cudaSuccess;
   const size_t es = prec == LR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const SmemLayout L = layout(plan.R, plan.Mp, plan.zs_smem, es, plan.tc, plan.gram_mode == 2);
   const void* kern = kernel_ptr(prec, plan.zs_smem, plan.tc, plan.frame, plan.gram_mode);
@@ -273,6 +330,17 @@ cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratc
 
 cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunParams& rp, lr_precision prec,
                             long step0, long n_steps, cudaStream_t s) {
+  if (plan.wide) {
+    const WideLayout L = wide_layout(plan, rp.n_traj, order_bytes(rp.n_traj));
+    char* sc = static_cast<char*>(p.scratch);
+    DevPtrs q = p;
+    q.Za = sc + L.za;
+    q.Zb = sc + L.zb;
+    q.acc = sc + L.acc;
+    q.X = reinterpret_cast<double2*>(sc + L.x);
+    q.part = reinterpret_cast<double*>(sc + L.part);
+    return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, s);
+  }
   const size_t es = prec == LR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const SmemLayout L = layout(plan.R, plan.Mp, plan.zs_smem, es, plan.tc, plan.gram_mode == 2);
   fz::Args a{};
@@ -303,7 +371,7 @@ cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunPa
   a.npad = L.npad;
   a.o_gs = L.o_gs;
   char* sc = static_cast<char*>(p.scratch);
-  size_t off = ((sizeof(int) * rp.n_traj + 255) / 256) * 256;
+  size_t off = order_bytes(rp.n_traj);
   a.order = reinterpret_cast<const int*>(sc);
   if (!plan.zs_smem) {
     a.zs_glob = sc + off;

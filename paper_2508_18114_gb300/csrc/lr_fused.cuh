@@ -30,6 +30,9 @@ struct FusedPlan {
   int Nmax;        // largest N in the batch
   int gram_mode;   // 0 native (bulk type), 1 double-word FP32 (FP64-class), 2 on the tensor cores (FP64-class)
   int es;          // bytes per complex state element
+  int wide;        // 1: the wide schedule (a few launches per stage over the whole chip) in place of the teams
+  int max_nblk;    // its row blocks, state elements and partial sums (doubles)
+  long long tot, part;
   std::vector<int> order;   // trajectories, largest work first
 };
 

@@ -258,12 +258,12 @@ cudaError_t launch_diagnostics(const DevPtrs& p, const RunParams& rp, long n_val
 // lr_plain.cu
 int plain_rows_per_block();
 size_t plain_partial_doubles(int M);
-// The plain engine on complex128 state (the reference GPU path), or on
-// complex64 state (fp32 = 1: the adjoint's FP32-bulk recomputation; the Gram
-// matrix is summed from exact products in double-word FP32, Cholesky and solves
-// in FP64, the rest in FP32).
+// The plain engine: complex128 state, the reference GPU path.
 cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0,
-                            long n_steps, cudaStream_t s, int fp32 = 0);
+                            long n_steps, cudaStream_t s);
+// Its kernels on complex64 state as the wide schedule of the fused engine: n_steps from
+// the device's step counter p.dstep; p.Za, p.Zb, p.acc, p.X and p.part in its scratch.
+cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s);
 // single kernels of the plain engine (used by the adjoint's recomputation)
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s);
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s);

@@ -240,4 +240,75 @@ __device__ __forceinline__ double2 mm_xk(const double2* gi, const double2* t, in
   return mk(xr, xi);
 }
 
+// ----------------------------------------------------------------- whole-chip schedules
+// Entry e of the upper triangle by columns: (i, j), i <= j (the lower one by rows: (j, i)).
+__device__ __forceinline__ void tri_entry(int e, int& i, int& j) {
+  j = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+  while (j * (j + 1) / 2 > e) --j;
+  while ((j + 1) * (j + 2) / 2 <= e) ++j;
+  i = e - j * (j + 1) / 2;
+}
+
+constexpr int ST = 544;   // threads of the solve kernels: one entry of the 32 x 32 triangle each
+
+// The FP64 entry arithmetic of the sweeps; a pivot counts as zero where it is lost in
+// the rounding of M updates of its diagonal entry (LR_MAX_RANK 2^-51 of it), so that a
+// rank-deficient state is told whatever the sign of that rounding.
+struct WidePivot : F64Arith {
+  static __device__ __forceinline__ double recip(double2 p) {
+    return p.x > 1e-30 && p.x < 1e30 ? F64Arith::recip(p) : 1.0 / p.x;
+  }
+  static __device__ __forceinline__ bool breakdown(double2 p, double d0) {
+    return !(p.x > LR_MAX_RANK * 0x1p-51 * d0) || !isfinite(p.x);
+  }
+};
+// Entries of G and T from their FP64 sums. FP32 state: G in double-word FP32 and an FP32
+// T, as in the fused kernels (a sweep of double-word FP32 takes ~2/3 of an FP64 one).
+__device__ __forceinline__ void to_entry(double2 v, double2& e) { e = v; }
+__device__ __forceinline__ void to_entry(double2 v, DWC& e) {
+  e.re.hi = (float)v.x;
+  e.re.lo = (float)(v.x - (double)e.re.hi);
+  e.im.hi = (float)v.y;
+  e.im.lo = (float)(v.y - (double)e.im.hi);
+}
+__device__ __forceinline__ void to_entry(double2 v, float2& e) { e = make_float2((float)v.x, (float)v.y); }
+__device__ __forceinline__ double2 to_sum(double2 v) { return v; }
+__device__ __forceinline__ double2 to_sum(float2 v) { return mk((double)v.x, (double)v.y); }
+template <typename A> struct XEntry { using t = double2; };
+template <> struct XEntry<DwArith> { using t = float2; };
+
+// The block's share of X_k = G^-1 T_k: whole columns of the K M of all jumps, XC at a
+// time with their T entries in shared memory (read from L2 in the dot products, a
+// chain of M loads, they took as long as the sweeps).
+constexpr int XC = 8;
+template <typename A>
+struct XColumns {
+  typename XEntry<A>::t t[XC][LR_MAX_RANK + 1];
+  // columns [c0, c0 + n) of T [K][M][M]
+  __device__ __forceinline__ void load(const double2* T, int M, int c0, int n, int tid) {
+    for (int e = tid; e < n * M; e += ST) {
+      const int c = e / M, l = e - c * M, k = (c0 + c) / M, j = c0 + c - k * M;
+      to_entry(T[(k * M + l) * M + j], t[c][l]);
+    }
+  }
+};
+// Called by every thread with the first columns loaded and G^-1 in Gs, both behind a
+// barrier; put(k, i, j, X_ij) stores.
+template <typename A, typename Put>
+__device__ __forceinline__ void x_columns(XColumns<A>& xc, const typename A::C* Gs, int ldg, const double2* T, int M, int lo,
+                                          int hi, int tid, Put put) {
+  for (int c0 = lo; c0 < hi; c0 += XC) {
+    const int n = min(XC, hi - c0);
+    if (c0 > lo) {
+      __syncthreads();
+      xc.load(T, M, c0, n, tid);
+      __syncthreads();
+    }
+    for (int e = tid; e < n * M; e += ST) {
+      const int c = e / M, i = e - c * M, k = (c0 + c) / M;
+      put(k, i, c0 + c - k * M, to_sum(mm_xk(Gs + i * ldg, xc.t[c], 1, M)));
+    }
+  }
+}
+
 }  // namespace lr

@@ -44,9 +44,16 @@ __host__ __device__ inline size_t pstride(int M) { return plain_pstride(M); }
 int plain_rows_per_block() { return PR; }
 size_t plain_partial_doubles(int M) { return pstride(M); }
 
+// The RK4 step of a launch on the device: *dstep + k of a run of n steps (the wide
+// schedule, which may be replayed from a graph); dstep null: the host's arguments.
+struct StepRef {
+  const long long* dstep = nullptr;
+  long k = 0, n = 0;
+};
+
 template <typename T2>
 __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ traj, const T2* __restrict__ Zin,
-                                                 double* __restrict__ part, int with_obs,
+                                                 double* __restrict__ part, int with_obs, StepRef sr, int pop_every,
                                                  const __grid_constant__ SqTab sq) {
   using T = typename real_of<T2>::type;
   const TrajDev d = traj[blockIdx.y];
@@ -95,10 +102,7 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
   for (int e0 = threadIdx.x; e0 < ne + 2 * MM; e0 += blockDim.x) {
     int mat = 0, i, j;
     if (e0 < ne) {
-      j = (int)((sqrtf(8.f * e0 + 1.f) - 1.f) * 0.5f);
-      while (j * (j + 1) / 2 > e0) --j;
-      while ((j + 1) * (j + 2) / 2 <= e0) ++j;
-      i = e0 - j * (j + 1) / 2;   // i <= j
+      tri_entry(e0, i, j);
     } else {
       const int e1 = e0 - ne;
       mat = 1 + e1 / MM;
@@ -149,6 +153,7 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
       out[2 * e + 1] = (double)im;
     }
   }
+  if (with_obs && sr.dstep) with_obs = (*sr.dstep + sr.k) % pop_every == 0;
   if (with_obs) {
     for (int i = threadIdx.x; i < PR; i += blockDim.x) {
       double w = 0.0;
@@ -172,54 +177,43 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
   }
 }
 
-// Entry o < a M^2 + b of every trajectory: the row blocks' partial sums in block
-// order, into block 0's. One thread per entry over the whole chip: in the one block
-// per trajectory that solves, the 125 partials of N = 2000, M = 20 (3e5 FP64 adds)
-// took ~75 us of one SM.
+// Entry o < a M^2 + b of every trajectory: the row blocks' partial sums into block
+// 0's, warp w of a block adding blocks w, w + 8, ... of 32 entries, then the eight warps
+// in order. Bound by the latency of the loads, eight of a thread in flight: ~2 us for
+// the 125 blocks of N = 2000 (one thread per entry: ~5 us; in the one block per
+// trajectory that solves, 3e5 FP64 adds at M = 20, ~75 us of one SM).
 __global__ void __launch_bounds__(PT) plain_reduce(const TrajDev* __restrict__ traj, double* __restrict__ part, int a,
                                                    int b) {
+  __shared__ double sh[PT / 32][32];
   const TrajDev d = traj[blockIdx.y];
-  const int o = blockIdx.x * PT + threadIdx.x;
-  if (o >= a * d.M * d.M + b) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = blockIdx.x * 32 + lane, no = a * d.M * d.M + b;
+  if ((int)blockIdx.x * 32 >= no) return;
   double* P = part + d.p_off + o;
   const size_t ps = pstride(d.M);
   double s = 0.0;
-  int k = 0;
-  for (; k + 8 <= d.nblk; k += 8) {   // eight loads in flight
-    double v[8];
+  if (o < no)
+    for (int k0 = warp; k0 < d.nblk; k0 += 64) {
+      double v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = P[(k + u) * ps];
+      for (int u = 0; u < 8; ++u) v[u] = k0 + 8 * u < d.nblk ? P[(size_t)(k0 + 8 * u) * ps] : 0.0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) s += v[u];
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+  sh[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && o < no) {
+    for (int w = 1; w < PT / 32; ++w) s += sh[w][lane];
+    P[0] = s;
   }
-  for (; k < d.nblk; ++k) s += P[k * ps];
-  P[0] = s;
 }
 
 void plain_reduce_launch(const TrajDev* traj, int n_traj, int max_M, double* part, int a, int b, cudaStream_t s) {
-  plain_reduce<<<dim3((a * max_M * max_M + b + PT - 1) / PT, n_traj), PT, 0, s>>>(traj, part, a, b);
-}
-
-// The FP64 entry arithmetic of the sweeps; a pivot counts as zero where it is lost in
-// the rounding of M updates of its diagonal entry (LR_MAX_RANK 2^-51 of it), so that a
-// rank-deficient state is told whatever the sign of that rounding.
-struct WidePivot : F64Arith {
-  static __device__ __forceinline__ double recip(double2 p) {
-    return p.x > 1e-30 && p.x < 1e30 ? F64Arith::recip(p) : 1.0 / p.x;
-  }
-  static __device__ __forceinline__ bool breakdown(double2 p, double d0) {
-    return !(p.x > LR_MAX_RANK * 0x1p-51 * d0) || !isfinite(p.x);
-  }
-};
-__device__ __forceinline__ double2 mac(double2 a, double2 b, double2 s) {   // s + a b
-  return mk(fma(a.x, b.x, fma(-a.y, b.y, s.x)), fma(a.x, b.y, fma(a.y, b.x, s.y)));
+  plain_reduce<<<dim3((a * max_M * max_M + b + 31) / 32, n_traj), PT, 0, s>>>(traj, part, a, b);
 }
 
 // Two doubles of the reduced sums carry the drive coefficient from plain_solve to
 // plain_rhs: the one after the populations, and the imaginary part of G_00.
 __device__ __forceinline__ double* drive_slot(double* P, int M, int c) { return P + (c ? 1 : 6 * M * M + LR_MAX_NT + 1); }
-
-constexpr int ST = 544;   // threads of plain_solve: one entry of the 32 x 32 triangle each
 
 // From the sums in the trajectory's first row block: G^-1 by symmetric sweeps and X_k
 // = G^-1 T_k (G^-1 to Gi unless null); at stage 0 the readout signal and the records;
@@ -227,22 +221,40 @@ constexpr int ST = 544;   // threads of plain_solve: one entry of the 32 x 32 tr
 // (latency, ~1000 cycles a sweep in FP64) and its share of X_k, whose 8 M^3 FMAs
 // take one SM 31k cycles at M = 20. It replaces a Cholesky factorisation and two
 // triangular sweeps over 2 M columns in one block, ~70 barriers of FP64 latency.
+// A: WidePivot, or DwArith for the FP32 state of the wide schedule (Gi null then).
+// StepRef: the step and the record are the device counter's.
+template <typename A>
 __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, double2* __restrict__ Gi, long step, int stage,
-                                                  int record, int do_solve, double t) {
+                                                  int record, int do_solve, double t, StepRef sr) {
+  if (sr.dstep) {
+    const long s0 = (long)*sr.dstep;
+    if (s0 < 0 || s0 + sr.n > rp.max_steps) {   // every launch of the schedule leaves
+      if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_error(p.err, DEV_CAPACITY);
+      return;
+    }
+    step = s0 + sr.k;
+    record = stage == 0 && step % rp.pop_every == 0;
+    t += (double)step * rp.dt;
+  }
   const int tj = blockIdx.y, g = blockIdx.x;
   const TrajDev d = p.traj[tj];
   const int M = d.M, MM = M * M, tid = threadIdx.x, ldg = M | 1;
-  __shared__ double2 Gs[LR_MAX_RANK * (LR_MAX_RANK + 1)];
+  __shared__ typename A::C Gs[LR_MAX_RANK * (LR_MAX_RANK + 1)];
   __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
-  __shared__ MmShared<WidePivot> mm;
+  __shared__ MmShared<A> mm;
+  __shared__ XColumns<A> xc;
   double* Pd = p.part + d.p_off;
   const double2* P = reinterpret_cast<const double2*>(Pd);   // p_off and the block size are even
   if (g == 0 && stage == 0) {
-    if (tid == ST - 1) {
-      double2 b = mk(0.0, 0.0);
-      for (int i = 0; i < M; ++i) b = mk(b.x + P[MM + i * M + i].x, b.y + P[MM + i * M + i].y);
-      p.beta[(size_t)tj * (rp.max_steps + 1) + step] = b;
-      if (!isfinite(b.x) || !isfinite(b.y)) set_error(p.err, DEV_NONFINITE);
+    if (tid >= ST - 32) {   // tr T_r, one lane per diagonal entry
+      const int i = tid - (ST - 32);
+      double2 b = i < M ? P[MM + i * M + i] : mk(0.0, 0.0);
+      for (int o = 16; o > 0; o >>= 1)
+        b = mk(b.x + __shfl_xor_sync(0xffffffffu, b.x, o), b.y + __shfl_xor_sync(0xffffffffu, b.y, o));
+      if (i == 0) {
+        p.beta[(size_t)tj * (rp.max_steps + 1) + step] = b;
+        if (!isfinite(b.x) || !isfinite(b.y)) set_error(p.err, DEV_NONFINITE);
+      }
     }
     if (record) {
       const long rec = step / rp.pop_every;
@@ -267,7 +279,11 @@ __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, doubl
     }
   }
   if (!do_solve) return;
-  if (g == (gridDim.x > 1 ? 1 : 0) && tid == ST - 33 && t >= 0.0) {
+  // the drive coefficient: ~12k cycles of FP64 latency, beside the sweeps of the warps
+  // that hold entries where one is left (M < 32)
+  const int nw = mm_warps(M, ST / 32);
+  auto drive = [&]() {
+    if (g != (gridDim.x > 1 ? 1 : 0) || tid != ST - 1 || t < 0.0) return;
     const PulseDev pulse = p.pulse[d.cand];
     if (rp.frame) {
       const double2 w = pulse_rwa_drive(pulse, rp.tau, t);
@@ -276,42 +292,49 @@ __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, doubl
     } else {
       *drive_slot(Pd, M, 0) = pulse_coefficient(pulse, rp.tau, t);
     }
-  }
+  };
+  const int per = (2 * M + gridDim.x - 1) / gridDim.x, c_lo = g * per, c_hi = min(2 * M, c_lo + per);
+  xc.load(P + MM, M, c_lo, min(XC, c_hi - c_lo), tid);
   if (tid == 0) mm.bad = 0;
-  for (int i = tid; i < M; i += ST)
-    for (int j = 0; j <= i; ++j) tri[i * (i + 1) / 2 + j] = make_short2((short)i, (short)j);
+  if (tid < M * (M + 1) / 2) {
+    int i, j;
+    tri_entry(tid, i, j);
+    tri[tid] = make_short2((short)j, (short)i);
+  }
   __syncthreads();
-  if (tid / 32 < mm_warps(M, ST / 32)) {
-    double2 e[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};   // the sums hold the upper triangle
+  if (tid / 32 < nw) {
+    typename A::C e[2] = {A::zero(), A::zero()};   // the sums hold the upper triangle
     if (tid < M * (M + 1) / 2) {
       const int i = tri[tid].x, j = tri[tid].y;
       const double2 v = P[j * M + i];
-      e[0] = mk(v.x, i == j ? 0.0 : -v.y);
+      to_entry(mk(v.x, i == j ? 0.0 : -v.y), e[0]);
     }
-    mm_invert<WidePivot, ST>(e, Gs, ldg, mm, tri, M, tid);
+    mm_invert<A, ST>(e, Gs, ldg, mm, tri, M, tid);
+    if (nw == ST / 32) drive();
+  } else {
+    drive();
   }
   __syncthreads();
   if (g == 0) {
     if (tid == 0 && mm.bad) set_error(p.err, DEV_NOT_PD);
     if (Gi)
-      for (int e = tid; e < MM; e += ST) Gi[(size_t)tj * LR_MAX_RANK * LR_MAX_RANK + e] = Gs[(e / M) * ldg + e % M];
+      for (int e = tid; e < MM; e += ST)
+        Gi[(size_t)tj * LR_MAX_RANK * LR_MAX_RANK + e] = A::value(Gs[(e / M) * ldg + e % M]);
   }
   double2* X = p.X + (size_t)tj * 2 * LR_MAX_RANK * LR_MAX_RANK;
-  const int per = (2 * MM + gridDim.x - 1) / gridDim.x;
-  for (int e = g * per + tid; e < min(2 * MM, (g + 1) * per); e += ST) {
-    const int k = e / MM, ij = e - k * MM, i = ij / M, j = ij - i * M;
-    const double2* tk = P + (1 + k) * MM + j;
-    double2 s = mk(0.0, 0.0);
-    for (int l = 0; l < M; ++l) s = mac(Gs[i * ldg + l], tk[l * M], s);
-    X[k * LR_MAX_RANK * LR_MAX_RANK + ij] = s;
-  }
+  x_columns<A>(xc, Gs, ldg, P + MM, M, c_lo, c_hi, tid, [&](int k, int i, int j, double2 v) {
+    X[k * LR_MAX_RANK * LR_MAX_RANK + i * M + j] = v;
+  });
 }
 
+// a trajectory's share of two blocks per SM, at most eight
+static int solve_blocks(const RunParams& rp, int do_solve) {
+  return do_solve ? std::max(1, std::min(8, 304 / rp.n_traj)) : 1;
+}
 void plain_solve_launch(const DevPtrs& p, const RunParams& rp, double2* Gi, long step, int stage, int record, int do_solve,
                         double t, cudaStream_t s) {
-  // a trajectory's share of two blocks per SM, at most eight
-  const int blocks = do_solve ? std::max(1, std::min(8, 304 / rp.n_traj)) : 1;
-  plain_solve<<<dim3(blocks, rp.n_traj), ST, 0, s>>>(p, rp, Gi, step, stage, record, do_solve, t);
+  plain_solve<WidePivot><<<dim3(solve_blocks(rp, do_solve), rp.n_traj), ST, 0, s>>>(p, rp, Gi, step, stage, record,
+                                                                                    do_solve, t, StepRef{});
 }
 
 // Thread: one row, the columns m and m + 1. Bound by the FP64 pipe for the
@@ -321,8 +344,9 @@ constexpr int RT = 128;   // threads per block
 template <typename T2>
 __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T2* __restrict__ Zin,
                                                 T2* __restrict__ Zout, int stage,
-                                                const double* __restrict__ ctab, int cstride,
+                                                const double* __restrict__ ctab, int cstride, StepRef ref,
                                                 const __grid_constant__ SqTab sq) {
+  if (ref.dstep && (*ref.dstep < 0 || *ref.dstep + ref.n > rp.max_steps)) return;
   using T = typename real_of<T2>::type;
   constexpr bool f32 = sizeof(T) == 4;
   const int tj = blockIdx.y;
@@ -383,57 +407,63 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
       }
     }
   }
-  auto add_row = [&](int off, T w) {
-    const T2* v = zrow + (long)off * ld;
-    const T2 v0 = v[m], v1 = v[m1];
-    hr[0] = fma(w, v0.x, hr[0]);
-    hi[0] = fma(w, v0.y, hi[0]);
-    hr[1] = fma(w, v1.x, hr[1]);
-    hi[1] = fma(w, v1.y, hi[1]);
+  // The neighbours' offsets and weights first (an absent one is the row itself with
+  // weight zero), so that their loads are in flight together: complex weights on the
+  // readout mode in the rotating frame only.
+  int off[10];
+  T w[10];
+  T wi = 0;
+  int na = 0;
+  auto add = [&](bool on, int o, T wt) {
+    off[na] = on ? o : 0;
+    w[na++] = on ? wt : (T)0;
   };
-  // g (b + b^dag)(a + a^dag)
+  // g (b + b^dag)(a + a^dag); RWA keeps g (b^dag a + b a^dag) only
 #pragma unroll
   for (int a = -1; a <= 1; a += 2) {
     const int it2 = ri.it + a;
-    if (it2 < 0 || it2 >= d.Nt) continue;
-    const double ct = sq_of(sq, max(ri.it, it2));
+    const bool ot = it2 >= 0 && it2 < d.Nt;
+    const T ct = (T)d.g * (T)sq_of(sq, max(ri.it, it2));
 #pragma unroll
     for (int bb = -1; bb <= 1; bb += 2) {
       const int ir2 = ri.ir + bb;
-      if (ir2 < 0 || ir2 >= d.Nr) continue;
-      if (rwa && a == bb) continue;   // RWA keeps g (b^dag a + b a^dag) only
-      add_row(a * st + bb * sr, (T)(d.g * ct * sq_of(sq, max(ri.ir, ir2))));
+      add(ot && ir2 >= 0 && ir2 < d.Nr && !(rwa && a == bb), a * st + bb * sr, ct * (T)sq_of(sq, max(ri.ir, ir2)));
     }
   }
-  if (d.n_modes == 3) {
-    // J (a + a^dag)(f + f^dag)
+  // J (a + a^dag)(f + f^dag); RWA keeps J (a^dag f + a f^dag) only
 #pragma unroll
-    for (int a = -1; a <= 1; a += 2) {
-      const int ir2 = ri.ir + a;
-      if (ir2 < 0 || ir2 >= d.Nr) continue;
-      const double cr = sq_of(sq, max(ri.ir, ir2));
+  for (int a = -1; a <= 1; a += 2) {
+    const int ir2 = ri.ir + a;
+    const bool or2 = d.n_modes == 3 && ir2 >= 0 && ir2 < d.Nr;
+    const T cr = (T)d.J * (T)sq_of(sq, max(ri.ir, ir2));
 #pragma unroll
-      for (int bb = -1; bb <= 1; bb += 2) {
-        const int if2 = ri.iff + bb;
-        if (if2 < 0 || if2 >= d.Nf) continue;
-        if (rwa && a == bb) continue;   // RWA keeps J (a^dag f + a f^dag) only
-        add_row(a * sr + bb, (T)(d.J * cr * sq_of(sq, max(ri.iff, if2))));
-      }
+    for (int bb = -1; bb <= 1; bb += 2) {
+      const int if2 = ri.iff + bb;
+      add(or2 && if2 >= 0 && if2 < d.Nf && !(rwa && a == bb), a * sr + bb, cr * (T)sq_of(sq, max(ri.iff, if2)));
     }
   }
   // drive on the readout mode (stride 1): lab frame c(t) (r + r^dag); RWA
   // w r + conj(w) r^dag with w = c + i ci (row n gets r from n+1, r^dag from n-1)
   const int iro = readout_index(d, ri), dro = readout_dim(d);
+  T sd[2];
 #pragma unroll
   for (int a = -1; a <= 1; a += 2) {
     const int i2 = iro + a;
-    if (i2 < 0 || i2 >= dro) continue;
-    const T s = (T)sq_of(sq, max(iro, i2));
-    add_row(a, c * s);
-    if (rwa) {
-      const T wi = (a > 0 ? ci : -ci) * s;
-      const T2* v = zrow + (long)a * ld;
-      const T2 v0 = v[m], v1 = v[m1];
+    const bool on = i2 >= 0 && i2 < dro;
+    const T s = on ? (T)sq_of(sq, max(iro, i2)) : (T)0;
+    sd[a > 0] = s;
+    add(on, a, c * s);
+  }
+#pragma unroll
+  for (int q = 0; q < 10; ++q) {
+    const T2* v = zrow + (long)off[q] * ld;
+    const T2 v0 = v[m], v1 = v[m1];
+    hr[0] = fma(w[q], v0.x, hr[0]);
+    hi[0] = fma(w[q], v0.y, hi[0]);
+    hr[1] = fma(w[q], v1.x, hr[1]);
+    hi[1] = fma(w[q], v1.y, hi[1]);
+    if (q >= 8 && rwa) {
+      wi = (q == 9 ? ci : -ci) * sd[q - 8];
       hr[0] = fma(-wi, v0.y, hr[0]);
       hi[0] = fma(wi, v0.x, hi[0]);
       hr[1] = fma(-wi, v1.y, hr[1]);
@@ -445,6 +475,7 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
   // + 1/2 kappa (rZ) X_r^dag + 1/2 gamma (bZ) X_b^dag
   auto project = [&](const T2* y, const T2* x, T s) {
     T pr[2] = {0, 0}, pi[2] = {0, 0};
+#pragma unroll 8
     for (int l = 0; l < M; ++l) {
       const T2 v = y[l], x0 = x[l * M + m], x1 = x[l * M + m1];   // v conj(x)
       pr[0] = fma(v.x, x0.x, fma(v.y, x0.y, pr[0]));
@@ -485,29 +516,29 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
 }
 
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s) {
-  plain_gram<double2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, sq_table());
+  plain_gram<double2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, StepRef{}, 1, sq_table());
 }
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s) {
-  plain_gram<float2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, sq_table());
+  plain_gram<float2><<<dim3(max_nblk, rp.n_traj), PT, 0, s>>>(p.traj, zin, p.part, 0, StepRef{}, 1, sq_table());
 }
 
 template <typename T2>
 void rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const T2* zin, T2* zout, int stage,
-                const double* coef, int cstride, cudaStream_t s) {
+                const double* coef, int cstride, StepRef ref, cudaStream_t s) {
   const int blocks = (int)(((long)max_N * (LR_MAX_RANK / 2) + RT - 1) / RT);   // those past a trajectory's rank leave at once
-  plain_rhs<T2><<<dim3(blocks, rp.n_traj), RT, 0, s>>>(p, rp, zin, zout, stage, coef, cstride, sq_table());
+  plain_rhs<T2><<<dim3(blocks, rp.n_traj), RT, 0, s>>>(p, rp, zin, zout, stage, coef, cstride, ref, sq_table());
 }
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const double2* zin, double2* zout, int stage,
                       const double* coef, int cstride, cudaStream_t s) {
-  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, s);
+  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, StepRef{}, s);
 }
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const float2* zin, float2* zout, int stage,
                       const double* coef, int cstride, cudaStream_t s) {
-  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, s);
+  rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, StepRef{}, s);
 }
 
 template <typename T2>
-cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0, long n_steps,
+static cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0, long n_steps,
                         cudaStream_t s) {
   T2* Zn = reinterpret_cast<T2*>(p.Zn);
   T2* Za = reinterpret_cast<T2*>(p.Za);
@@ -520,10 +551,10 @@ cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int
       const T2* zin = stage == 0 ? Zn : (stage == 2 ? Zb : Za);
       T2* zout = stage == 1 ? Zb : (stage == 3 ? nullptr : Za);
       const double ts = tn + (stage == 0 ? 0.0 : (stage == 3 ? rp.dt : 0.5 * rp.dt));
-      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, zin, p.part, stage == 0 && record, sq_table());
+      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, zin, p.part, stage == 0 && record, StepRef{}, 1, sq_table());
       plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 && record ? LR_MAX_NT + 1 : 0, s);
       plain_solve_launch(p, rp, nullptr, st, stage, stage == 0 && record, 1, ts, s);
-      rhs_launch(p, rp, max_N, zin, zout, stage, nullptr, 0, s);
+      rhs_launch(p, rp, max_N, zin, zout, stage, nullptr, 0, StepRef{}, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -531,16 +562,38 @@ cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int
   // observables of the final state
   const long se = step0 + n_steps;
   const int record = (se % rp.pop_every) == 0;
-  plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Zn, p.part, record, sq_table());
+  plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Zn, p.part, record, StepRef{}, 1, sq_table());
   plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, record ? LR_MAX_NT + 1 : 0, s);
   plain_solve_launch(p, rp, nullptr, se, 0, record, 0, 0.0, s);
   return cudaGetLastError();
 }
 
 cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0,
-                            long n_steps, cudaStream_t s, int fp32) {
-  return fp32 ? integrate_t<float2>(p, rp, max_nblk, max_N, step0, n_steps, s)
-              : integrate_t<double2>(p, rp, max_nblk, max_N, step0, n_steps, s);
+                            long n_steps, cudaStream_t s) {
+  return integrate_t<double2>(p, rp, max_nblk, max_N, step0, n_steps, s);
+}
+
+// The wide schedule of the fused engine: complex64 state, double-word Gram and M x M
+// phase, the step counter on the device. The buffers of p are the caller's.
+cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s) {
+  float2* Z[4] = {reinterpret_cast<float2*>(p.Zn), reinterpret_cast<float2*>(p.Za), reinterpret_cast<float2*>(p.Zb),
+                  reinterpret_cast<float2*>(p.Za)};
+  const dim3 ggrid(max_nblk, rp.n_traj);
+  const double c[4] = {0.0, 0.5 * rp.dt, 0.5 * rp.dt, rp.dt};
+  for (long k = 0; k <= n_steps; ++k) {
+    const StepRef ref{p.dstep, k, n_steps};
+    for (int stage = 0; stage < (k < n_steps ? 4 : 1); ++stage) {
+      const int solve = k < n_steps;
+      plain_gram<float2><<<ggrid, PT, 0, s>>>(p.traj, Z[stage], p.part, stage == 0, ref, rp.pop_every, sq_table());
+      plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 ? LR_MAX_NT + 1 : 0, s);
+      plain_solve<DwArith><<<dim3(solve_blocks(rp, solve), rp.n_traj), ST, 0, s>>>(p, rp, nullptr, 0, stage, 0, solve,
+                                                                                   c[stage], ref);
+      if (solve) rhs_launch(p, rp, max_N, Z[stage], stage < 3 ? Z[stage + 1] : nullptr, stage, nullptr, 0, ref, s);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace lr
