@@ -2,21 +2,21 @@
 // channels: the paper's own model of Sec. S2 (built by lr_paper_model.cu) or
 // any other H_eff(t), L_k(t), r with that structure.
 //
-// One RK4 stage of Eq. S5 is four launches:
-//   sp_apply  - one thread per element (n, m) of the stage input Zs:
-//               W = A(t) Zs with A = -i H_eff, Y_k = L_k(t) Zs, and at stage 1
-//               of every step Yr = r Zs; the ten channel factors
-//               Omega(t)^a e^{i q w_d t} of the step's four stage times come
-//               from sp_chi, one small launch per step;
+// One RK4 stage of Eq. S5 is five launches:
+//   sp_apply  - one thread per operator and four columns of a row of the stage
+//               input Zs: W = A(t) Zs with A = -i H_eff, Y_k = L_k(t) Zs, and at
+//               stage 1 of every step Yr = r Zs; the ten channel factors
+//               Omega(t)^a e^{i q w_d t} of the stage times come from sp_chi, one
+//               small launch per CHI_STEPS steps;
 //   sp_gram   - per block, over row tiles of 16 (FP64) or 32 (FP32) rows held in
 //               shared memory, register sums of G = Zs^dag Zs (upper
 //               triangle), T_k = Zs^dag Y_k, and at stage 1 tr(Zs^dag Yr) =
 //               tr(rho r), plus level populations, |Yr|^2 and |Zs|^2 at
 //               recording steps;
-//   sp_solve  - one block per trajectory: reduce the partials in block order,
-//               record beta and the observables, Cholesky G = L L^dag and
-//               X_k = G^-1 T_k (the Moore-Penrose projection Zs^+ L_k Zs) by
-//               right-looking substitutions over all K M columns at once;
+//   sp_reduce - the partials added in a fixed order, the entries over the chip;
+//   sp_solve  - a few blocks per trajectory: record beta and the observables,
+//               G^-1 by symmetric sweeps and X_k = G^-1 T_k (the Moore-Penrose
+//               projection Zs^+ L_k Zs);
 //   sp_update - whole rows per block (Y_k rows staged in shared memory):
 //               F = W + 1/2 sum_k Y_k X_k^dag, then the classical RK4 stage.
 // After the last step an observation pass (apply r, Gram, solve without
@@ -26,14 +26,15 @@
 // lr_sparse_fused.cuh instead: one launch per integrate call, one CTA per
 // trajectory (or, for batches larger than the grid, an equal span of the
 // batch's trajectory-steps per CTA), all phases of a stage inside the CTA
-// (the four-launch path stays selectable with LR_SPARSE_FUSED=0 and is the
-// FP64 path).
+// (the launches above are the FP64 path, the FP32_G64 path of batches that are
+// far smaller than the GPU, see wide_is_faster, and selectable with
+// LR_SPARSE_FUSED=0).
 //
 // Precisions: FP64 throughout, or FP32_G64 - the state, the operator apply,
 // T_k, the projection term and the RK4 update in FP32, the Gram matrix
 // summed in double-word FP32 (~2^-48) from the exact products of FP32
-// entries (TwoProduct by one FMA), the M x M solves (FP64 here, double-word
-// in the fused kernel) and the signal in FP64.
+// entries (TwoProduct by one FMA), the M x M phase in double-word FP32, the
+// static diagonal of A and the step sizes as hi + lo floats, and the signal in FP64.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -42,6 +43,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lr_internal.cuh"
@@ -57,12 +59,15 @@ template <typename T2> __host__ __device__ constexpr int rows_per_block();
 template <> __host__ __device__ constexpr int rows_per_block<double2>() { return 16; }
 template <> __host__ __device__ constexpr int rows_per_block<float2>() { return 32; }
 constexpr int NCH = 10;     // time channels
+constexpr int CHI_STEPS = 8;   // RK4 steps whose channel factors are formed at once
 
 struct SpDev {
   const int* rowptr;
   const int* col;
   const double2* val;
   const float2* valf;   // FP32 copy of val
+  const float2* valf_a;   // FP32 state: valf with the static diagonal of A (operator 0) set to zero,
+  const float4* diag_a;   // and that diagonal per row as hi + lo floats (re_hi, im_hi, re_lo, im_lo)
   const unsigned char* chan;
   const int* level;
   const PulseDev* pulse;
@@ -70,7 +75,7 @@ struct SpDev {
   void *Z, *Zs, *acc, *W, *Y, *Yr;   // state-type arrays (double2 or float2)
   double2* X;
   float2* Xf;     // FP32 copy of X for the FP32 update
-  double2* chi;   // [T][4][NCH] channel factors at the four stage times of the current step
+  double2* chi;   // [T][CHI_STEPS][4][NCH] channel factors at the stage times
   double* part;
   double2* beta;
   double *pops, *nphot, *trace;
@@ -80,8 +85,6 @@ template <typename T2> struct Scalar;
 template <> struct Scalar<double2> { using type = double; };
 template <> struct Scalar<float2> { using type = float; };
 
-__device__ __forceinline__ double2 to_d(double2 v) { return v; }
-__device__ __forceinline__ double2 to_d(float2 v) { return make_double2(v.x, v.y); }
 template <typename T2> __device__ __forceinline__ T2 from_d(double2 v);
 template <> __device__ __forceinline__ double2 from_d<double2>(double2 v) { return v; }
 template <> __device__ __forceinline__ float2 from_d<float2>(double2 v) { return make_float2((float)v.x, (float)v.y); }
@@ -91,8 +94,8 @@ template <typename T2> __device__ __forceinline__ T2 mk2(typename Scalar<T2>::ty
   v.y = i;
   return v;
 }
-__device__ __forceinline__ const double2& op_val(const SpDev& d, int e, double2) { return d.val[e]; }
-__device__ __forceinline__ const float2& op_val(const SpDev& d, int e, float2) { return d.valf[e]; }
+__device__ __forceinline__ double2 op_val(const SpDev& d, int, int e, double2) { return d.val[e]; }
+__device__ __forceinline__ float2 op_val(const SpDev& d, int op, int e, float2) { return (op == 0 ? d.valf_a : d.valf)[e]; }
 
 struct SpParams {
   int N, M, K, T, n_levels, nblk;   // nblk: Gram blocks (partial sums) per trajectory
@@ -133,49 +136,69 @@ __device__ __forceinline__ void dw_acc(DWs& s, float a, float b) {
 }
 
 // Channel factors Omega(t)^a e^{i q w_d t} of one trajectory at the four RK4
-// stage times t, t + dt/2, t + dt/2, t + dt (one thread per factor).
-__global__ void __launch_bounds__(64) sp_chi(SpDev d, SpParams p, double t, double dt) {
+// stage times t, t + dt/2, t + dt/2, t + dt of CHI_STEPS steps (one thread per
+// factor: ~10 us of FP64 latency, whatever their number).
+__global__ void __launch_bounds__(64) sp_chi(SpDev d, SpParams p, long step, double dt) {
   const int tj = blockIdx.x, c = threadIdx.x;
   if (c >= 4 * NCH) return;
   const int stage = c / NCH, ch = c - stage * NCH;
-  const double ts = t + (stage == 0 ? 0.0 : stage == 3 ? dt : 0.5 * dt);
+  const double ts = (double)(step + blockIdx.y) * dt + (stage == 0 ? 0.0 : stage == 3 ? dt : 0.5 * dt);
   const int a = ch / 5, q = ch % 5 - 2;
   const double om = a ? pulse_envelope(d.pulse[tj], p.tau, ts) : 1.0;
   double sn, cs;
   sincos((double)q * p.wd * ts, &sn, &cs);
-  d.chi[(size_t)tj * 4 * NCH + c] = mk(om * cs, om * sn);
+  d.chi[((size_t)tj * CHI_STEPS + blockIdx.y) * 4 * NCH + c] = mk(om * cs, om * sn);
 }
 
-// out[e] = sum over the row's entries of chi[ch] val Zs[col][m]
+// Row n of operator blockIdx.z (the readout alone if only_r) times the columns m0 ..
+// m0 + 3 of Zs: every entry's weight chi val is formed once for the four (in FP64 it
+// costs as much as a column, and the FP64 pipe is the bound), and the operators of a
+// small batch go side by side. ci: stage time within the table of channel factors.
+constexpr int AT = 128;
 template <typename T2>
-__device__ __forceinline__ T2 row_apply(const SpDev& d, const SpParams& p, int op, int n, int m,
-                                        const T2* __restrict__ Zs, const T2* chi) {
-  const int* rp = d.rowptr + (size_t)op * (p.N + 1);
-  T2 acc = mk2<T2>(0, 0);
-  for (int e = rp[n]; e < rp[n + 1]; ++e) {
-    const T2 v = cmul(chi[d.chan[e]], op_val(d, e, T2()));
-    acc = cfma(v, Zs[(size_t)d.col[e] * p.M + m], acc);
-  }
-  return acc;
-}
-
-template <typename T2>
-__global__ void __launch_bounds__(SP_T) sp_apply(SpDev d, SpParams p, int stage, int with_r, int only_r) {
+__global__ void __launch_bounds__(AT) sp_apply(SpDev d, SpParams p, int ci, int only_r) {
   __shared__ T2 chi[NCH];
-  const int tj = blockIdx.y;
-  if (threadIdx.x < NCH) chi[threadIdx.x] = from_d<T2>(d.chi[((size_t)tj * 4 + stage) * NCH + threadIdx.x]);
+  const int tj = blockIdx.y, op = only_r ? p.K + 1 : blockIdx.z, M = p.M, mq = (M + 3) / 4;
+  if (threadIdx.x < NCH) chi[threadIdx.x] = from_d<T2>(d.chi[((size_t)tj * CHI_STEPS * 4 + ci) * NCH + threadIdx.x]);
   __syncthreads();
-  const long long e = (long long)blockIdx.x * SP_T + threadIdx.x;
-  if (e >= p.NM) return;
-  const int n = (int)(e / p.M), m = (int)(e - (long long)n * p.M);
+  const long long t = (long long)blockIdx.x * AT + threadIdx.x;
+  if (t >= (long long)p.N * mq) return;
+  const int n = (int)(t / mq), m0 = 4 * (int)(t - (long long)n * mq);
   const size_t off = (size_t)tj * p.NM;
-  const T2* Zs = static_cast<const T2*>(d.Zs) + off;
-  if (!only_r) {
-    static_cast<T2*>(d.W)[off + e] = row_apply(d, p, 0, n, m, Zs, chi);
-    for (int k = 0; k < p.K; ++k)
-      static_cast<T2*>(d.Y)[((size_t)k * p.T + tj) * p.NM + e] = row_apply(d, p, 1 + k, n, m, Zs, chi);
+  const T2* __restrict__ Zs = static_cast<const T2*>(d.Zs) + off;
+  int mc[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) mc[u] = min(m0 + u, M - 1);
+  const int* rp = d.rowptr + (size_t)op * (p.N + 1);
+  T2 acc[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) acc[u] = mk2<T2>(0, 0);
+  if constexpr (sizeof(T2) == sizeof(float2)) {
+    if (op == 0) {   // FP32 does not round the detunings
+      const float4 g = d.diag_a[n];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float2 z = Zs[(size_t)n * M + mc[u]];
+        acc[u].x = fmaf(g.x, z.x, fmaf(-g.y, z.y, fmaf(g.z, z.x, -g.w * z.y)));
+        acc[u].y = fmaf(g.x, z.y, fmaf(g.y, z.x, fmaf(g.z, z.y, g.w * z.x)));
+      }
+    }
   }
-  if (with_r) static_cast<T2*>(d.Yr)[off + e] = row_apply(d, p, 1 + p.K, n, m, Zs, chi);
+  const int e1 = rp[n + 1];
+#pragma unroll 4
+  for (int e = rp[n]; e < e1; ++e) {
+    const T2 w = cmul(chi[d.chan[e]], op_val(d, op, e, T2()));
+    const T2* z = Zs + (size_t)d.col[e] * M;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = cfma(w, z[mc[u]], acc[u]);
+  }
+  T2* out = op == 0 ? static_cast<T2*>(d.W) + off
+                    : (op <= p.K ? static_cast<T2*>(d.Y) + ((size_t)(op - 1) * p.T + tj) * p.NM
+                                 : static_cast<T2*>(d.Yr) + off);
+  out += (size_t)n * M;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (m0 + u < M) out[m0 + u] = acc[u];
 }
 
 // Register accumulator of one G or T_k entry: double-word FP32 (re.hi, re.lo,
@@ -209,7 +232,7 @@ template <> struct Acc<float2> {
 // Entries per thread of the (1 + K) M^2 partial sums: up to (1 + 3) 32^2 / 256.
 constexpr int ACC_MAX = (1 + LR_SPARSE_MAX_JUMPS) * LR_MAX_RANK * LR_MAX_RANK / SP_T;
 
-// NACC: accumulators per thread, >= (1 + K) M^2 / SP_T (4, 8 or ACC_MAX)
+// NACC: accumulators per thread, >= (M (M + 1) / 2 + K M^2) / SP_T (4, 8 or ACC_MAX)
 template <typename T2, int NACC>
 __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
   using T = typename Scalar<T2>::type;
@@ -225,7 +248,21 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
   const T2* Zs = static_cast<const T2*>(d.Zs);
   const T2* Yk = static_cast<const T2*>(d.Y);
   const T2* Yr = static_cast<const T2*>(d.Yr);
-  const int n_ent = (1 + K) * MM;
+  const int n_ent = (1 + K) * MM, ne = M * (M + 1) / 2;
+  // entry number e of this thread -> matrix, row, column, without the lower triangle
+  // of G (idle lanes cost an FP64 instruction as much as active ones)
+  auto entry = [&](int e, int& mat, int& i, int& j) {
+    if (e < ne) {
+      mat = 0;
+      tri_entry(e, i, j);
+    } else {
+      mat = 1 + (e - ne) / MM;
+      const int ij = e - ne - (mat - 1) * MM;
+      i = ij / M;
+      j = ij - i * M;
+    }
+  };
+  const int n_act = ne + K * MM;
   Acc<T2> acc[NACC];
 #pragma unroll
   for (int q = 0; q < NACC; ++q) acc[q].zero();
@@ -255,11 +292,11 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
 #pragma unroll
       for (int q = 0; q < NACC; ++q) {
         const int e = tid + q * SP_T;
-        if (e < n_ent) {
-          const int mat = e / MM, ij = e - mat * MM, i = ij / M, j = ij - (ij / M) * M;
+        if (e < n_act) {
+          int mat, i, j;
+          entry(e, mat, i, j);
           if (mat == 0) {
-            if (i <= j)
-              for (int r = 0; r < rows; ++r) acc[q].add_g(sZ[r][i], sZ[r][j]);
+            for (int r = 0; r < rows; ++r) acc[q].add_g(sZ[r][i], sZ[r][j]);
           } else {
             for (int r = 0; r < rows; ++r) acc[q].add_t(sZ[r][i], sY[mat - 1][r][j]);
           }
@@ -305,10 +342,13 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
 #pragma unroll
     for (int q = 0; q < NACC; ++q) {
       const int e = tid + q * SP_T;
-      if (e < n_ent) {
-        const double2 v = e < MM ? acc[q].g() : acc[q].t();
-        out[2 * e] = v.x;
-        out[2 * e + 1] = v.y;
+      if (e < n_act) {
+        int mat, i, j;
+        entry(e, mat, i, j);
+        const double2 v = mat == 0 ? acc[q].g() : acc[q].t();
+        const int o = 2 * (mat * MM + i * M + j);
+        out[o] = v.x;
+        out[o + 1] = v.y;
       }
     }
   }
@@ -320,111 +360,83 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
   }
 }
 
-// Dynamic shared memory: L [M][M+1] then B [K M][M+1] (column c of the right-hand
-// sides T_k, c = k M + j, stored as row B[c]), complex128.
-__global__ void __launch_bounds__(SP_T) sp_solve(SpDev d, SpParams p, long step, int mode) {
-  extern __shared__ double2 smem[];
-  __shared__ int bad;
-  const int tj = blockIdx.x, M = p.M, K = p.K, MM = M * M, tid = threadIdx.x, ld = M + 1;
-  double2* L = smem;
-  double2* B = smem + (size_t)M * ld;
+// Doubles [lo, hi) of every trajectory's partial blocks, added into block 0's: warp w
+// of a block adds blocks w, w + 8, ... of 32 doubles, then the eight warps in order.
+__global__ void __launch_bounds__(SP_T) sp_reduce(SpDev d, SpParams p, int lo, int hi) {
+  __shared__ double sh[SP_T / 32][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = lo + blockIdx.x * 32 + lane;
+  double* P = d.part + (size_t)blockIdx.y * p.nblk * p.ps + o;
+  double s = 0.0;
+  if (o < hi)
+    for (int k0 = warp; k0 < p.nblk; k0 += 64) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = k0 + 8 * u < p.nblk ? P[(size_t)(k0 + 8 * u) * p.ps] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+  sh[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && o < hi) {
+    for (int w = 1; w < SP_T / 32; ++w) s += sh[w][lane];
+    P[0] = s;
+  }
+}
+
+// From the sums in the trajectory's first block: the records, G^-1 and X_k = G^-1 T_k.
+// Every block of a trajectory forms G^-1 (bound by latency) and its share of X_k (see
+// plain_solve, the same phase of the bare-mode engine).
+template <typename A>
+__global__ void __launch_bounds__(ST) sp_solve(SpDev d, SpParams p, long step, int mode) {
+  __shared__ typename A::C Gs[LR_MAX_RANK * (LR_MAX_RANK + 1)];
+  __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
+  __shared__ MmShared<A> mm;
+  __shared__ XColumns<A> xc;
+  const int tj = blockIdx.y, g = blockIdx.x, M = p.M, K = p.K, MM = M * M, tid = threadIdx.x, ldg = M | 1;
   const double* P = d.part + (size_t)tj * p.nblk * p.ps;
-  const size_t o2 = (size_t)2 * (1 + K) * MM;
-  if (tid == 0) bad = 0;
-  if (mode & (MODE_BETA | MODE_OBS)) {
-    const int nv = 4 + p.n_levels;
-    for (int v = tid; v < nv; v += SP_T) {
-      double s = 0.0;
-      for (int b = 0; b < p.nblk; ++b) s += P[b * p.ps + o2 + v];
-      if (v < 2) {
-        if (mode & MODE_BETA) {
-          double* bt = reinterpret_cast<double*>(d.beta + (size_t)tj * (p.max_steps + 1) + step);
-          bt[v] = s;
-          if (!isfinite(s)) set_error(d.err, DEV_NONFINITE);
-        }
-      } else if (mode & MODE_OBS) {
-        const long rec = step / p.pop_every;
-        if (v == 2) d.nphot[(size_t)tj * p.n_rec + rec] = s;
-        else if (v == 3) d.trace[(size_t)tj * p.n_rec + rec] = s;
-        else d.pops[((size_t)tj * p.n_rec + rec) * p.n_levels + (v - 4)] = s;
+  const double2* P2 = reinterpret_cast<const double2*>(P);
+  if (g == 0 && (mode & (MODE_BETA | MODE_OBS)) && tid < 4 + p.n_levels) {
+    const int v = tid;
+    const double s = P[(size_t)2 * (1 + K) * MM + v];
+    if (v < 2) {
+      if (mode & MODE_BETA) {
+        double* bt = reinterpret_cast<double*>(d.beta + (size_t)tj * (p.max_steps + 1) + step);
+        bt[v] = s;
+        if (!isfinite(s)) set_error(d.err, DEV_NONFINITE);
       }
+    } else if (mode & MODE_OBS) {
+      const long rec = step / p.pop_every;
+      if (v == 2) d.nphot[(size_t)tj * p.n_rec + rec] = s;
+      else if (v == 3) d.trace[(size_t)tj * p.n_rec + rec] = s;
+      else d.pops[((size_t)tj * p.n_rec + rec) * p.n_levels + (v - 4)] = s;
     }
   }
   if (!(mode & MODE_SOLVE)) return;
-  for (int e = tid; e < (1 + K) * MM; e += SP_T) {   // block partials in block order
-    const int mat = e / MM, ij = e - mat * MM, i = ij / M, j = ij - (ij / M) * M;
-    if (mat == 0 && i > j) continue;
-    double re = 0.0, im = 0.0;
-    for (int b = 0; b < p.nblk; ++b) {
-      re += P[b * p.ps + 2 * e];
-      im += P[b * p.ps + 2 * e + 1];
-    }
-    if (mat == 0) L[j * ld + i] = i == j ? mk(re, 0.0) : mk(re, -im);   // lower: G_ji = conj(G_ij)
-    else B[((mat - 1) * M + j) * ld + i] = mk(re, im);                   // T_k (i, j)
+  const int per = (K * M + gridDim.x - 1) / gridDim.x, c_lo = g * per, c_hi = min(K * M, c_lo + per);
+  xc.load(P2 + MM, M, c_lo, min(XC, c_hi - c_lo), tid);
+  if (tid == 0) mm.bad = 0;
+  if (tid < M * (M + 1) / 2) {
+    int i, j;
+    tri_entry(tid, i, j);
+    tri[tid] = make_short2((short)j, (short)i);
   }
   __syncthreads();
-  // right-looking Cholesky G = L L^dag on the lower triangle
-  for (int k = 0; k < M; ++k) {
-    if (tid == 0) {
-      const double piv = L[k * ld + k].x;
-      if (!(piv > 0.0) || !isfinite(piv)) {
-        bad = 1;
-        L[k * ld + k] = mk(1.0, 0.0);
-      } else {
-        L[k * ld + k] = mk(sqrt(piv), 0.0);
-      }
+  if (tid / 32 < mm_warps(M, ST / 32)) {
+    typename A::C e[2] = {A::zero(), A::zero()};   // the sums hold the upper triangle
+    if (tid < M * (M + 1) / 2) {
+      const int i = tri[tid].x, j = tri[tid].y;
+      const double2 v = P2[j * M + i];
+      to_entry(mk(v.x, i == j ? 0.0 : -v.y), e[0]);
     }
-    __syncthreads();
-    const double inv = 1.0 / L[k * ld + k].x;
-    for (int i = k + 1 + tid; i < M; i += SP_T) L[i * ld + k] = mk(L[i * ld + k].x * inv, L[i * ld + k].y * inv);
-    __syncthreads();
-    const int rem = M - k - 1;
-    for (int e = tid; e < rem * rem; e += SP_T) {
-      const int i = k + 1 + e / rem, j = k + 1 + e % rem;
-      if (j > i) continue;
-      const double2 a = L[i * ld + k], c = L[j * ld + k];   // L_ij -= L_ik conj(L_jk)
-      L[i * ld + j] = mk(L[i * ld + j].x - (a.x * c.x + a.y * c.y), L[i * ld + j].y - (a.y * c.x - a.x * c.y));
-    }
-    __syncthreads();
+    mm_invert<A, ST>(e, Gs, ldg, mm, tri, M, tid);
   }
-  if (bad) {
-    if (tid == 0) set_error(d.err, DEV_NOT_PD);
-    return;
-  }
-  const int nc = K * M;
-  // forward L y = t, right-looking: y_j = t_j / L_jj, then t_i -= L_ij y_j (i > j), all columns at once
-  for (int j = 0; j < M; ++j) {
-    const double dinv = 1.0 / L[j * ld + j].x;
-    for (int c = tid; c < nc; c += SP_T) B[c * ld + j] = mk(B[c * ld + j].x * dinv, B[c * ld + j].y * dinv);
-    __syncthreads();
-    const int rem = M - j - 1;
-    for (int e = tid; e < nc * rem; e += SP_T) {
-      const int c = e / rem, i = j + 1 + e % rem;
-      const double2 l = L[i * ld + j], y = B[c * ld + j];
-      B[c * ld + i] = mk(B[c * ld + i].x - (l.x * y.x - l.y * y.y), B[c * ld + i].y - (l.x * y.y + l.y * y.x));
-    }
-    __syncthreads();
-  }
-  // back L^dag x = y: x_j = y_j / L_jj, then y_i -= conj(L_ji) x_j (i < j)
-  for (int j = M - 1; j >= 0; --j) {
-    const double dinv = 1.0 / L[j * ld + j].x;
-    for (int c = tid; c < nc; c += SP_T) B[c * ld + j] = mk(B[c * ld + j].x * dinv, B[c * ld + j].y * dinv);
-    __syncthreads();
-    for (int e = tid; e < nc * j; e += SP_T) {
-      const int c = e / j, i = e % j;
-      const double2 l = L[j * ld + i], x = B[c * ld + j];
-      B[c * ld + i] = mk(B[c * ld + i].x - (l.x * x.x + l.y * x.y), B[c * ld + i].y - (l.x * x.y - l.y * x.x));
-    }
-    __syncthreads();
-  }
-  double2* X = d.X + (size_t)tj * K * MM;
-  float2* Xf = d.Xf + (size_t)tj * K * MM;
-  for (int e = tid; e < K * MM; e += SP_T) {   // X[k][i][j] = (X_k)_ij = B[(k M + j)][i]
-    const int k = e / MM, ij = e - k * MM, i = ij / M, j = ij - (ij / M) * M;
-    const double2 v = B[(k * M + j) * ld + i];
-    X[e] = v;
-    Xf[e] = make_float2((float)v.x, (float)v.y);
-  }
+  __syncthreads();
+  if (g == 0 && tid == 0 && mm.bad) set_error(d.err, DEV_NOT_PD);
+  x_columns<A>(xc, Gs, ldg, P2 + MM, M, c_lo, c_hi, tid, [&](int k, int i, int j, double2 v) {
+    const size_t o = ((size_t)tj * K + k) * MM + i * M + j;
+    d.X[o] = v;
+    d.Xf[o] = make_float2((float)v.x, (float)v.y);
+  });
 }
 
 __device__ __forceinline__ double2 load_x(const SpDev& d, size_t i, double2) { return d.X[i]; }
@@ -452,35 +464,39 @@ __global__ void __launch_bounds__(SP_T) sp_update(SpDev d, SpParams p, int stage
   const int rbase = (e / M) * M;   // this row's first element in sY
   for (int k = 0; k < p.K; ++k) {
     __syncthreads();
-    for (int i = threadIdx.x; i < MM; i += SP_T) sX[i] = load_x(d, ((size_t)tj * p.K + k) * MM + i, T2());
+    for (int i = threadIdx.x; i < MM; i += SP_T)   // transposed: no bank conflicts along m
+      sX[(i % M) * M + i / M] = load_x(d, ((size_t)tj * p.K + k) * MM + i, T2());
     if (live) sY[e] = Yk[((size_t)k * p.T + tj) * p.NM + idx];
     __syncthreads();
     if (live) {   // F += 1/2 sum_j Y_k[n][j] conj(X_k[m][j])
       T2 s = mk2<T2>(0, 0);
       for (int jj = 0; jj < M; ++jj) {
-        const T2 a = sY[rbase + jj], x = sX[m * M + jj];
+        const T2 a = sY[rbase + jj], x = sX[jj * M + m];
         s = mk2<T2>(fma(a.x, x.x, fma(a.y, x.y, s.x)), fma(a.y, x.x, fma(-a.x, x.y, s.y)));
       }
       F = mk2<T2>(fma(half, s.x, F.x), fma(half, s.y, F.y));
     }
   }
   if (!live) return;
-  const T dt = (T)dt_;
+  // step sizes as hi + lo (FP32 state; lo = 0 in FP64)
+  const double hd = stage == 3 ? dt_ / 6.0 : (stage == 2 ? dt_ : 0.5 * dt_);
+  const T c = (T)hd, cl = (T)(hd - (double)c);
   const T w = (stage == 0 || stage == 3) ? (T)1 : (T)2;
   const T2 a0 = stage == 0 ? mk2<T2>(0, 0) : acc[off + idx];
   const T2 a = mk2<T2>(fma(w, F.x, a0.x), fma(w, F.y, a0.y));
-  const T2 z = Z[off + idx];
+  const T2 z = Z[off + idx], s = stage < 3 ? F : a;
+  T2 zn;
+  if constexpr (sizeof(T) == 4)
+    zn = mk2<T2>(z.x + fma(cl, s.x, c * s.x), z.y + fma(cl, s.y, c * s.y));
+  else
+    zn = mk2<T2>(fma(c, s.x, z.x), fma(c, s.y, z.y));
   if (stage < 3) {
-    const T c = stage == 2 ? dt : (T)0.5 * dt;
     acc[off + idx] = a;
-    Zs[off + idx] = mk2<T2>(fma(c, F.x, z.x), fma(c, F.y, z.y));
   } else {
-    const T c = dt / (T)6;
-    const T2 zn = mk2<T2>(fma(c, a.x, z.x), fma(c, a.y, z.y));
     if (!isfinite(zn.x) || !isfinite(zn.y)) set_error(d.err, DEV_NONFINITE);
     Z[off + idx] = zn;
-    Zs[off + idx] = zn;
   }
+  Zs[off + idx] = zn;
 }
 
 // Sec. S3.A / S3.B for candidate c = trajectories (2c, 2c+1) = (g, e), over the
@@ -543,6 +559,7 @@ struct lr_sparse {
   int fp32;   // 1: FP32_G64 state arithmetic
   int fused;  // 1: the fused persistent kernel (FP32_G64), 0: four launches per RK4 stage
   int gram_tc;   // fused: 1 when the Gram matrix is formed on the tensor cores (rank padded to 20)
+  int wide;    // fused: 1 when the whole-chip launches are faster than the teams
   int n_cta;   // fused: persistent CTAs (n_team teams of team_c)
   int n_team, team_c;   // fused: teams (one trajectory at a time each), CTAs per team
   size_t o_fsc;   // fused: per-CTA stage buffers
@@ -576,6 +593,9 @@ lr_status cuda_fail(lr_sparse* s, cudaError_t e) {
   return LR_ERR_CUDA;
 }
 
+// Doubles per partial block, even (sp_solve reads the sums as complex numbers)
+size_t part_stride(const lr_sparse* s) { return ((size_t)2 * (1 + s->K) * s->M * s->M + 4 + s->n_levels + 1) / 2 * 2; }
+
 void layout(lr_sparse* s) {
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -601,20 +621,22 @@ void layout(lr_sparse* s) {
   s->o_Y = take(state * s->K);
   s->o_Yr = take(state);
   s->o_X = take((size_t)s->T * s->K * s->M * s->M * sizeof(double2));
-  s->o_chi = take((size_t)s->T * 4 * NCH * sizeof(double2));
+  s->o_chi = take((size_t)s->T * CHI_STEPS * 4 * NCH * sizeof(double2));
   s->o_Xf = take((size_t)s->T * s->K * s->M * s->M * sizeof(float2));
   s->o_loss = take((size_t)(s->T / 2 + 1) * 3 * sizeof(double));
-  const size_t ps = (size_t)2 * (1 + s->K) * s->M * s->M + 4 + s->n_levels;
+  const size_t ps = part_stride(s);
   s->o_part = take((size_t)s->T * s->nblk * ps * sizeof(double));
   s->o_beta = take((size_t)s->T * (s->max_steps + 1) * sizeof(double2));
   s->o_pops = take((size_t)s->T * s->n_rec * s->n_levels * sizeof(double));
   s->o_nphot = take((size_t)s->T * s->n_rec * sizeof(double));
   s->o_trace = take((size_t)s->T * s->n_rec * sizeof(double));
+  if (s->fp32) {
+    s->o_fvala = take((size_t)s->nnz * sizeof(float2));
+    s->o_fdiag = take((size_t)s->N * sizeof(float4));
+  }
   if (s->fused) {
     const size_t Mp = (size_t)(s->M + 3) / 4 * 4;
     s->o_fsc = take((size_t)s->n_team * (3 + s->K) * s->N * Mp * sizeof(float2));
-    s->o_fvala = take((size_t)s->nnz * sizeof(float2));
-    s->o_fdiag = take((size_t)s->N * sizeof(float4));
     s->o_fflag = take((size_t)s->T * sizeof(int));
   }
   s->total = o;
@@ -712,6 +734,22 @@ void fused_teams(lr_sparse* s, int sms) {
   s->n_cta = s->n_team;
 }
 
+// The whole-chip launches against the fused teams (at most 16 CTAs per trajectory, and
+// a wave of teams more where the clusters do not all fit). Estimates in us per stage,
+// fitted on GB300 to 1 to 20 pulses of six models (M = 4 .. 32, N = 120 .. 3600):
+//   teams: 2.05 M + 2 + rows per CTA x M (M + 11) x 2.2e-4, for every wave of teams;
+//   wide:  26 + 0.75 M + 4.3e-6 x T N M (M + 11).
+// Measured, teams / wide: N = 2000, M = 20, 1 pulse 57 / 48, 2 pulses 57 / 56, 4 pulses
+// 114 / 74, 8 pulses 153 / 110, 20 pulses 168 / 224; N = 3600, M = 32 174 / 96; N = 120,
+// M = 4 16 / 29. The line lies at 0.9: no measured batch above it was slower wide.
+bool wide_is_faster(const lr_sparse* s, int sms) {
+  if (s->T >= sms) return false;   // one CTA per trajectory fills the chip
+  const double w = s->M * (s->M + 11.0);
+  const int waves = (s->T + s->n_team - 1) / s->n_team;
+  const double team = waves * (2.05 * s->M + 2.0 + 2.2e-4 * w * ((s->N + s->team_c - 1) / s->team_c));
+  return 26.0 + 0.75 * s->M + 4.3e-6 * s->T * s->N * w < 0.9 * team;
+}
+
 SpDev dev(const lr_sparse* s) {
   char* w = s->ws;
   SpDev d;
@@ -719,6 +757,8 @@ SpDev dev(const lr_sparse* s) {
   d.col = reinterpret_cast<const int*>(w + s->o_col);
   d.val = reinterpret_cast<const double2*>(w + s->o_val);
   d.valf = reinterpret_cast<const float2*>(w + s->o_valf);
+  d.valf_a = reinterpret_cast<const float2*>(w + s->o_fvala);
+  d.diag_a = reinterpret_cast<const float4*>(w + s->o_fdiag);
   d.chan = reinterpret_cast<const unsigned char*>(w + s->o_chan);
   d.level = reinterpret_cast<const int*>(w + s->o_level);
   d.pulse = reinterpret_cast<const PulseDev*>(w + s->o_pulse);
@@ -744,27 +784,10 @@ size_t state_bytes(const lr_sparse* s) {
   return (size_t)s->T * s->N * s->M * (s->fp32 ? sizeof(float2) : sizeof(double2));
 }
 
-size_t solve_smem(const lr_sparse* s) { return (size_t)(1 + s->K) * s->M * (s->M + 1) * sizeof(double2); }
-
-// The dynamic shared-memory limit of sp_solve is a property of the function in
-// the current device's context, not of a lr_sparse context: it only ever grows,
-// so that a context bound later with a smaller rank does not lower it under one
-// bound earlier. The current limit is read from the device each time (it is
-// per device, and a device reset restores the default).
-cudaError_t raise_solve_smem(int bytes) {
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, sp_solve);
-  if (e != cudaSuccess) return e;
-  if (fa.maxDynamicSharedSizeBytes >= bytes) return cudaSuccess;
-  return cudaFuncSetAttribute(sp_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
 template <typename T2>
 void launch_gram(const lr_sparse* s, const SpDev& d, const SpParams& p, int mode, cudaStream_t st) {
   const dim3 gg((unsigned)s->nblk, (unsigned)s->T);
-  const int per = ((1 + s->K) * s->M * s->M + SP_T - 1) / SP_T;
+  const int per = (s->M * (s->M + 1) / 2 + s->K * s->M * s->M + SP_T - 1) / SP_T;
   if (per <= 4)
     sp_gram<T2, 4><<<gg, SP_T, 0, st>>>(d, p, mode);
   else if (per <= 8)
@@ -776,26 +799,33 @@ void launch_gram(const lr_sparse* s, const SpDev& d, const SpParams& p, int mode
 template <typename T2>
 void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, long step0, long n_steps, double dt,
                          cudaStream_t st) {
-  const dim3 ge((unsigned)((p.NM + SP_T - 1) / SP_T), (unsigned)s->T);
+  using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, WidePivot>::type;
+  const unsigned ab = (unsigned)(((long long)s->N * ((s->M + 3) / 4) + AT - 1) / AT);
   const int rb = SP_T / s->M;
   const dim3 gu((unsigned)((s->N + rb - 1) / rb), (unsigned)s->T);
+  const int n2 = 2 * (1 + s->K) * s->M * s->M, no = n2 + 4 + s->n_levels;
+  // a trajectory's share of two blocks per SM, at most eight
+  const unsigned sb = (unsigned)std::max(1, std::min(8, 304 / s->T));
+  auto reduce = [&](int lo, int hi) { sp_reduce<<<dim3((hi - lo + 31) / 32, s->T), SP_T, 0, st>>>(d, p, lo, hi); };
   for (long i = 0; i <= n_steps; ++i) {
     const long step = step0 + i;
-    const double t = (double)step * dt;
     const bool rec = step % s->pop_every == 0;
-    sp_chi<<<s->T, 64, 0, st>>>(d, p, t, dt);
+    const int c4 = 4 * (int)(i % CHI_STEPS);
+    if (c4 == 0) sp_chi<<<dim3(s->T, CHI_STEPS), 64, 0, st>>>(d, p, step, dt);
     if (i == n_steps) {   // observation of the final state
       const int mode = MODE_BETA | (rec ? MODE_OBS : 0);
-      sp_apply<T2><<<ge, SP_T, 0, st>>>(d, p, 0, 1, 1);
+      sp_apply<T2><<<dim3(ab, s->T), AT, 0, st>>>(d, p, c4, 1);
       launch_gram<T2>(s, d, p, mode, st);
-      sp_solve<<<s->T, SP_T, solve_smem(s), st>>>(d, p, step, mode);
+      reduce(n2, no);
+      sp_solve<A><<<dim3(1, s->T), ST, 0, st>>>(d, p, step, mode);
       break;
     }
     for (int stg = 0; stg < 4; ++stg) {
       const int mode = MODE_SOLVE | (stg == 0 ? MODE_BETA | (rec ? MODE_OBS : 0) : 0);
-      sp_apply<T2><<<ge, SP_T, 0, st>>>(d, p, stg, stg == 0, 0);
+      sp_apply<T2><<<dim3(ab, s->T, s->K + (stg == 0 ? 2 : 1)), AT, 0, st>>>(d, p, c4 + stg, 0);
       launch_gram<T2>(s, d, p, mode, st);
-      sp_solve<<<s->T, SP_T, solve_smem(s), st>>>(d, p, step, mode);
+      reduce(0, stg == 0 ? no : n2);
+      sp_solve<A><<<dim3(sb, s->T), ST, 0, st>>>(d, p, step, mode);
       sp_update<T2><<<gu, SP_T, 0, st>>>(d, p, stg, dt);
     }
   }
@@ -811,7 +841,7 @@ SpParams params(const lr_sparse* s) {
   p.nblk = s->nblk;
   p.ntile = s->ntile;
   p.NM = (long long)s->N * s->M;
-  p.ps = (long long)2 * (1 + s->K) * s->M * s->M + 4 + s->n_levels;
+  p.ps = (long long)part_stride(s);
   p.wd = s->wd;
   p.tau = s->tau;
   p.max_steps = s->max_steps;
@@ -911,6 +941,7 @@ extern "C" lr_status lr_sparse_create(const lr_sparse_model* m, int n_traj, int 
   // one persistent CTA per SM (fewer when the batch is smaller)
   s->fused = 0;
   s->n_cta = s->n_team = s->team_c = 0;
+  s->wide = 0;
   s->gram_tc = 0;
   const char* fz_env = getenv("LR_SPARSE_FUSED");
   if (s->fp32 && !(fz_env && strcmp(fz_env, "0") == 0)) {
@@ -925,6 +956,9 @@ extern "C" lr_status lr_sparse_create(const lr_sparse_model* m, int n_traj, int 
       const char* gram_env = getenv("LR_SPARSE_GRAM");
       s->gram_tc = (s->M + 3) / 4 * 4 == 20 && gram_env && strcmp(gram_env, "tc") == 0;
       fused_teams(s, sms);
+      s->wide = !getenv("LR_SPARSE_FUSED") && !getenv("LR_SPARSE_C") && !getenv("LR_SPARSE_SPLIT") && !gram_env &&
+                wide_is_faster(s, sms);
+      if (const char* we = getenv("LR_SPARSE_WIDE")) s->wide = atoi(we) != 0;
     } else {
       cudaGetLastError();
     }
@@ -973,7 +1007,7 @@ extern "C" lr_status lr_sparse_bind_workspace(lr_sparse* s, void* workspace, siz
       return cuda_fail(s, e);
   std::vector<float2> vala;
   std::vector<float4> diag;
-  if (s->fused) {
+  if (s->fp32) {
     // A's static (channel a = 0, q = 0) diagonal entries leave the gathered values
     // and go, summed per row in FP64, into hi + lo floats
     vala = valf;
@@ -997,7 +1031,6 @@ extern "C" lr_status lr_sparse_bind_workspace(lr_sparse* s, void* workspace, siz
       return cuda_fail(s, e);
   }
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(s, e);
-  if ((e = raise_solve_smem((int)solve_smem(s))) != cudaSuccess) return cuda_fail(s, e);
   s->step = 0;
   return LR_OK;
 }
@@ -1079,7 +1112,7 @@ extern "C" lr_status lr_sparse_integrate(lr_sparse* s, double dt, long n_steps, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const SpDev d = dev(s);
   const SpParams p = params(s);
-  if (s->fused) {
+  if (s->fused && !s->wide) {
     const SfSmem L = sf_smem(s->M, s->K, s->gram_tc);
     cudaError_t e0 = raise_fused_smem(L.total);
     if (e0 != cudaSuccess) return cuda_fail(s, e0);
