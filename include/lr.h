@@ -43,7 +43,7 @@
  *
  * Errors: every call returns an lr_status; nothing crosses the ABI as an
  * exception. lr_last_error() gives a human-readable message for the last
- * failing call on a context. Device-side failures (Cholesky breakdown,
+ * failing call on a context. Device-side failures (a pivot of the Gram matrix lost,
  * non-finite values, a device wait that ran out) set an error word in the
  * workspace; lr_observables and lr_sync read it and return the status.
  *
@@ -88,7 +88,7 @@ typedef enum {
  * T_k = Z^dag L_k Z, the projection term and the RK4 stages in complex64.
  * The Gram matrix Z^dag Z is accumulated from exact FP32 products in a
  * double-word FP32 sum (hi + lo floats, about 2^-48 relative: FP64-class,
- * not IEEE FP64). Its LDL^dag factorisation, L^-1 and G^-1 run in the same
+ * not IEEE FP64). Its inverse G^-1 (symmetric sweeps) runs in the same
  * double-word FP32 arithmetic (Dekker products, Knuth sums, a Newton
  * reciprocal; about 2^-48 relative), and so is X_k = G^-1 T_k (from the FP32
  * T_k), which is rounded to FP32 once. The readout signal beta, the populations,
@@ -332,9 +332,10 @@ lr_status lr_sync(lr_ctx* ctx, void* stream);
  * FP32-bulk context (FP32_G64, FP32, TF32_G64): the checkpoints, stage
  * inputs, cotangents and every per-element product in complex64 / FP32; the
  * Gram matrix summed from exact FP32 products in double-word FP32 (~2^-48,
- * FP64-class); the Cholesky factor, G^-1 and the M x M adjoint factors in
+ * FP64-class); G^-1 and the M x M adjoint factors in
  * FP64; the readout signal and the gradient sums in FP64. The checkpoint
- * segments are recomputed with the PLAIN engine's kernels in that arithmetic
+ * segments are recomputed with the PLAIN engine's kernels in that arithmetic,
+ * and a segment's stage inputs and factors are kept up to 8 GB of workspace
  * (the copies in the workspace are complex64 then: half the memory).
  * Synchronous; returns the device error status. */
 lr_status lr_backward_workspace_size(const lr_ctx* ctx, int ckpt_every, size_t* bytes);
@@ -497,14 +498,14 @@ lr_status lr_paper_model_build(const lr_paper_params* p, int* rowptr, int* col, 
  * pulses[i]. Copies the operator arrays (they may be freed afterwards).
  * tau places the falling pulse edge; max_steps and pop_every size the
  * recorded observables as for lr_options. Per RK4 stage: an apply kernel
- * (A Z, L_k Z, r Z from the CSR rows, one thread per element of Z), a
+ * (A Z, L_k Z, r Z from the CSR rows, one thread per four columns), a
  * row-block Gram kernel (Z^dag Z, Z^dag L_k Z and the observables), a
- * per-trajectory solve (Cholesky, X_k = G^-1 Z^dag L_k Z) and an update
+ * solve (G^-1 by symmetric sweeps, X_k = G^-1 Z^dag L_k Z) and an update
  * kernel (F = A Z + 1/2 sum_k (L_k Z) X_k^dag, RK4).
  * precision: LR_PREC_FP64 (complex128 throughout) or LR_PREC_FP32_G64 (state,
  * apply, Z^dag L_k Z, projection term and RK4 in complex64; the Gram matrix
- * accumulated in FP64 from the exact products of the FP32 entries; Cholesky,
- * solves and observables in FP64); others give LR_ERR_UNSUPPORTED. */
+ * accumulated in double-word FP32 from the exact products of the FP32 entries; G^-1,
+ * X_k and observables in FP64, or in the fused kernel's arithmetic); others give LR_ERR_UNSUPPORTED. */
 lr_status lr_sparse_create(const lr_sparse_model* model, int n_traj, int M, lr_precision precision,
                            const lr_pulse* pulses, double tau, long max_steps, int pop_every, lr_sparse** out);
 /* Bytes of device workspace the context needs (256-byte aligned). */
@@ -547,8 +548,9 @@ lr_status lr_sparse_loss(lr_sparse* s, double eta, double kappa, double gamma, d
  * persistent kernel (FP32_G64 contexts by default: one launch per
  * lr_sparse_integrate; the stage input, the operator images and the RK4
  * accumulator in a per-team L2-resident region; the Gram matrix in
- * double-word FP32 and its LDL^dag factorisation, L^-1 and G^-1 in
- * double-word FP32), 0 for the four launches per RK4 stage described at
+ * double-word FP32 and its inverse in double-word FP32; batches far smaller
+ * than the GPU run the launches of lr_sparse_create in the same arithmetic
+ * where that is faster, LR_SPARSE_WIDE = 0 / 1 forces either), 0 for the four launches per RK4 stage described at
  * lr_sparse_create (FP64 contexts, or FP32_G64 with the environment variable
  * LR_SPARSE_FUSED=0 at lr_sparse_create). *team (may be NULL) = the CTAs
  * (one thread-block cluster) that share each trajectory's rows: 1 when the

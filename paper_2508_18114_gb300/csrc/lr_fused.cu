@@ -104,29 +104,62 @@ int rows_per_cta(const TrajDev& d, int C) {
   return d.Nt * ((d.Nr + C - 1) / C) * d.Nf;
 }
 
+// Trajectories of costs t on n teams, in rows of n: the largest first, and in every row
+// the largest to the team with the least so far. Returns the largest team's sum; order
+// (unless null) lists them as the kernel takes them, team c = entries c, c + n, ...
+double assign_teams(const std::vector<double>& t, int n, std::vector<int>* order) {
+  const int T = (int)t.size();
+  std::vector<int> by(T), team(n);
+  for (int j = 0; j < T; ++j) by[j] = j;
+  std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return t[a] > t[b]; });
+  std::vector<double> load(n, 0.0);
+  std::vector<std::vector<int>> list(n);
+  for (int r = 0; r < T; r += n) {
+    for (int c = 0; c < n; ++c) team[c] = c;
+    std::stable_sort(team.begin(), team.end(), [&](int a, int b) { return load[a] < load[b]; });
+    for (int c = 0; c < std::min(n, T - r); ++c) {
+      load[team[c]] += t[by[r + c]];
+      list[team[c]].push_back(by[r + c]);
+    }
+  }
+  if (order) {   // the teams with an entry in the last, partial row first
+    std::stable_sort(list.begin(), list.end(),
+                     [](const std::vector<int>& a, const std::vector<int>& b) { return a.size() > b.size(); });
+    order->clear();
+    for (size_t r = 0; r < list[0].size(); ++r)
+      for (int c = 0; c < n && r < list[c].size(); ++c) order->push_back(list[c][r]);
+  }
+  return *std::max_element(load.begin(), load.end());
+}
+
 // The wide schedule (four launches per RK4 stage, each over the whole chip) against the
 // teams: a team holds a trajectory on at most min(16, N_r) SMs, so a batch of one or
 // two candidates leaves most of the chip idle. Estimates in us per stage, fitted on
 // GB300 to 1 to 16 candidates of 13 models (M = 4 .. 32, N = 40 .. 9600):
 //   teams: 2.05 M (1.5 M on one CTA; the M x M phase and the barrier) + rows per CTA x
 //          M (M + 11) x 1.7e-4 (stage state in L2: 2.3e-4; two modes, shared memory: 1e-4),
-//          for every wave of teams;
+//          the sum over a team's trajectories;
 //   wide:  20 + 1.1 M (launches and the M x M phase) + 4.6e-6 x sum N M (M + 11).
+// FP64 state, bound by the FP64 pipe (18 M^2 + 47 M FMAs a row at 2.05 per clock and SM):
+//   teams: 3 M + rows per CTA x (M^2 + 2.6 M) x 4.5e-3, likewise;
+//   wide:  25 + 1.5 M + 4.5e-3 / 152 x sum N (M^2 + 2.6 M).
 // Measured, teams / wide: N = 2000, M = 20, 1 candidate 62 / 47, 2 candidates 62 / 61;
 // N = 480, M = 32 (two modes) 202 / 62, 8 candidates 203 / 114; N = 8000, M = 32 269 /
 // 148; N = 2000, M = 10 32 / 35; N = 40, M = 4 10 / 28. The line lies at 0.9, where no
 // measured batch lost more than 1%.
 bool wide_is_faster(const std::vector<TrajDev>& traj, const FusedPlan& plan) {
-  double team = 0.0, wide = 0.0;
+  double wide = 0.0;
+  std::vector<double> team;
+  const bool fp64 = plan.es == (int)sizeof(double2);
   for (const TrajDev& d : traj) {
-    const double w = d.M * (d.M + 11.0);
-    const double slope = !plan.zs_smem ? 2.3e-4 : (d.n_modes == 2 ? 1.0e-4 : 1.7e-4);
-    team = std::max(team, (plan.C > 1 ? 2.05 : 1.5) * d.M + slope * w * rows_per_cta(d, plan.C));
-    wide = std::max(wide, 20.0 + 1.1 * d.M);
+    const double w = fp64 ? d.M * (d.M + 2.6) : d.M * (d.M + 11.0);
+    const double slope = fp64 ? 4.5e-3 : (!plan.zs_smem ? 2.3e-4 : (d.n_modes == 2 ? 1.0e-4 : 1.7e-4));
+    team.push_back((fp64 ? 3.0 : (plan.C > 1 ? 2.05 : 1.5)) * d.M + slope * w * rows_per_cta(d, plan.C));
+    wide = std::max(wide, fp64 ? 25.0 + 1.5 * d.M : 20.0 + 1.1 * d.M);
   }
-  for (const TrajDev& d : traj) wide += 4.6e-6 * d.N * d.M * (d.M + 11.0);
-  const int waves = ((int)traj.size() + plan.n_clusters - 1) / plan.n_clusters;
-  return wide < 0.9 * waves * team;
+  for (const TrajDev& d : traj)
+    wide += d.N * (fp64 ? 4.5e-3 / 152 * d.M * (d.M + 2.6) : 4.6e-6 * d.M * (d.M + 11.0));
+  return wide < 0.9 * assign_teams(team, plan.n_clusters, nullptr);
 }
 
 // Wide schedule: two stage buffers and the accumulator, X_k, partial sums, from `off`.
@@ -140,9 +173,9 @@ WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
     return at;
   };
   WideLayout L{};
-  L.za = take(sizeof(float2) * plan.tot);
-  L.zb = take(sizeof(float2) * plan.tot);
-  L.acc = take(sizeof(float2) * plan.tot);
+  L.za = take(plan.es * (size_t)plan.tot);
+  L.zb = take(plan.es * (size_t)plan.tot);
+  L.acc = take(plan.es * (size_t)plan.tot);
   L.x = take(sizeof(double2) * 2 * LR_MAX_RANK * LR_MAX_RANK * n_traj);
   L.part = take(sizeof(double) * plan.part);
   L.total = off;
@@ -177,7 +210,7 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
   }
   const int Mp = (Mmax + 3) / 4 * 4;
   // Variants (stage state placement, tensor-core passes of the projection).
-  // Overrides for tuning and tests: LR_FUSED_WIDE = 0 / 1 (teams / wide schedule, FP32_G64),
+  // Overrides for tuning and tests: LR_FUSED_WIDE = 0 / 1 (teams / wide schedule, FP32_G64 and FP64),
   // LR_FUSED_C = cluster size, LR_FUSED_ZS =
   // "global" keeps the stage state in L2, LR_FUSED_TC = 0 keeps the FP32_G64
   // projection on the CUDA cores (3: only the tensor-core variant).
@@ -247,11 +280,6 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
         cudaGetLastError();
         continue;
       }
-      const int n_traj = (int)traj.size();
-      // only as many teams as the waves need: the same number of waves, less
-      // scratch, and every team runs the same number of trajectories
-      const int waves_needed = (n_traj + ncl - 1) / ncl;
-      const int used = std::min((n_traj + waves_needed - 1) / waves_needed, n_traj);
       // Cost model, fitted to measurements on GB300 (N = 2000, M = 20 batch):
       // a stage costs ~0.16 us per row per CTA with the stage state in shared
       // memory (x1.3 in L2; x1.7 and x1.55 in L2 with the projection on the
@@ -261,16 +289,39 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
       // sequential elimination steps) that does not shrink with C; teams run
       // trajectories in waves.
       const double row_cost = zs_smem ? 1.0 : (tc == 3 ? 1.7 : tc == 1 ? 1.55 : gs ? 1.0 : 1.3);
-      const double waves = std::ceil((double)n_traj / used);
-      double t = 0.0;
+      std::vector<double> cost;
       for (const TrajDev& d : traj) {
         const double rows = (double)rows_per_cta(d, C) * row_cost * (d.M * d.M) / 400.0;
         const double fixed = 375.0 * d.M / 20.0 * (C > 1 ? 1.0 : 0.95);
-        t += rows + fixed;
+        cost.push_back(rows + fixed);
       }
-      t = waves * t / n_traj;
+      // Only as many teams as the waves need (the same number of waves, less scratch), or
+      // all that fit where an uneven batch gains by it. 256 trajectories of N = 1000 ..
+      // 4000, M = 10 .. 30: their mean cost times the waves chose single CTAs, whose
+      // largest pair took 1548 us a stage; the largest team's sum, and the assignment
+      // that keeps it small, take 935 us.
+      const int n_traj = (int)traj.size();
+      const int waves_needed = (n_traj + ncl - 1) / ncl;
+      int used = std::min((n_traj + waves_needed - 1) / waves_needed, n_traj);
+      const int all = std::min(ncl, n_traj);
+      double sum = 0.0, lo = cost[0], hi = cost[0];
+      for (double c : cost) {
+        sum += c;
+        lo = std::min(lo, c);
+        hi = std::max(hi, c);
+      }
+      if (std::max(hi, sum / all) >= best) continue;
+      double t = hi == lo ? waves_needed * hi : assign_teams(cost, used, nullptr);
+      if (all > used && hi > lo) {
+        const double ta = assign_teams(cost, all, nullptr);
+        if (ta < 0.99 * t) {
+          t = ta;
+          used = all;
+        }
+      }
       if (t < best) {
         best = t;
+        assign_teams(cost, used, &plan->order);
         plan->ok = 1;
         plan->C = C;
         plan->n_clusters = used;
@@ -293,15 +344,9 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
     plan->tot += (long long)d.N * d.M;
     plan->part += (long long)d.nblk * (long long)plain_pstride(d.M);
   }
-  plan->wide = prec == LR_PREC_FP32_G64 && !force_c && !force_global && force_tc < 0 && !gram_dw &&
-               wide_is_faster(traj, *plan);
-  if (const char* e = getenv("LR_FUSED_WIDE")) plan->wide = prec == LR_PREC_FP32_G64 && atoi(e);
-  // largest work first, round-robin over the teams
-  std::vector<std::pair<double, int>> w;
-  for (size_t j = 0; j < traj.size(); ++j)
-    w.push_back({-(double)traj[j].N * traj[j].M * (traj[j].M + 11.0), (int)j});
-  std::stable_sort(w.begin(), w.end());
-  for (auto& x : w) plan->order.push_back(x.second);
+  const bool has_wide = prec == LR_PREC_FP32_G64 || prec == LR_PREC_FP64;
+  plan->wide = has_wide && !force_c && !force_global && force_tc < 0 && !gram_dw && wide_is_faster(traj, *plan);
+  if (const char* e = getenv("LR_FUSED_WIDE")) plan->wide = has_wide && atoi(e);
   return true;
 }
 
@@ -339,7 +384,7 @@ cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunPa
     q.acc = sc + L.acc;
     q.X = reinterpret_cast<double2*>(sc + L.x);
     q.part = reinterpret_cast<double*>(sc + L.part);
-    return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, s);
+    return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, prec != LR_PREC_FP64, s);
   }
   const size_t es = prec == LR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const SmemLayout L = layout(plan.R, plan.Mp, plan.zs_smem, es, plan.tc, plan.gram_mode == 2);

@@ -33,7 +33,7 @@ struct FusedPlan {
   int wide;        // 1: the wide schedule (a few launches per stage over the whole chip) in place of the teams
   int max_nblk;    // its row blocks, state elements and partial sums (doubles)
   long long tot, part;
-  std::vector<int> order;   // trajectories, largest work first
+  std::vector<int> order;   // trajectories by team: c, c + n_clusters, ... for team c
 };
 
 // Decide whether the fused engine supports this batch and with which shape.

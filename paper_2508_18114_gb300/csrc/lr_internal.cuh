@@ -261,9 +261,10 @@ size_t plain_partial_doubles(int M);
 // The plain engine: complex128 state, the reference GPU path.
 cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0,
                             long n_steps, cudaStream_t s);
-// Its kernels on complex64 state as the wide schedule of the fused engine: n_steps from
-// the device's step counter p.dstep; p.Za, p.Zb, p.acc, p.X and p.part in its scratch.
-cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s);
+// Its kernels as the wide schedule of the fused engine: n_steps from the device's step
+// counter p.dstep; p.Za, p.Zb, p.acc, p.X and p.part in its scratch.
+cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, int fp32,
+                           cudaStream_t s);
 // single kernels of the plain engine (used by the adjoint's recomputation)
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s);
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s);

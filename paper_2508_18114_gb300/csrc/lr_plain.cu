@@ -22,6 +22,7 @@
 // that FP32 does not round the mode frequencies or dt).
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "lr_mm.cuh"
 
@@ -219,9 +220,10 @@ __device__ __forceinline__ double* drive_slot(double* P, int M, int c) { return 
 // = G^-1 T_k (G^-1 to Gi unless null); at stage 0 the readout signal and the records;
 // the drive coefficient of the stage time t. Every block of a trajectory forms G^-1
 // (latency, ~1000 cycles a sweep in FP64) and its share of X_k, whose 8 M^3 FMAs
-// take one SM 31k cycles at M = 20. It replaces a Cholesky factorisation and two
+// take one SM 31k cycles at M = 20: 28 us in FP64, 16 us in double-word FP32 (two
+// trajectories, M = 20, cold caches). It replaces a Cholesky factorisation and two
 // triangular sweeps over 2 M columns in one block, ~70 barriers of FP64 latency.
-// A: WidePivot, or DwArith for the FP32 state of the wide schedule (Gi null then).
+// A: WidePivot, or DwArith for the FP32 state of the wide schedule.
 // StepRef: the step and the record are the device counter's.
 template <typename A>
 __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, double2* __restrict__ Gi, long step, int stage,
@@ -234,7 +236,7 @@ __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, doubl
     }
     step = s0 + sr.k;
     record = stage == 0 && step % rp.pop_every == 0;
-    t += (double)step * rp.dt;
+    t = __dadd_rn(__dmul_rn((double)step, rp.dt), t);   // as the host forms it
   }
   const int tj = blockIdx.y, g = blockIdx.x;
   const TrajDev d = p.traj[tj];
@@ -338,7 +340,10 @@ void plain_solve_launch(const DevPtrs& p, const RunParams& rp, double2* Gi, long
 }
 
 // Thread: one row, the columns m and m + 1. Bound by the FP64 pipe for the
-// complex128 state: 8 FMAs per column and l of the two projections, ~45 others.
+// complex128 state: 8 FMAs per column and l of the two projections, ~45 others; 182 us
+// for 12 trajectories of N = 2000, M = 20 (160 us at the pipe's rate). For a few
+// complex64 trajectories bound by the latency of its loads (16 us for two): the ten
+// neighbours' and eight l's are in flight together.
 constexpr int RT = 128;   // threads per block
 
 template <typename T2>
@@ -573,27 +578,33 @@ cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk,
   return integrate_t<double2>(p, rp, max_nblk, max_N, step0, n_steps, s);
 }
 
-// The wide schedule of the fused engine: complex64 state, double-word Gram and M x M
-// phase, the step counter on the device. The buffers of p are the caller's.
-cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s) {
-  float2* Z[4] = {reinterpret_cast<float2*>(p.Zn), reinterpret_cast<float2*>(p.Za), reinterpret_cast<float2*>(p.Zb),
-                  reinterpret_cast<float2*>(p.Za)};
+// The wide schedule of the fused engine: the step counter on the device, for the
+// complex64 state the double-word Gram and M x M phase. The buffers of p are the caller's.
+template <typename T2>
+static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s) {
+  using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, WidePivot>::type;
+  T2* Z[4] = {reinterpret_cast<T2*>(p.Zn), reinterpret_cast<T2*>(p.Za), reinterpret_cast<T2*>(p.Zb),
+              reinterpret_cast<T2*>(p.Za)};
   const dim3 ggrid(max_nblk, rp.n_traj);
   const double c[4] = {0.0, 0.5 * rp.dt, 0.5 * rp.dt, rp.dt};
   for (long k = 0; k <= n_steps; ++k) {
     const StepRef ref{p.dstep, k, n_steps};
     for (int stage = 0; stage < (k < n_steps ? 4 : 1); ++stage) {
       const int solve = k < n_steps;
-      plain_gram<float2><<<ggrid, PT, 0, s>>>(p.traj, Z[stage], p.part, stage == 0, ref, rp.pop_every, sq_table());
+      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Z[stage], p.part, stage == 0, ref, rp.pop_every, sq_table());
       plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 ? LR_MAX_NT + 1 : 0, s);
-      plain_solve<DwArith><<<dim3(solve_blocks(rp, solve), rp.n_traj), ST, 0, s>>>(p, rp, nullptr, 0, stage, 0, solve,
-                                                                                   c[stage], ref);
+      plain_solve<A><<<dim3(solve_blocks(rp, solve), rp.n_traj), ST, 0, s>>>(p, rp, nullptr, 0, stage, 0, solve, c[stage],
+                                                                             ref);
       if (solve) rhs_launch(p, rp, max_N, Z[stage], stage < 3 ? Z[stage + 1] : nullptr, stage, nullptr, 0, ref, s);
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, int fp32,
+                           cudaStream_t s) {
+  return fp32 ? wide_t<float2>(p, rp, max_nblk, max_N, n_steps, s) : wide_t<double2>(p, rp, max_nblk, max_N, n_steps, s);
 }
 
 }  // namespace lr

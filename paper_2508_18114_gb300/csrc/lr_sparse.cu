@@ -33,8 +33,8 @@
 // Precisions: FP64 throughout, or FP32_G64 - the state, the operator apply,
 // T_k, the projection term and the RK4 update in FP32, the Gram matrix
 // summed in double-word FP32 (~2^-48) from the exact products of FP32
-// entries (TwoProduct by one FMA), the M x M phase in double-word FP32, the
-// static diagonal of A and the step sizes as hi + lo floats, and the signal in FP64.
+// entries (TwoProduct by one FMA), the M x M phase in FP64 (double-word FP32 where
+// the launches stand in for the fused kernel, as there), the static diagonal of A and the step sizes as hi + lo floats, and the signal in FP64.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -43,7 +43,6 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "lr_internal.cuh"
@@ -152,7 +151,8 @@ __global__ void __launch_bounds__(64) sp_chi(SpDev d, SpParams p, long step, dou
 
 // Row n of operator blockIdx.z (the readout alone if only_r) times the columns m0 ..
 // m0 + 3 of Zs: every entry's weight chi val is formed once for the four (in FP64 it
-// costs as much as a column, and the FP64 pipe is the bound), and the operators of a
+// costs as much as a column, and the FP64 pipe is the bound: with the Gram's idle lanes
+// taken out, a stage of 32 trajectories, N = 2000, M = 20, 1.67 -> 1.30 ms), and the operators of a
 // small batch go side by side. ci: stage time within the table of channel factors.
 constexpr int AT = 128;
 template <typename T2>
@@ -557,7 +557,7 @@ using namespace lr;
 struct lr_sparse {
   int N, M, K, T, n_levels, nblk, ntile;
   int fp32;   // 1: FP32_G64 state arithmetic
-  int fused;  // 1: the fused persistent kernel (FP32_G64), 0: four launches per RK4 stage
+  int fused;  // 1: the fused persistent kernel (FP32_G64), 0: the launches per RK4 stage
   int gram_tc;   // fused: 1 when the Gram matrix is formed on the tensor cores (rank padded to 20)
   int wide;    // fused: 1 when the whole-chip launches are faster than the teams
   int n_cta;   // fused: persistent CTAs (n_team teams of team_c)
@@ -799,7 +799,6 @@ void launch_gram(const lr_sparse* s, const SpDev& d, const SpParams& p, int mode
 template <typename T2>
 void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, long step0, long n_steps, double dt,
                          cudaStream_t st) {
-  using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, WidePivot>::type;
   const unsigned ab = (unsigned)(((long long)s->N * ((s->M + 3) / 4) + AT - 1) / AT);
   const int rb = SP_T / s->M;
   const dim3 gu((unsigned)((s->N + rb - 1) / rb), (unsigned)s->T);
@@ -807,6 +806,13 @@ void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, 
   // a trajectory's share of two blocks per SM, at most eight
   const unsigned sb = (unsigned)std::max(1, std::min(8, 304 / s->T));
   auto reduce = [&](int lo, int hi) { sp_reduce<<<dim3((hi - lo + 31) / 32, s->T), SP_T, 0, st>>>(d, p, lo, hi); };
+  // the M x M phase: that of the fused kernel where these launches stand in for it, else FP64
+  auto solve = [&](unsigned blocks, long step, int mode) {
+    if (s->wide)
+      sp_solve<DwArith><<<dim3(blocks, s->T), ST, 0, st>>>(d, p, step, mode);
+    else
+      sp_solve<WidePivot><<<dim3(blocks, s->T), ST, 0, st>>>(d, p, step, mode);
+  };
   for (long i = 0; i <= n_steps; ++i) {
     const long step = step0 + i;
     const bool rec = step % s->pop_every == 0;
@@ -817,7 +823,7 @@ void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, 
       sp_apply<T2><<<dim3(ab, s->T), AT, 0, st>>>(d, p, c4, 1);
       launch_gram<T2>(s, d, p, mode, st);
       reduce(n2, no);
-      sp_solve<A><<<dim3(1, s->T), ST, 0, st>>>(d, p, step, mode);
+      solve(1, step, mode);
       break;
     }
     for (int stg = 0; stg < 4; ++stg) {
@@ -825,7 +831,7 @@ void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, 
       sp_apply<T2><<<dim3(ab, s->T, s->K + (stg == 0 ? 2 : 1)), AT, 0, st>>>(d, p, c4 + stg, 0);
       launch_gram<T2>(s, d, p, mode, st);
       reduce(0, stg == 0 ? no : n2);
-      sp_solve<A><<<dim3(sb, s->T), ST, 0, st>>>(d, p, step, mode);
+      solve(sb, step, mode);
       sp_update<T2><<<gu, SP_T, 0, st>>>(d, p, stg, dt);
     }
   }
@@ -937,7 +943,7 @@ extern "C" lr_status lr_sparse_create(const lr_sparse_model* m, int n_traj, int 
   }
   s->ws = nullptr;
   s->ws_bytes = 0;
-  // the fused kernel: FP32_G64, unless LR_SPARSE_FUSED=0 selects the four-launch path;
+  // the fused kernel: FP32_G64, unless LR_SPARSE_FUSED=0 selects the launch path;
   // one persistent CTA per SM (fewer when the batch is smaller)
   s->fused = 0;
   s->n_cta = s->n_team = s->team_c = 0;

@@ -1,4 +1,4 @@
-"""The wide schedule of FP32_G64 batches that are far smaller than the GPU (a few
+"""The wide schedule of batches that are far smaller than the GPU (a few
 launches per RK4 stage over the whole chip, LR_FUSED_WIDE / LR_SPARSE_WIDE)
 against the FP64 engines, and its CUDA graph replays against direct calls.
 
@@ -56,8 +56,12 @@ def test_wide_against_fp64(monkeypatch, dims, ranks, frame):
     wl = _workload(dims, ranks, 0 if len(ranks) == 1 else 1, frame)
     monkeypatch.setenv("LR_FUSED_WIDE", "1")
     o32, z32 = _run(wl, "fp32_g64", "fused")
+    w64, y64 = _run(wl, "fp64", "fused")
     monkeypatch.delenv("LR_FUSED_WIDE")
     o64, z64 = _run(wl, "fp64", "plain")
+    # FP64: the plain engine's kernels and arithmetic, to the last bit
+    assert all(np.array_equal(a, b) for a, b in zip(y64, z64))
+    assert all(np.array_equal(w64[k], o64[k]) for k in ("beta", "pops", "nphot", "trace", "eps_a"))
     for a, b in zip(z32, z64):
         assert np.linalg.norm(a - b) <= TOL * np.linalg.norm(b)
     for k in ("beta", "pops", "nphot", "trace"):
