@@ -44,16 +44,16 @@ FP64_FMA_PER_CLK = 2
 # and eps_a in FP64.
 DTYPE_LABEL = {
     "fp64": "f64",
-    "fp32_g64": "f32 bulk; double-word f32 (~2^-48) Gram, LDL^dag, G^-1 and X_k; f64 signal",
-    "fp32": "f32 bulk and Gram; double-word f32 (~2^-48) LDL^dag, G^-1 and X_k; f64 signal",
-    "tf32_g64": "f32 bulk, tf32 projection; double-word f32 (~2^-48) Gram, LDL^dag, G^-1 and X_k; f64 signal",
+    "fp32_g64": "f32 bulk; double-word f32 (~2^-48) Gram, G^-1 and X_k; f64 signal",
+    "fp32": "f32 bulk and Gram; double-word f32 (~2^-48) G^-1 and X_k; f64 signal",
+    "tf32_g64": "f32 bulk, tf32 projection; double-word f32 (~2^-48) Gram, G^-1 and X_k; f64 signal",
 }
 # DRAM bytes per trajectory-step of the tensor-core-Gram kernel, from its ncu capture on the
 # 76-trajectory, 10-step case (0.578 GB read + 1.713 GB written for 760 trajectory-steps)
 TRAFFIC_GRAM_TC = 3.015e6
 # FP32_G64 with the Gram matrix on the tensor cores (the default plan of the N=2000, M=20 batch)
 DTYPE_GRAM_TC = ("f32 bulk; FP64-class (~2^-48) Gram from exact bf16-slice tcgen05 MMAs (f32 accumulation, "
-                 "exact) and double-word sums; double-word f32 LDL^dag, G^-1 and X_k; f64 signal")
+                 "exact) and double-word sums; double-word f32 G^-1 and X_k; f64 signal")
 
 
 def parse():
@@ -446,7 +446,7 @@ def run_ours(args):
     # kernels per bench step: the integrator's (plain: 3 per RK4 stage pair and
     # records; fused: one persistent launch), the eps_a epilogue and the step advance
     if engine == "plain":
-        launches = (12 * chunk + 2) + 2
+        launches = (16 * chunk + 3) + 2
     else:
         launches = 3
     launches *= args.steps
@@ -493,7 +493,7 @@ def run_ours(args):
         pv = world * bp.n_traj * args.plain_steps / (pms * 1e-3)
         plain = {"value": pv, "unit": "traj*steps/s", "engine": "plain", "dtype": "f64",
                  "steps_timed": args.plain_steps, "speedup": value / pv,
-                 "workload": "the same batch on the plain FP64 kernels (three launches per stage, state in HBM)",
+                 "workload": "the same batch on the plain FP64 kernels (four launches per stage, state in HBM)",
                  "accuracy": {"plain_fp64": "1e-10 relative against the FP64 oracle (parity tests)",
                               "this_line": "error_vs_oracle_full_pulse (FP32 bulk over the whole pulse)"}}
         bp.close()
@@ -587,7 +587,7 @@ def run_adjoint(args):
                  "adjoint": "lr_backward, plain-kernel recomputation per checkpoint segment (%d steps), %s"
                             % (ck, "FP64" if prec == "fp64" else
                                "FP32 bulk with the Gram matrix summed from exact products in double-word FP32, FP64 "
-                               "Cholesky/G^-1/solves, FP64 signal and gradient sums")})
+                               "G^-1 and X_k, FP64 signal and gradient sums")})
     print(json.dumps({"metric": "adjoint_traj_steps_per_s", "value": value, "unit": "traj*steps/s",
                       "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * tt / args.steps,
                       "higher_is_better": True, "dtype": "f64" if prec == "fp64" else "f32 bulk (f64 Gram/solves)",
@@ -686,7 +686,7 @@ def run_paper(args):
         and os.environ.get("LR_SPARSE_SPLIT", "1") != "0"
     kname = (("sf_kernel (fused persistent sparse kernel, one launch per integrate; %s)"
               % ("equal spans of trajectory-steps per CTA" if split else "%d CTA(s) per trajectory" % team))
-             if b.fused else "integrate (sparse engine, 4 launches per RK4 stage)")
+             if b.fused else "integrate (sparse engine, 5 launches per RK4 stage)")
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": None, "kernel": kname,
                 "peak_source": "%s FMA pipe: 152 SMs x %d FMA/clk x 2 x %.0f MHz sampled SM clock (unit counts)"
@@ -694,10 +694,10 @@ def run_paper(args):
     pm = pipe_peak_measured("fp64_fma" if prec == "fp64" else "fp32_fma", stream)
     roofline["peak_measured"] = pm
     roofline["frac_of_measured"] = achieved / pm if pm else None
-    # fused: one integrate launch and sp_loss per bench step; four-launch path: per RK4
-    # step sp_chi + 4 x (apply, gram, solve, update), the closing observation pass
-    # sp_chi, apply, gram, solve, then sp_loss
-    launches = (2 if b.fused else 17 * chunk + 4 + 1) * args.steps
+    # fused: one integrate launch and sp_loss per bench step; launch path: per RK4 step
+    # 4 x (apply, gram, reduce, solve, update), sp_chi every eight steps, the closing
+    # observation pass apply, gram, reduce, solve, then sp_loss
+    launches = (2 if b.fused else 20 * chunk + chunk // 8 + 1 + 4 + 1) * args.steps
 
     e2e = None
     if not args.no_e2e:
@@ -740,10 +740,10 @@ def run_paper(args):
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "f64" if prec == "fp64" else (DTYPE_GRAM_TC if b.fused and b.gram_tc else
-                                                   ("f32 bulk; double-word f32 (~2^-48) Gram, LDL^dag, G^-1 "
+                                                   ("f32 bulk; double-word f32 (~2^-48) Gram, G^-1 "
                                                     "and X_k; f64 signal") if b.fused else
-                                                   "f32 bulk; double-word f32 (~2^-48) Gram; f64 Cholesky, "
-                                                   "solves and signal"),
+                                                   "f32 bulk; double-word f32 (~2^-48) Gram; f64 G^-1, "
+                                                   "X_k and signal"),
             "data": "synthetic (seeded flat-top pulses, seeded initial states)",
             "config": {"workload": "paper: %d candidates x {g,e} = %d trajectories, normal-mode model of Sec. S2 "
                                    "(%s), N=%d (%s), M=%d, dt=%g ns, tau=%g ns, %s"
@@ -751,7 +751,7 @@ def run_paper(args):
                                       else "frame of the drive, counter-rotating terms kept", model["N"],
                                       "x".join(map(str, wl.dims)), wl.M, dt, wl.tau, prec),
                        "trajectories": T, "N": model["N"], "M": wl.M, "nnz": int(model["nnz"]),
-                       "engine": "sparse (fused persistent kernel)" if b.fused else "sparse (four launches per stage)",
+                       "engine": "sparse (fused persistent kernel)" if b.fused else "sparse (five launches per stage)",
                        "gram": ("tcgen05 bf16 slices (exact), double-word sums" if b.fused and b.gram_tc else
                                 "double-word FP32 on the CUDA cores" if prec != "fp64" else "f64"),
                        "schedule": (("equal spans of the batch's trajectory-steps, one per CTA" if split else
