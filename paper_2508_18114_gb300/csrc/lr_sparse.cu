@@ -33,8 +33,10 @@
 // Precisions: FP64 throughout, or FP32_G64 - the state, the operator apply,
 // T_k, the projection term and the RK4 update in FP32, the Gram matrix
 // summed in double-word FP32 (~2^-48) from the exact products of FP32
-// entries (TwoProduct by one FMA), the M x M phase in FP64 (double-word FP32 where
-// the launches stand in for the fused kernel, as there), the static diagonal of A and the step sizes as hi + lo floats, and the signal in FP64.
+// entries (TwoProduct by one FMA), the signal, photons and populations from exact
+// products too (double-word FP32 inside a block, FP64 across), the M x M phase in FP64
+// (double-word FP32 where the launches stand in for the fused kernel, as there), the
+// static diagonal of A and the step sizes as hi + lo floats.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -229,6 +231,24 @@ template <> struct Acc<float2> {
   __device__ double2 t() const { return mk((double)re.hi, (double)im.hi); }
 };
 
+// Sum of an observable: FP64, or for the FP32 state the exact products of its entries
+// in double-word FP32 (eps_a depends on the small difference of two signals).
+template <typename T> struct ObsSum;
+template <> struct ObsSum<double> {
+  double s = 0.0;
+  __device__ void add_prod(double a, double b) { s = fma(a, b, s); }
+  __device__ void add_down(int o) { s += __shfl_down_sync(0xffffffffu, s, o); }
+  __device__ double value() const { return s; }
+};
+template <> struct ObsSum<float> {
+  DW s{0.f, 0.f};
+  __device__ void add_prod(float a, float b) { dw_add_prod(s, a, b); }
+  __device__ void add_down(int o) {
+    dw_add(s, DW{__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o)});
+  }
+  __device__ double value() const { return dw_value(s); }
+};
+
 // Entries per thread of the (1 + K) M^2 partial sums: up to (1 + 3) 32^2 / 256.
 constexpr int ACC_MAX = (1 + LR_SPARSE_MAX_JUMPS) * LR_MAX_RANK * LR_MAX_RANK / SP_T;
 
@@ -238,8 +258,8 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
   using T = typename Scalar<T2>::type;
   constexpr int R = rows_per_block<T2>();
   __shared__ T2 sZ[R][LR_MAX_RANK], sY[LR_SPARSE_MAX_JUMPS + 1][R][LR_MAX_RANK];
-  __shared__ T rsum[R][4];
-  __shared__ T stot[4 + LR_MAX_NT];   // signal, photons, trace, populations (written by thread 0)
+  __shared__ double rsum[R];              // |z|^2 of the tile's rows
+  __shared__ double wsum[SP_T / 32][3];   // signal and photons by warp
   __shared__ int slev[R];
   const int tj = blockIdx.y, b = blockIdx.x, M = p.M, K = p.K, MM = M * M;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -266,7 +286,8 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
   Acc<T2> acc[NACC];
 #pragma unroll
   for (int q = 0; q < NACC; ++q) acc[q].zero();
-  if (tid < 4 + LR_MAX_NT) stot[tid] = 0;
+  ObsSum<T> sig[3];    // this lane's share of Re, Im conj(z) r z and |r z|^2
+  double lev = 0.0;    // thread l < n_levels: population of level l; the next one: the trace
   // row tiles b, b + nblk, b + 2 nblk, ... in increasing order
   for (int tile = b; tile < p.ntile; tile += p.nblk) {
     const int r0 = tile * R, rows = min(R, p.N - r0);
@@ -304,36 +325,30 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
       }
     }
     if (beta || obs) {
-      // one warp per row, lanes over m: conj(z) r z, |r z|^2, |z|^2 in the
-      // state's arithmetic; then one lane per row; fixed-order shuffle sums
+      // one warp per row, lanes over m
       for (int r = warp; r < R; r += SP_T / 32) {
-        T v[4] = {0, 0, 0, 0};
+        ObsSum<T> w;
         if (r < rows && lane < M) {
           const T2 z = sZ[r][lane], y = sY[LR_SPARSE_MAX_JUMPS][r][lane];
-          v[0] = fma(z.x, y.x, z.y * y.y);
-          v[1] = fma(z.x, y.y, -z.y * y.x);
-          v[2] = fma(y.x, y.x, y.y * y.y);
-          v[3] = fma(z.x, z.x, z.y * z.y);
+          sig[0].add_prod(z.x, y.x);
+          sig[0].add_prod(z.y, y.y);
+          sig[1].add_prod(z.x, y.y);
+          sig[1].add_prod(-z.y, y.x);
+          sig[2].add_prod(y.x, y.x);
+          sig[2].add_prod(y.y, y.y);
+          w.add_prod(z.x, z.x);
+          w.add_prod(z.y, z.y);
         }
-        for (int o = 16; o > 0; o >>= 1)
-          for (int c = 0; c < 4; ++c) v[c] += __shfl_down_sync(0xffffffffu, v[c], o);
-        if (lane == 0)
-          for (int c = 0; c < 4; ++c) rsum[r][c] = v[c];
+        if (obs) {
+          for (int o = 16; o > 0; o >>= 1) w.add_down(o);
+          if (lane == 0) rsum[r] = w.value();
+        }
       }
-      __syncthreads();
-      if (warp == 0) {
-        T v[4];
-        for (int c = 0; c < 4; ++c) v[c] = lane < rows ? rsum[lane][c] : (T)0;
-        for (int o = 16; o > 0; o >>= 1)
-          for (int c = 0; c < 4; ++c) v[c] += __shfl_down_sync(0xffffffffu, v[c], o);
-        if (lane == 0)
-          for (int c = 0; c < 4; ++c) stot[c] += v[c];
-        if (obs)
-          for (int l = 0; l < p.n_levels; ++l) {
-            T w = (lane < rows && slev[lane] == l) ? rsum[lane][3] : (T)0;
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
-            if (lane == 0) stot[4 + l] += w;
-          }
+      if (obs) {
+        __syncthreads();
+        if (tid <= p.n_levels)
+          for (int r = 0; r < rows; ++r)
+            if (slev[r] == tid || tid == p.n_levels) lev += rsum[r];
       }
     }
   }
@@ -353,10 +368,19 @@ __global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
     }
   }
   const size_t o2 = (size_t)2 * n_ent;   // beta re, im, nphot, trace, pops[n_levels]
-  if ((beta || obs) && tid == 0) {   // stot was last written by this thread
-    for (int c = 0; c < 4; ++c) out[o2 + c] = (double)stot[c];
-    if (obs)
-      for (int l = 0; l < p.n_levels; ++l) out[o2 + 4 + l] = (double)stot[4 + l];
+  if (beta || obs) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      for (int o = 16; o > 0; o >>= 1) sig[c].add_down(o);
+      if (lane == 0) wsum[warp][c] = sig[c].value();
+    }
+    __syncthreads();
+    if (tid < 3) {
+      double v = wsum[0][tid];
+      for (int w = 1; w < SP_T / 32; ++w) v += wsum[w][tid];
+      out[o2 + tid] = v;
+    }
+    if (obs && tid <= p.n_levels) out[o2 + (tid == p.n_levels ? 3 : 4 + tid)] = lev;
   }
 }
 
