@@ -179,6 +179,11 @@ lr_status lr_create(int n_cand, const lr_model* models, const int* ranks, const 
       d.J = m.n_modes == 3 ? m.J : 0.0;
       d.kappa = m.kappa;
       d.gamma = m.gamma;
+      const double rate[4] = {d.g, d.J, 0.5 * d.kappa, 0.5 * d.gamma};
+      for (int k = 0; k < 4; ++k) {
+        d.rate32[k].x = (float)rate[k];
+        d.rate32[k].y = (float)(rate[k] - (double)d.rate32[k].x);
+      }
       z_off += N * M;
       p_off += (long long)d.nblk * (long long)lr::plain_partial_doubles(M);
       c->nt_max = std::max(c->nt_max, Nt);

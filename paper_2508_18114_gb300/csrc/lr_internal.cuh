@@ -24,6 +24,7 @@ struct TrajDev {
   long long z_off;  // offset of this trajectory in the state arrays (complex elements)
   long long p_off;  // plain engine: offset in the partial-sum array (doubles)
   double wq, alpha, wr, wf, g, J, kappa, gamma;
+  float2 rate32[4];  // g, J, kappa / 2, gamma / 2 as hi + lo floats, for the kernels of the complex64 state
 };
 
 struct PulseDev {

@@ -37,6 +37,60 @@ const SqTab& sq_table() {
   return t;
 }
 
+// sqrt(k) = hi + lo (x, y), for the weights of a complex64 state.
+struct SqTabF {
+  float2 v[SQ_N];
+};
+static const SqTabF& sq_table_f() {
+  static const SqTabF t = [] {
+    SqTabF x;
+    for (int k = 0; k < SQ_N; ++k) {
+      const double v = std::sqrt((double)k);
+      x.v[k].x = (float)v;
+      x.v[k].y = (float)(v - (double)x.v[k].x);
+    }
+    return x;
+  }();
+  return t;
+}
+
+// A matrix element g sqrt(k) .. sqrt(l), rounded once to the state's type. FP32 state:
+// the factors as hi + lo floats (exact products by FMA, ~2^-46 before the rounding),
+// so that no coupling is off by several roundings in every step, without FP64.
+template <typename T>
+struct Weight;
+template <>
+struct Weight<double> {
+  using Tab = SqTab;
+  double v;
+  __device__ __forceinline__ Weight(double g, float2) : v(g) {}
+  __device__ __forceinline__ Weight times(const Tab& t, int k) const { return Weight(v * sq_of(t, k), float2()); }
+  __device__ __forceinline__ double round() const { return v; }
+};
+template <>
+struct Weight<float> {
+  using Tab = SqTabF;
+  float hi, lo;
+  __device__ __forceinline__ Weight(double, float2 g) : hi(g.x), lo(g.y) {}
+  __device__ __forceinline__ Weight times(const Tab& t, int k) const {
+    Weight s(*this);
+    float2 q;
+    if (k < SQ_N) {
+      q = t.v[k];
+    } else {
+      const double v = sqrt((double)k);
+      q.x = (float)v;
+      q.y = (float)(v - (double)q.x);
+    }
+    s.hi = hi * q.x;
+    s.lo = fmaf(hi, q.x, -s.hi) + fmaf(hi, q.y, lo * q.x);
+    return s;
+  }
+  __device__ __forceinline__ float round() const { return hi + lo; }
+};
+static const SqTab& weight_table(double) { return sq_table(); }
+static const SqTabF& weight_table(float) { return sq_table_f(); }
+
 constexpr int PR = 16;        // rows per Gram block
 constexpr int PT = 256;       // threads per block
 
@@ -350,7 +404,8 @@ template <typename T2>
 __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T2* __restrict__ Zin,
                                                 T2* __restrict__ Zout, int stage,
                                                 const double* __restrict__ ctab, int cstride, StepRef ref,
-                                                const __grid_constant__ SqTab sq) {
+                                                const __grid_constant__
+                                                typename Weight<typename real_of<T2>::type>::Tab sq) {
   if (ref.dstep && (*ref.dstep < 0 || *ref.dstep + ref.n > rp.max_steps)) return;
   using T = typename real_of<T2>::type;
   constexpr bool f32 = sizeof(T) == 4;
@@ -423,16 +478,17 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
     off[na] = on ? o : 0;
     w[na++] = on ? wt : (T)0;
   };
+  using W = Weight<T>;
   // g (b + b^dag)(a + a^dag); RWA keeps g (b^dag a + b a^dag) only
 #pragma unroll
   for (int a = -1; a <= 1; a += 2) {
     const int it2 = ri.it + a;
     const bool ot = it2 >= 0 && it2 < d.Nt;
-    const T ct = (T)d.g * (T)sq_of(sq, max(ri.it, it2));
+    const W ct = W(d.g, d.rate32[0]).times(sq, max(ri.it, it2));
 #pragma unroll
     for (int bb = -1; bb <= 1; bb += 2) {
       const int ir2 = ri.ir + bb;
-      add(ot && ir2 >= 0 && ir2 < d.Nr && !(rwa && a == bb), a * st + bb * sr, ct * (T)sq_of(sq, max(ri.ir, ir2)));
+      add(ot && ir2 >= 0 && ir2 < d.Nr && !(rwa && a == bb), a * st + bb * sr, ct.times(sq, max(ri.ir, ir2)).round());
     }
   }
   // J (a + a^dag)(f + f^dag); RWA keeps J (a^dag f + a f^dag) only
@@ -440,11 +496,11 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
   for (int a = -1; a <= 1; a += 2) {
     const int ir2 = ri.ir + a;
     const bool or2 = d.n_modes == 3 && ir2 >= 0 && ir2 < d.Nr;
-    const T cr = (T)d.J * (T)sq_of(sq, max(ri.ir, ir2));
+    const W cr = W(d.J, d.rate32[1]).times(sq, max(ri.ir, ir2));
 #pragma unroll
     for (int bb = -1; bb <= 1; bb += 2) {
       const int if2 = ri.iff + bb;
-      add(or2 && if2 >= 0 && if2 < d.Nf && !(rwa && a == bb), a * sr + bb, cr * (T)sq_of(sq, max(ri.iff, if2)));
+      add(or2 && if2 >= 0 && if2 < d.Nf && !(rwa && a == bb), a * sr + bb, cr.times(sq, max(ri.iff, if2)).round());
     }
   }
   // drive on the readout mode (stride 1): lab frame c(t) (r + r^dag); RWA
@@ -455,7 +511,7 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
   for (int a = -1; a <= 1; a += 2) {
     const int i2 = iro + a;
     const bool on = i2 >= 0 && i2 < dro;
-    const T s = on ? (T)sq_of(sq, max(iro, i2)) : (T)0;
+    const T s = on ? W(1.0, make_float2(1.f, 0.f)).times(sq, max(iro, i2)).round() : (T)0;
     sd[a > 0] = s;
     add(on, a, c * s);
   }
@@ -494,8 +550,8 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
       fi[u] = fma(s, pi[u], fi[u]);
     }
   };
-  if (iro + 1 < dro) project(zrow + ld, sX[0], (T)(0.5 * d.kappa * sq_of(sq, iro + 1)));
-  if (ri.it + 1 < d.Nt) project(zrow + (size_t)st * ld, sX[1], (T)(0.5 * d.gamma * sq_of(sq, ri.it + 1)));
+  if (iro + 1 < dro) project(zrow + ld, sX[0], W(0.5 * d.kappa, d.rate32[2]).times(sq, iro + 1).round());
+  if (ri.it + 1 < d.Nt) project(zrow + (size_t)st * ld, sX[1], W(0.5 * d.gamma, d.rate32[3]).times(sq, ri.it + 1).round());
   // RK4 (weights 1/6, 1/3, 1/3, 1/6)
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
@@ -531,7 +587,8 @@ template <typename T2>
 void rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const T2* zin, T2* zout, int stage,
                 const double* coef, int cstride, StepRef ref, cudaStream_t s) {
   const int blocks = (int)(((long)max_N * (LR_MAX_RANK / 2) + RT - 1) / RT);   // those past a trajectory's rank leave at once
-  plain_rhs<T2><<<dim3(blocks, rp.n_traj), RT, 0, s>>>(p, rp, zin, zout, stage, coef, cstride, ref, sq_table());
+  plain_rhs<T2><<<dim3(blocks, rp.n_traj), RT, 0, s>>>(p, rp, zin, zout, stage, coef, cstride, ref,
+                                                         weight_table(typename real_of<T2>::type()));
 }
 void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const double2* zin, double2* zout, int stage,
                       const double* coef, int cstride, cudaStream_t s) {
