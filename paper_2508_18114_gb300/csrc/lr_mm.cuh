@@ -42,17 +42,28 @@ __device__ __forceinline__ DW dw_norm(DW a) {   // |lo| <= ulp(hi) / 2
   r.lo = a.lo - (r.hi - a.hi);
   return r;
 }
-__device__ __forceinline__ DW dw_sum(DW a, DW b) {
-  const float s = a.hi + b.hi, bb = s - a.hi;
-  float e = (a.hi - (s - bb)) + (b.hi - bb);
-  e += a.lo + b.lo;
-  DW r;
-  r.hi = s + e;
-  r.lo = e - (r.hi - s);
-  return r;
-}
 struct alignas(16) DWC {
   DW re, im;
+};
+// A sum of a team's double-word partials in three floats: each addition keeps what lies
+// below 2^-48 of the sum, which a double-word one drops (an FP64 sum of the same terms
+// holds the FP64 pipe for ~1000 cycles at M = 20).
+struct DWSum {
+  float h = 0.f, m = 0.f, l = 0.f;
+  static __device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = a + b, t = s - a;
+    e = (a - (s - t)) + (b - t);
+    return s;
+  }
+  __device__ __forceinline__ void add(DW v) {
+    float e1, e2, e3;
+    h = two_sum(h, v.hi, e1);
+    m = two_sum(m, v.lo, e2);
+    m = two_sum(m, e1, e3);
+    l += e2 + e3;
+  }
+  __device__ __forceinline__ DW dw() const { return dw_norm(DW{h, m + l}); }
+  __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
 };
 
 // ----------------------------------------------------------------- entry arithmetic
@@ -71,7 +82,12 @@ struct DwArith {
   static __device__ __forceinline__ C conj(C v) { return C{v.re, {-v.im.hi, -v.im.lo}}; }
   static __device__ __forceinline__ C neg(C v) { return C{{-v.re.hi, -v.re.lo}, {-v.im.hi, -v.im.lo}}; }
   static __device__ __forceinline__ float magnitude(C v) { return v.re.hi; }
-  static __device__ __forceinline__ C sum(C a, C b) { return C{dw_sum(a.re, b.re), dw_sum(a.im, b.im)}; }
+  struct Sum {   // of a team's partials
+    DWSum re, im;
+    __device__ __forceinline__ void add(C v) { re.add(v.re), im.add(v.im); }
+    __device__ __forceinline__ C entry() const { return C{re.dw(), im.dw()}; }
+    __device__ __forceinline__ double2 value() const { return make_double2(re.value(), im.value()); }
+  };
   static __device__ __forceinline__ double2 value(C v) { return make_double2(dw_value(v.re), dw_value(v.im)); }
   // p e with p + e = a b to ~2^-48 (not normalised)
   static __device__ __forceinline__ DW prod(DW a, DW b) {
@@ -112,7 +128,12 @@ struct F64Arith {
   static __device__ __forceinline__ C conj(C v) { return mk(v.x, -v.y); }
   static __device__ __forceinline__ C neg(C v) { return mk(-v.x, -v.y); }
   static __device__ __forceinline__ double magnitude(C v) { return v.x; }
-  static __device__ __forceinline__ C sum(C a, C b) { return mk(a.x + b.x, a.y + b.y); }
+  struct Sum {
+    double x = 0.0, y = 0.0;
+    __device__ __forceinline__ void add(C v) { x += v.x, y += v.y; }
+    __device__ __forceinline__ C entry() const { return mk(x, y); }
+    __device__ __forceinline__ double2 value() const { return mk(x, y); }
+  };
   static __device__ __forceinline__ double2 value(C v) { return v; }
   static __device__ __forceinline__ C update(C v, C x, C y, R d) {   // v - x conj(y) d
     const double sr = y.x * d, si = y.y * d;

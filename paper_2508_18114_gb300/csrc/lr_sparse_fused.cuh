@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
   float2* XT = reinterpret_cast<float2*>(smem + a.o_xt);      // [K][Mp][Mp] (l, m)
   // [8..11) signal partials (Re, Im beta, photons), [64..96) population partials
   double* misc = reinterpret_cast<double*>(smem + a.o_misc);
-  DWC* gpart = reinterpret_cast<DWC*>(smem + a.o_gpart);           // [Mp][Mp]  G (i <= j) over this CTA's rows
+  double2* gpart = reinterpret_cast<double2*>(smem + a.o_gpart);   // [Mp][Mp]  G (i <= j) over this CTA's rows, FP64
   float2* tsum = reinterpret_cast<float2*>(smem + a.o_tsum);       // [K][Mp*Mp]  T_k of the team
   cg::cluster_group cluster = cg::this_cluster();
   const int C = TEAM ? a.C : 1;
@@ -541,9 +541,8 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
         dw_add(re, Sb[210 + e]);
         const DW n2 = Sb[420 + j * 20 + i];
         dw_add(im, DW{-n2.hi, -n2.lo});
-        re = dw_norm(re);
-        im = dw_norm(im);
-        gpart[i * Mp + j] = DWC{{re.hi * si * sj, re.lo * si * sj}, {im.hi * si * sj, im.lo * si * sj}};
+        const double sc = (double)si * (double)sj;
+        gpart[i * Mp + j] = mk(dw_value(re) * sc, dw_value(im) * sc);
       }
     } else if (warp == SG_W) {
       // the issuing warp
@@ -784,11 +783,12 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
                 dw_add(keep, t);
               });
               const int i = i0 + (lane >> 3), j = j0 + ((lane >> 1) & 3), c = lane & 1;
-              // G[i][j] over this CTA's rows, summed over the row blocks in order
+              // G[i][j] over this CTA's rows, summed over the row blocks in order (FP64: a
+              // double-word sum loses what lies below 2^-48 of it)
               if (i <= j) {
-                DW* gp = reinterpret_cast<DW*>(gpart) + 2 * (i * Mp + j) + c;
-                const DW val = i == j && c ? DW{0.f, 0.f} : dw_norm(v[0]);
-                *gp = blk ? dw_sum(*gp, val) : val;
+                double* gp = reinterpret_cast<double*>(gpart) + 2 * (i * Mp + j) + c;
+                const double val = i == j && c ? 0.0 : dw_value(v[0]);
+                *gp = blk ? *gp + val : val;
               }
             } else {
               const int t2 = task - n_g, k = t2 / (nt_ * nt_), r2 = t2 - k * nt_ * nt_, ti = r2 / nt_,
@@ -863,9 +863,12 @@ __global__ void __launch_bounds__(NT, 1) sf_kernel(const Args a) {
               g[u] = DwArith::zero();
               if (e < M * (M + 1) / 2) {
                 const int i = tri[e].x, j = tri[e].y, o = j * Mp + i;
-                g[u] = at_rank(gpart, 0)[o];
-                for (int r = 1; r < C; ++r) g[u] = DwArith::sum(g[u], at_rank(gpart, r)[o]);
-                g[u] = DwArith::conj(g[u]);   // G_ij, i >= j
+                double2 v = at_rank(gpart, 0)[o];
+                for (int r = 1; r < C; ++r) {
+                  const double2 w = at_rank(gpart, r)[o];
+                  v = mk(v.x + w.x, v.y + w.y);
+                }
+                to_entry(mk(v.x, -v.y), g[u]);   // G_ij, i >= j
               }
             }
             asm volatile("bar.sync 2, %0;" ::"r"(nw * 32) : "memory");   // mm.bad is clear
