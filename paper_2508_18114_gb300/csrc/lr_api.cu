@@ -335,10 +335,7 @@ lr_status lr_set_initial(lr_ctx* c, uint64_t seed, double eps, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DevPtrs p = dev_ptrs(c);
   RunParams rp = run_params(c);
-  int min_N = c->max_N;
-  for (const TrajDev& d : c->traj) min_N = std::min(min_N, d.N);
-  cudaError_t e =
-      lr::launch_initial_state(p, rp, min_N, c->max_N, c->max_M, c->opt.precision != LR_PREC_FP64, seed, eps, s);
+  cudaError_t e = lr::launch_initial_state(p, rp, c->max_N, c->max_M, c->opt.precision != LR_PREC_FP64, seed, eps, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "initial state kernel");
   e = cudaMemsetAsync(c->ws + c->o_err, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "clearing error word");

@@ -48,12 +48,13 @@ __device__ double block_sum(double v, double* sh) {
 // component is removed by zeroing one row; the rest is Cholesky QR: G = W^dag W
 // = L L^dag over the M - 1 Gaussian columns, Q = W L^-dag, which has the same q_j
 // (a QR factor with a positive diagonal is unique). Everything is FP64. A second
-// round brings the orthogonality from cond(W)^2 2^-53 to 2^-53; `rounds` is 1
-// where it cannot be seen (FP32 states with N >= 4 M: cond(W) < ~3).
+// round brings the orthogonality from cond(W)^2 2^-53 to 2^-53; there is one where it
+// cannot be seen (FP32 states with N >= 4 M: cond(W) < ~3).
 //
-// A cluster of CTAs per trajectory, each on N / C rows in tiles of ITR rows in
-// shared memory: draws and Gram sums of a tile in one sweep, the partial G of the
-// team added in rank order over distributed shared memory, the M x M factor in
+// A cluster of CTAs per trajectory. The rows go in up to IV parts, chosen by N alone, so
+// that the state does not depend on the batch around it; a CTA takes whole parts, in
+// tiles of ITR rows in shared memory: draws and Gram sums of a tile in one sweep, the
+// parts' G added in their order over distributed shared memory, the M x M factor in
 // every CTA, then Q tile by tile. Bound by the FP64 pipe (2 FMA/clk/SM): the draws
 // (~100 FP64 instructions a pair) and the 8 N M^2 FMAs of the two products. Column
 // by column Gram-Schmidt in one block per trajectory took a block sum and a sweep
@@ -61,16 +62,20 @@ __device__ double block_sum(double v, double* sh) {
 // 6.3 ms; two trajectories 5.7 ms, here 0.3 ms.
 constexpr int ITR = 128;            // rows per tile
 constexpr int IM = LR_MAX_RANK - 1; // most padding columns
+constexpr int IV = 8;               // most parts (the portable cluster size)
 
 __host__ __device__ inline int init_ldt(int m1) { return m1 | 1; }   // odd row stride: no bank conflicts down a column
-inline size_t init_smem(int m1) {
-  return sizeof(double2) * ((size_t)ITR * init_ldt(m1) + IT + 2 * (size_t)m1 * init_ldt(m1) + (size_t)m1 * (m1 + 1) / 2);
+// parts whose sums a CTA of a team of C keeps (alone it adds them as they come)
+inline int init_slots(int C) { return C == 1 ? 1 : (IV + C - 1) / C; }
+inline size_t init_smem(int m1, int slots) {
+  return sizeof(double2) *
+         ((size_t)ITR * init_ldt(m1) + IT + 2 * (size_t)m1 * init_ldt(m1) + (size_t)slots * m1 * (m1 + 1) / 2);
 }
 
 template <typename T2>
 __global__ void __launch_bounds__(IT) initial_state_kernel(const TrajDev* __restrict__ traj, double2* __restrict__ Wbase,
                                                            T2* __restrict__ Zbase, unsigned long long seed, double eps,
-                                                           int max_m1, int two_rounds) {
+                                                           int max_m1) {
   extern __shared__ __align__(16) unsigned char init_sm[];
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -83,12 +88,16 @@ __global__ void __launch_bounds__(IT) initial_state_kernel(const TrajDev* __rest
   double2* gred = tile + (size_t)ITR * init_ldt(max_m1);              // [groups][nep] partial sums
   double2* L = gred + IT;                                             // [M1][ldt]
   double2* Li = L + (size_t)max_m1 * init_ldt(max_m1);                // [M1][ldt]  L^-1
-  double2* gsum = Li + (size_t)max_m1 * init_ldt(max_m1);             // [M1 (M1 + 1) / 2]  G over the own rows
+  double2* gsum = Li + (size_t)max_m1 * init_ldt(max_m1);             // [slots][M1 (M1 + 1) / 2]  G over the own parts
   __shared__ double dinv[IM + 1];
   double2* W = Wbase + d.z_off;
   T2* Z = Zbase + d.z_off;
   const int psi = d.level0 * d.Nr * d.Nf;
-  const int r_lo = (int)((long long)N * q / C), r_hi = (int)((long long)N * (q + 1) / C);
+  const int V = min(IV, (N + ITR - 1) / ITR);   // parts; those of rank r: [V r / C, V (r + 1) / C)
+  const int v_lo = V * q / C, v_hi = V * (q + 1) / C;
+  auto row_of = [N, V](int v) { return (int)((long long)N * v / V); };
+  const int r_lo = row_of(v_lo), r_hi = row_of(v_hi);
+  const int two_rounds = sizeof(T2) == sizeof(double2) || N < 4 * M;
   const unsigned long long ts = splitmix64(seed, (unsigned long long)tj);
   const double w0 = sqrt(1.0 - M1 * eps), we = sqrt(eps);
   // column 0, and the rank padding of the row
@@ -104,47 +113,56 @@ __global__ void __launch_bounds__(IT) initial_state_kernel(const TrajDev* __rest
   const int gi = ent - gj * (gj + 1) / 2;
   const bool mine = ent < ne && group < groups;
   for (int round = 0; round < (M1 > 0 ? 1 + two_rounds : 0); ++round) {
-    double gr = 0.0, gim = 0.0;
-    for (int t0 = r_lo; t0 < r_hi; t0 += ITR) {
-      const int rows = min(ITR, r_hi - t0);
-      for (int e = tid; e < rows * M1; e += IT) {
-        const int r = e / M1, j = e - r * M1, n = t0 + r;
-        double2 w;
-        if (round == 0) {
-          const unsigned long long pidx = (unsigned long long)j * N + n;
-          const double u1 = uniform_open0(ts, 2ull * pidx), u2 = uniform_open0(ts, 2ull * pidx + 1ull);
-          const double rad = sqrt(-2.0 * log(u1));
-          double sn, cs;
-          sincospi(2.0 * u2, &sn, &cs);
-          w = n == psi ? mk(0.0, 0.0) : mk(rad * cs, rad * sn);
-          W[(size_t)n * ld + j + 1] = w;
-        } else {
-          w = W[(size_t)n * ld + j + 1];
+    for (int v = v_lo; v < v_hi; ++v) {
+      double gr = 0.0, gim = 0.0;
+      const int p_hi = row_of(v + 1);
+      for (int t0 = row_of(v); t0 < p_hi; t0 += ITR) {
+        const int rows = min(ITR, p_hi - t0);
+        for (int e = tid; e < rows * M1; e += IT) {
+          const int r = e / M1, j = e - r * M1, n = t0 + r;
+          double2 w;
+          if (round == 0) {
+            const unsigned long long pidx = (unsigned long long)j * N + n;
+            const double u1 = uniform_open0(ts, 2ull * pidx), u2 = uniform_open0(ts, 2ull * pidx + 1ull);
+            const double rad = sqrt(-2.0 * log(u1));
+            double sn, cs;
+            sincospi(2.0 * u2, &sn, &cs);
+            w = n == psi ? mk(0.0, 0.0) : mk(rad * cs, rad * sn);
+            W[(size_t)n * ld + j + 1] = w;
+          } else {
+            w = W[(size_t)n * ld + j + 1];
+          }
+          tile[r * ldt + j] = w;
         }
-        tile[r * ldt + j] = w;
+        __syncthreads();
+        if (mine)
+          for (int r = group; r < rows; r += groups) {
+            const double2 a = tile[r * ldt + gi], b = tile[r * ldt + gj];   // conj(a) b
+            gr = fma(a.x, b.x, fma(a.y, b.y, gr));
+            gim = fma(a.x, b.y, fma(-a.y, b.x, gim));
+          }
+        __syncthreads();
+      }
+      if (mine) gred[group * nep + ent] = mk(gr, gim);
+      __syncthreads();
+      for (int e = tid; e < ne; e += IT) {
+        double2 s = gred[e];
+        for (int g = 1; g < groups; ++g) s = mk(s.x + gred[g * nep + e].x, s.y + gred[g * nep + e].y);
+        double2* out = gsum + (C == 1 ? 0 : v - v_lo) * ne + e;
+        *out = C == 1 && v > 0 ? mk(out->x + s.x, out->y + s.y) : s;
       }
       __syncthreads();
-      if (mine)
-        for (int r = group; r < rows; r += groups) {
-          const double2 a = tile[r * ldt + gi], b = tile[r * ldt + gj];   // conj(a) b
-          gr = fma(a.x, b.x, fma(a.y, b.y, gr));
-          gim = fma(a.x, b.y, fma(-a.y, b.x, gim));
-        }
-      __syncthreads();
-    }
-    if (mine) gred[group * nep + ent] = mk(gr, gim);
-    __syncthreads();
-    for (int e = tid; e < ne; e += IT) {
-      double2 s = gred[e];
-      for (int g = 1; g < groups; ++g) s = mk(s.x + gred[g * nep + e].x, s.y + gred[g * nep + e].y);
-      gsum[e] = s;
     }
     cluster.sync();
-    for (int e = tid; e < ne; e += IT) {   // the team's partials in rank order; lower triangle G_ji = conj(G_ij)
-      double2 s = mk(0.0, 0.0);
-      for (int r = 0; r < C; ++r) {
-        const double2 v = cluster.map_shared_rank(gsum, r)[e];
-        s = mk(s.x + v.x, s.y + v.y);
+    for (int e = tid; e < ne; e += IT) {   // the parts in order; lower triangle G_ji = conj(G_ij)
+      double2 s = gsum[e];
+      if (C > 1) {
+        s = mk(0.0, 0.0);
+        for (int r = 0; r < C; ++r)
+          for (int k = 0; k < V * (r + 1) / C - V * r / C; ++k) {
+            const double2 w = cluster.map_shared_rank(gsum, r)[k * ne + e];
+            s = mk(s.x + w.x, s.y + w.y);
+          }
       }
       int j = 0;
       while ((j + 1) * (j + 2) / 2 <= e) ++j;
@@ -390,20 +408,21 @@ cudaError_t launch_grow(const DevPtrs& dst, const DevPtrs& src, int n_traj, int 
 
 template <typename T2>
 static cudaError_t launch_initial_t(const DevPtrs& p, const RunParams& rp, int max_N, int max_M, unsigned long long seed,
-                                    double eps, int two_rounds, cudaStream_t s) {
+                                    double eps, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(initial_state_kernel<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)init_smem(IM));
+    e = cudaFuncSetAttribute(initial_state_kernel<T2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)init_smem(IM, init_slots(2)));
   if (e != cudaSuccess) return e;
   // one CTA per SM in all: a team takes the SMs that the batch leaves over, at
   // least a tile of rows per CTA, within the portable cluster size
-  const int C = std::max(1, std::min({8, sms / std::max(1, rp.n_traj), (max_N + ITR - 1) / ITR}));
+  const int C = std::max(1, std::min({IV, sms / std::max(1, rp.n_traj), (max_N + ITR - 1) / ITR}));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C * rp.n_traj);
   cfg.blockDim = dim3(IT);
-  cfg.dynamicSmemBytes = init_smem(std::max(1, max_M - 1));
+  cfg.dynamicSmemBytes = init_smem(std::max(1, max_M - 1), init_slots(C));
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -413,13 +432,13 @@ static cudaError_t launch_initial_t(const DevPtrs& p, const RunParams& rp, int m
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, initial_state_kernel<T2>, p.traj, reinterpret_cast<double2*>(p.Za),
-                            reinterpret_cast<T2*>(p.Zn), seed, eps, std::max(1, max_M - 1), two_rounds);
+                            reinterpret_cast<T2*>(p.Zn), seed, eps, std::max(1, max_M - 1));
 }
 
-cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int min_N, int max_N, int max_M, int prec_fp32,
-                                 uint64_t seed, double eps, cudaStream_t s) {
-  if (prec_fp32) return launch_initial_t<float2>(p, rp, max_N, max_M, seed, eps, min_N < 4 * max_M, s);
-  return launch_initial_t<double2>(p, rp, max_N, max_M, seed, eps, 1, s);
+cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int max_N, int max_M, int prec_fp32, uint64_t seed,
+                                 double eps, cudaStream_t s) {
+  if (prec_fp32) return launch_initial_t<float2>(p, rp, max_N, max_M, seed, eps, s);
+  return launch_initial_t<double2>(p, rp, max_N, max_M, seed, eps, s);
 }
 
 // One block per candidate: trapezoid of |beta_e - beta_g|^2 over the step grid,

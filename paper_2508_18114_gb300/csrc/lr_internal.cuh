@@ -233,9 +233,9 @@ struct RunParams {
 };
 
 // lr_common.cu
-// min_N, max_N, max_M: over the batch's trajectories
-cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int min_N, int max_N, int max_M, int prec_fp32,
-                                 uint64_t seed, double eps, cudaStream_t s);
+// max_N, max_M: over the batch's trajectories
+cudaError_t launch_initial_state(const DevPtrs& p, const RunParams& rp, int max_N, int max_M, int prec_fp32, uint64_t seed,
+                                 double eps, cudaStream_t s);
 // Rank growth: dst's states = src's columns plus orthonormal padding columns of
 // weight eps, one block per trajectory (both contexts hold the same trajectories).
 cudaError_t launch_grow(const DevPtrs& dst, const DevPtrs& src, int n_traj, int prec_fp32, uint64_t seed, double eps,

@@ -1086,7 +1086,7 @@ extern "C" lr_status lr_sparse_set_initial(lr_sparse* s, const int* psi, uint64_
   RunParams rp;
   memset(&rp, 0, sizeof(rp));
   rp.n_traj = s->T;
-  if ((e = launch_initial_state(p, rp, s->N, s->N, s->M, s->fp32, seed, eps, st)) != cudaSuccess) return cuda_fail(s, e);
+  if ((e = launch_initial_state(p, rp, s->N, s->M, s->fp32, seed, eps, st)) != cudaSuccess) return cuda_fail(s, e);
   if ((e = cudaMemcpyAsync(d.Zs, d.Z, state_bytes(s), cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
     return cuda_fail(s, e);
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(s, e);
