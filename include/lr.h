@@ -334,11 +334,16 @@ lr_status lr_sync(lr_ctx* ctx, void* stream);
  * Gram matrix summed from exact FP32 products in double-word FP32 (~2^-48,
  * FP64-class); G^-1 and the M x M adjoint factors in
  * FP64; the readout signal and the gradient sums in FP64. The checkpoint
- * segments are recomputed with the PLAIN engine's kernels in that arithmetic,
- * and a segment's stage inputs and factors are kept up to 8 GB of workspace
+ * segments are recomputed with the PLAIN engine's kernels in that arithmetic
  * (the copies in the workspace are complex64 then: half the memory).
+ * With a workspace of lr_backward_workspace_size_kept bytes (three more copies of
+ * all states and 12 M x M factors per trajectory for every step of a segment; the same
+ * as lr_backward_workspace_size where that is over 8 GB) a segment's stage inputs and
+ * factors are kept when it is recomputed, instead of forming them again step by step:
+ * about 1.25 times as fast, the same gradient to the last bit.
  * Synchronous; returns the device error status. */
 lr_status lr_backward_workspace_size(const lr_ctx* ctx, int ckpt_every, size_t* bytes);
+lr_status lr_backward_workspace_size_kept(const lr_ctx* ctx, int ckpt_every, size_t* bytes);
 lr_status lr_backward(lr_ctx* ctx, void* dev_ws, size_t ws_bytes, const double* d_eps_a, double* d_theta,
                       int ckpt_every, void* stream);
 

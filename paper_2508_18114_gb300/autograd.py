@@ -15,7 +15,7 @@ import torch
 
 class AssignmentError(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, theta, batch, kinds, tau, dt, n_steps, seed, eps, ckpt_every):
+    def forward(ctx, theta, batch, kinds, tau, dt, n_steps, seed, eps, ckpt_every, keep):
         th = theta.detach().cpu().double().numpy()
         pulses = [(int(k), th[c, : (4 if int(k) == 0 else 8)]) for c, k in enumerate(kinds)]
         batch.set_pulse(pulses, tau)
@@ -24,15 +24,17 @@ class AssignmentError(torch.autograd.Function):
         out = batch.observables()
         ctx.batch = batch
         ctx.ckpt = ckpt_every
+        ctx.keep = keep
         ctx.kinds = list(kinds)
         return torch.from_numpy(np.array(out["eps_a"], dtype=np.float64))
 
     @staticmethod
     def backward(ctx, grad_eps):
         g = grad_eps.detach().cpu().double().numpy()
-        dth = ctx.batch.backward(g, ctx.ckpt)
-        return (torch.from_numpy(dth),) + (None,) * 8
+        dth = ctx.batch.backward(g, ctx.ckpt, keep=ctx.keep)
+        return (torch.from_numpy(dth),) + (None,) * 9
 
 
-def assignment_error(theta, batch, kinds, tau, dt, n_steps, seed, eps=1e-5, ckpt_every=200):
-    return AssignmentError.apply(theta, batch, kinds, tau, dt, n_steps, seed, eps, ckpt_every)
+def assignment_error(theta, batch, kinds, tau, dt, n_steps, seed, eps=1e-5, ckpt_every=200, keep=True):
+    """keep: as for ``LowRankBatch.backward``."""
+    return AssignmentError.apply(theta, batch, kinds, tau, dt, n_steps, seed, eps, ckpt_every, keep)

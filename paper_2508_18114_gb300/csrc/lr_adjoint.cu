@@ -28,8 +28,8 @@
 // Im tr(Fbar^dag (r + r^dag) U) dc/dtheta_i at the stage time.
 //
 // Forward stages run the plain engine's kernels. States are stored every `ckpt_every` steps; a segment is recomputed once,
-// keeping every stage input U_s, G^-1 and X_k' of its steps where they fit in
-// KEEP_BYTES, else step by step (the same kernels on the same inputs: the gradient
+// keeping every stage input U_s, G^-1 and X_k' of its steps where the caller's workspace
+// has room for them, else step by step (the same kernels on the same inputs: the gradient
 // does not depend on it), and the last segment is kept by the forward pass itself.
 //
 // Bound by the FP64 pipe (2 FMA/clk/SM; a warp instruction holds it for 16 cycles
@@ -466,12 +466,12 @@ __global__ void adj_gcoef(Ptrs a, const double* __restrict__ deps, double eta, l
 // ------------------------------------------------------------------ driver
 
 namespace {
-// Stage inputs and factors of a whole segment are kept up to this size (3% of HBM);
-// beyond it every step of the reverse pass recomputes its own.
+// Stage inputs and factors of a whole segment are kept up to this size (3% of HBM), in
+// a workspace that has the room; else every step of the reverse pass recomputes its own.
 constexpr size_t KEEP_BYTES = (size_t)8 << 30;
 }  // namespace
 
-BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles, long S, int K, int fp32) {
+BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles, long S, int K, int fp32, int keep) {
   BwdLayout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -484,7 +484,7 @@ BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles,
   L.K = std::min<long>(K, S);
   L.fp32 = fp32;
   L.n_seg = (S + L.K - 1) / L.K;
-  L.slots = (size_t)L.K <= KEEP_BYTES / (3 * T + fac) ? L.K : 1;
+  L.slots = keep && (size_t)L.K <= KEEP_BYTES / (3 * T + fac) ? L.K : 1;
   L.ck = take(T * L.n_seg);
   L.seg = take(T * (L.K + 1));
   L.cur = take(T);

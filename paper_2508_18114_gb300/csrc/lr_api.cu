@@ -583,14 +583,24 @@ lr_status lr_sync(lr_ctx* c, void* stream) {
   return check_device_error(c);
 }
 
+static lr::BwdLayout backward_layout(const lr_ctx* c, int ckpt_every, int keep) {
+  size_t part = 0;
+  for (const TrajDev& d : c->traj) part += (size_t)d.nblk * lr::plain_pstride(d.M);
+  return lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, part, c->step, ckpt_every, c->opt.precision != LR_PREC_FP64,
+                        keep);
+}
+
 lr_status lr_backward_workspace_size(const lr_ctx* c, int ckpt_every, size_t* bytes) {
   if (!c || !bytes || ckpt_every < 1) return LR_ERR_ARG;
   if (c->step < 1) return LR_ERR_STATE;
-  size_t part = 0;
-  for (const TrajDev& d : c->traj) part += (size_t)d.nblk * lr::plain_pstride(d.M);
-  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, part, c->step, ckpt_every,
-                                         c->opt.precision != LR_PREC_FP64);
-  *bytes = L.total;
+  *bytes = backward_layout(c, ckpt_every, 0).total;
+  return LR_OK;
+}
+
+lr_status lr_backward_workspace_size_kept(const lr_ctx* c, int ckpt_every, size_t* bytes) {
+  if (!c || !bytes || ckpt_every < 1) return LR_ERR_ARG;
+  if (c->step < 1) return LR_ERR_STATE;
+  *bytes = backward_layout(c, ckpt_every, 1).total;
   return LR_OK;
 }
 
@@ -608,10 +618,8 @@ lr_status lr_backward(lr_ctx* c, void* dev_ws, size_t ws_bytes, const double* d_
   if (c->opt.frame != 0) return fail(c, LR_ERR_UNSUPPORTED, "lr_backward supports the lab frame only");
   for (int k = 0; k < c->n_cand; ++k)
     if (!std::isfinite(d_eps_a[k])) return fail(c, LR_ERR_ARG, "non-finite cotangent");
-  size_t part = 0;
-  for (const TrajDev& d : c->traj) part += (size_t)d.nblk * lr::plain_pstride(d.M);
-  const lr::BwdLayout L = lr::bwd_layout(c->tot_elems, c->n_traj, c->n_cand, part, c->step, ckpt_every,
-                                         c->opt.precision != LR_PREC_FP64);
+  lr::BwdLayout L = backward_layout(c, ckpt_every, 1);
+  if (ws_bytes < L.total) L = backward_layout(c, ckpt_every, 0);
   if (!dev_ws || ws_bytes < L.total) return fail(c, LR_ERR_WORKSPACE, "backward workspace missing or too small");
   if (reinterpret_cast<uintptr_t>(dev_ws) % 256 != 0) return fail(c, LR_ERR_WORKSPACE, "backward workspace misaligned");
   cudaStream_t s = static_cast<cudaStream_t>(stream);

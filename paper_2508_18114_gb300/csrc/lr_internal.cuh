@@ -284,12 +284,13 @@ void plain_reduce_launch(const TrajDev* traj, int n_traj, int max_M, double* par
 
 // lr_adjoint.cu
 struct BwdLayout {
-  size_t ck, seg, cur, acc, U, Ub, Fb, lam, lamn, part, Xs, Gi, EP, Xs32, bpart, beta, coef, gcoef, deps, thbar, total;
+  size_t ck, seg, cur, acc, U, Ub, Fb, lam, lamn, part, Xs, Gi, EP, bpart, beta, coef, gcoef, deps, thbar, total;
   long n_seg, K;
-  long slots;   // steps whose stage inputs and M x M factors are kept: K, or 1 (recomputed step by step)
+  long slots;   // steps whose stage inputs and M x M factors have room: K, or 1 (recomputed step by step)
   int fp32;     // 1: FP32-bulk adjoint (complex64 states and cotangents)
 };
-BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles, long S, int K, int fp32);
+// keep: room for a whole segment's stage inputs and factors (where KEEP_BYTES allow)
+BwdLayout bwd_layout(long long tot, int n_traj, int n_cand, size_t part_doubles, long S, int K, int fp32, int keep);
 cudaError_t backward_run(const DevPtrs& main, const RunParams& rp, char* ws, const BwdLayout& L, long long tot,
                          int max_nblk, int max_N, int max_M, long S, const void* z0, int z0_fp32, const double* deps_host,
                          double* dtheta_host, cudaStream_t s);

@@ -35,7 +35,7 @@ EXPORTS = (
     "lr_set_initial", "lr_set_state", "lr_get_state", "lr_integrate",
     "lr_observables", "lr_sync", "lr_query", "lr_status_string",
     "lr_last_error", "lr_destroy", "lr_integrate_plain_noalloc",
-    "lr_backward_workspace_size", "lr_backward", "lr_loss", "lr_diagnostics",
+    "lr_backward_workspace_size", "lr_backward_workspace_size_kept", "lr_backward", "lr_loss", "lr_diagnostics",
     "lr_paper_model_size", "lr_paper_model_build", "lr_sparse_create", "lr_sparse_workspace_size",
     "lr_sparse_bind_workspace", "lr_sparse_set_initial", "lr_sparse_set_state", "lr_sparse_get_state",
     "lr_sparse_integrate", "lr_sparse_observables", "lr_sparse_loss", "lr_sparse_last_error",
@@ -109,6 +109,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.lr_destroy.restype = None
     lib.lr_integrate_plain_noalloc.argtypes = [C.POINTER(lr_model), i, C.POINTER(lr_pulse), d, vp, vp, d, l, l, vp]
     lib.lr_backward_workspace_size.argtypes = [vp, i, C.POINTER(C.c_size_t)]
+    lib.lr_backward_workspace_size_kept.argtypes = [vp, i, C.POINTER(C.c_size_t)]
     lib.lr_backward.argtypes = [vp, vp, C.c_size_t, vp, vp, i, vp]
     lib.lr_loss.argtypes = [vp, vp, vp, vp]
     lib.lr_assignment_shots.argtypes = [vp, d, l, i, C.c_uint64, vp, vp, vp, vp]
@@ -384,14 +385,24 @@ class LowRankBatch:
                                              C.c_void_p(_stream_ptr(stream))))
         return pur, eig
 
-    def backward(self, d_eps_a, ckpt_every=200, stream=None):
-        """dL/dtheta [n_cand, 8] for cotangents dL/deps_a (lr_backward)."""
+    def backward(self, d_eps_a, ckpt_every=200, stream=None, keep=True):
+        """dL/dtheta [n_cand, 8] for cotangents dL/deps_a (lr_backward). keep: take the
+        larger workspace that keeps a segment's stage inputs (faster, the same
+        gradient) where the device has the memory for it."""
         import torch
         n = len(self.models)
         g = np.ascontiguousarray(np.asarray(d_eps_a, dtype=np.float64).reshape(n))
         sz = C.c_size_t()
-        self._check(self._lib.lr_backward_workspace_size(self._h, int(ckpt_every), C.byref(sz)))
-        ws = torch.empty(int(sz.value) + 256, dtype=torch.uint8, device=self.device)
+        ws = None
+        if keep:
+            self._check(self._lib.lr_backward_workspace_size_kept(self._h, int(ckpt_every), C.byref(sz)))
+            try:
+                ws = torch.empty(int(sz.value) + 256, dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                pass
+        if ws is None:
+            self._check(self._lib.lr_backward_workspace_size(self._h, int(ckpt_every), C.byref(sz)))
+            ws = torch.empty(int(sz.value) + 256, dtype=torch.uint8, device=self.device)
         ptr = (ws.data_ptr() + 255) // 256 * 256
         out = np.zeros((n, 8))
         self._check(self._lib.lr_backward(self._h, C.c_void_p(ptr), sz, g.ctypes.data_as(C.c_void_p),
