@@ -76,7 +76,7 @@ typedef enum {
   LR_ERR_CUDA = 2,        /* a CUDA runtime call or kernel launch failed */
   LR_ERR_NOMEM = 3,       /* host allocation failed */
   LR_ERR_WORKSPACE = 4,   /* no workspace bound, or it is too small or misaligned */
-  LR_ERR_NOT_PD = 5,      /* Gram matrix Z^dag Z not positive definite (Cholesky breakdown) */
+  LR_ERR_NOT_PD = 5,      /* Gram matrix Z^dag Z not positive definite: see lr_precision */
   LR_ERR_NONFINITE = 6,   /* NaN/Inf reached the state or the readout signal */
   LR_ERR_TIMEOUT = 7,     /* a device-side wait exceeded its iteration budget */
   LR_ERR_STATE = 8,       /* call out of order (e.g. integrate before set_pulse) */
@@ -104,7 +104,15 @@ typedef enum {
  * accumulation): the reduced-precision variant, for measuring its error;
  * only for batches whose operand tiles fit in shared memory (else
  * LR_ERR_UNSUPPORTED).
- * The PLAIN engine runs FP64 only. */
+ * The PLAIN engine runs FP64 only.
+ *
+ * LR_ERR_NOT_PD: the k-th pivot of the elimination of Z^dag Z (k = 0, 1, ... in column
+ * order) counts as zero when it is not above k 2^-51 of its diagonal entry in the PLAIN
+ * engine, the gradient and the sparse engine's FP64 launches (what rounding leaves of a
+ * dependent column), and when it is not above 1e-13 of it or is below 1e-30 in the FUSED
+ * engine (either schedule) and the sparse engine's FP32_G64 contexts. AUTO picks
+ * the engine by the size of the batch, so a nearly dependent FP64 state may be refused in
+ * a large batch and accepted in a small one. */
 typedef enum { LR_PREC_FP64 = 0, LR_PREC_FP32_G64 = 1, LR_PREC_FP32 = 2, LR_PREC_TF32_G64 = 3 } lr_precision;
 
 /* PLAIN: straightforward HBM-resident kernels, several launches per RK4

@@ -115,7 +115,7 @@ struct DwArith {
     return dw_norm(DW{r, r * fmaf(e, e, e)});
   }
   static __device__ __forceinline__ R one() { return R{1.f, 0.f}; }
-  static __device__ __forceinline__ bool breakdown(C p, float d0) {
+  static __device__ __forceinline__ bool breakdown(C p, float d0, int) {
     return !(p.re.hi > 1e-13f * d0) || !isfinite(p.re.hi) || p.re.hi < 1e-30f;
   }
 };
@@ -146,7 +146,7 @@ struct F64Arith {
     return r * fma(-p.x, r, 2.0);
   }
   static __device__ __forceinline__ R one() { return 1.0; }
-  static __device__ __forceinline__ bool breakdown(C p, double d0) {
+  static __device__ __forceinline__ bool breakdown(C p, double d0, int) {
     return !(p.x > 1e-13 * d0) || !isfinite(p.x) || p.x < 1e-30;
   }
 };
@@ -200,7 +200,7 @@ __device__ __forceinline__ void mm_invert(typename A::C (&g)[2], typename A::C* 
   auto leave = [&](int q, int k) {
     if (ej[q] == k) {
       if (ei[q] == k) {
-        const bool bad = A::breakdown(g[q], d0[q]);
+        const bool bad = A::breakdown(g[q], d0[q], k);
         if (bad) sh.bad = 1;
         sh.rec[k & 1] = bad ? A::one() : A::recip(g[q]);
         sh.col[k & 1][k] = A::minus_one();
@@ -273,14 +273,14 @@ __device__ __forceinline__ void tri_entry(int e, int& i, int& j) {
 constexpr int ST = 544;   // threads of the solve kernels: one entry of the 32 x 32 triangle each
 
 // The FP64 entry arithmetic of the sweeps; a pivot counts as zero where it is lost in
-// the rounding of M updates of its diagonal entry (LR_MAX_RANK 2^-51 of it), so that a
-// rank-deficient state is told whatever the sign of that rounding.
+// the rounding of the k updates of its diagonal entry so far (k 2^-51 of it), so that a
+// rank-deficient state is told whatever the sign of that rounding and any other is taken.
 struct WidePivot : F64Arith {
   static __device__ __forceinline__ double recip(double2 p) {
     return p.x > 1e-30 && p.x < 1e30 ? F64Arith::recip(p) : 1.0 / p.x;
   }
-  static __device__ __forceinline__ bool breakdown(double2 p, double d0) {
-    return !(p.x > LR_MAX_RANK * 0x1p-51 * d0) || !isfinite(p.x);
+  static __device__ __forceinline__ bool breakdown(double2 p, double d0, int k) {
+    return !(p.x > k * 0x1p-51 * d0) || !isfinite(p.x);
   }
 };
 // Entries of G and T from their FP64 sums. FP32 state: G in double-word FP32 and an FP32

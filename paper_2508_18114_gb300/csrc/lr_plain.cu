@@ -277,7 +277,7 @@ __device__ __forceinline__ double* drive_slot(double* P, int M, int c) { return 
 // take one SM 31k cycles at M = 20: 28 us in FP64, 16 us in double-word FP32 (two
 // trajectories, M = 20, cold caches). It replaces a Cholesky factorisation and two
 // triangular sweeps over 2 M columns in one block, ~70 barriers of FP64 latency.
-// A: WidePivot, or DwArith for the FP32 state of the wide schedule.
+// A: WidePivot; in the wide schedule F64Arith, or DwArith for the FP32 state.
 // StepRef: the step and the record are the device counter's.
 template <typename A>
 __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, double2* __restrict__ Gi, long step, int stage,
@@ -639,7 +639,9 @@ cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk,
 // complex64 state the double-word Gram and M x M phase. The buffers of p are the caller's.
 template <typename T2>
 static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s) {
-  using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, WidePivot>::type;
+  // the team kernel's arithmetic and limits of a pivot: one context refuses the same
+  // states whichever schedule it runs
+  using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, F64Arith>::type;
   T2* Z[4] = {reinterpret_cast<T2*>(p.Zn), reinterpret_cast<T2*>(p.Za), reinterpret_cast<T2*>(p.Zb),
               reinterpret_cast<T2*>(p.Za)};
   const dim3 ggrid(max_nblk, rp.n_traj);
