@@ -117,7 +117,11 @@ typedef enum { LR_PREC_FP64 = 0, LR_PREC_FP32_G64 = 1, LR_PREC_FP32 = 2, LR_PREC
 
 /* PLAIN: straightforward HBM-resident kernels, several launches per RK4
  * stage (the reference GPU path). FUSED: one persistent launch per
- * integrate call, state resident on chip. AUTO picks FUSED when supported,
+ * integrate call, state resident on chip; batches far smaller than the GPU
+ * (FP64, FP32_G64) run the wide schedule instead, four launches per RK4 stage
+ * over the whole chip in the same arithmetic, where that is faster for one
+ * context at a time. LR_FUSED_WIDE = 0 / 1 at lr_create forces either: 0 is the faster
+ * one for several such contexts on streams of their own. AUTO picks FUSED when supported,
  * except for FP64 contexts whose fused plan needs teams of more than two CTAs
  * per trajectory (batches far smaller than the GPU), which run PLAIN. */
 typedef enum { LR_ENGINE_AUTO = 0, LR_ENGINE_PLAIN = 1, LR_ENGINE_FUSED = 2 } lr_engine;
@@ -243,7 +247,9 @@ lr_status lr_grow_rank(lr_ctx* dst, const lr_ctx* src, uint64_t seed, double eps
  *
  * CUDA graphs (FUSED engine): the call may be captured into a CUDA graph on
  * `stream` (it then issues three kernels: the persistent integrator, the
- * eps_a epilogue and a one-thread step advance, with no copy or host sync).
+ * eps_a epilogue and a one-thread step advance, with no copy or host sync;
+ * also where a direct call takes the wide schedule, whose results differ in the
+ * last bits, unless LR_FUSED_WIDE = 1: 16 n_steps + 5 kernels).
  * The step counter lives in device memory, so every replay of the graph
  * continues the pulse run by n_steps. A replay that would pass max_steps
  * runs nothing and leaves LR_ERR_STATE for the next synchronising call.
@@ -563,8 +569,8 @@ lr_status lr_sparse_loss(lr_sparse* s, double eta, double kappa, double gamma, d
  * accumulator in a per-team L2-resident region; the Gram matrix in
  * double-word FP32 and its inverse in double-word FP32; batches far smaller
  * than the GPU run the launches of lr_sparse_create in the same arithmetic
- * where that is faster, LR_SPARSE_WIDE = 0 / 1 forces either), 0 for the four launches per RK4 stage described at
- * lr_sparse_create (FP64 contexts, or FP32_G64 with the environment variable
+ * where that is faster, except under stream capture; LR_SPARSE_WIDE = 0 / 1
+ * forces either), 0 for the launches per RK4 stage described at lr_sparse_create (FP64 contexts, or FP32_G64 with the environment variable
  * LR_SPARSE_FUSED=0 at lr_sparse_create). *team (may be NULL) = the CTAs
  * (one thread-block cluster) that share each trajectory's rows: 1 when the
  * batch has at least as many trajectories as the GPU has SMs (each CTA then

@@ -210,8 +210,8 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
   }
   const int Mp = (Mmax + 3) / 4 * 4;
   // Variants (stage state placement, tensor-core passes of the projection).
-  // Overrides for tuning and tests: LR_FUSED_WIDE = 0 / 1 (teams / wide schedule, FP32_G64 and FP64),
-  // LR_FUSED_C = cluster size, LR_FUSED_ZS =
+  // Overrides for tuning and tests: LR_FUSED_WIDE = 0 / 1 (teams / wide schedule, the latter
+  // also under capture; FP32_G64 and FP64), LR_FUSED_C = cluster size, LR_FUSED_ZS =
   // "global" keeps the stage state in L2, LR_FUSED_TC = 0 keeps the FP32_G64
   // projection on the CUDA cores (3: only the tensor-core variant).
   int force_c = 0, force_global = 0, force_tc = -1, gram_dw = 0;
@@ -346,25 +346,24 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
   }
   const bool has_wide = prec == LR_PREC_FP32_G64 || prec == LR_PREC_FP64;
   plan->wide = has_wide && !force_c && !force_global && force_tc < 0 && !gram_dw && wide_is_faster(traj, *plan);
-  if (const char* e = getenv("LR_FUSED_WIDE")) plan->wide = has_wide && atoi(e);
+  if (const char* e = getenv("LR_FUSED_WIDE")) plan->wide = has_wide && atoi(e) ? 2 : 0;
   return true;
 }
 
 size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj) {
   // order list, then global stage buffers (only without smem residency) and accumulators per team
   size_t b = order_bytes(n_traj);
-  if (plan.wide) return wide_layout(plan, n_traj, b).total;
+  const size_t wide = plan.wide ? wide_layout(plan, n_traj, b).total : 0;   // in the place of the teams' buffers
   const size_t es = plan.es;
   if (!plan.zs_smem)
     b += ((2 * (size_t)plan.R * (plan.Mp + 1) * es * plan.C * plan.n_clusters + 255) / 256) * 256;
   b += (((size_t)plan.Nmax * plan.Mp * es * plan.n_clusters + 255) / 256) * 256;
-  return b;
+  return std::max(b, wide);
 }
 
 cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratch, int n_traj) {
   cudaError_t e = cudaMemcpy(scratch, plan.order.data(), sizeof(int) * n_traj, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return e;
-  if (plan.wide) return cudaSuccess;
   const size_t es = prec == LR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const SmemLayout L = layout(plan.R, plan.Mp, plan.zs_smem, es, plan.tc, plan.gram_mode == 2);
   const void* kern = kernel_ptr(prec, plan.zs_smem, plan.tc, plan.frame, plan.gram_mode);
@@ -374,8 +373,9 @@ cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratc
 }
 
 cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunParams& rp, lr_precision prec,
-                            long step0, long n_steps, cudaStream_t s) {
-  if (plan.wide) {
+                            long step0, long n_steps, int capturing, cudaStream_t s) {
+  // a capture holds the teams' one kernel: the wide schedule is 16 nodes a step
+  if (plan.wide == 2 || (plan.wide && !capturing)) {
     const WideLayout L = wide_layout(plan, rp.n_traj, order_bytes(rp.n_traj));
     char* sc = static_cast<char*>(p.scratch);
     DevPtrs q = p;

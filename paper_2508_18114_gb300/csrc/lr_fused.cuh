@@ -31,6 +31,7 @@ struct FusedPlan {
   int gram_mode;   // 0 native (bulk type), 1 double-word FP32 (FP64-class), 2 on the tensor cores (FP64-class)
   int es;          // bytes per complex state element
   int wide;        // 1: the wide schedule (a few launches per stage over the whole chip) in place of the teams
+                   // (which a capture takes all the same), 2: in a capture too
   int max_nblk;    // its row blocks, state elements and partial sums (doubles)
   long long tot, part;
   std::vector<int> order;   // trajectories by team: c, c + n_clusters, ... for team c
@@ -45,6 +46,6 @@ size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj);
 // makes no host-to-device copy and can be captured in a CUDA graph.
 cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratch, int n_traj);
 cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunParams& rp, lr_precision prec,
-                            long step0, long n_steps, cudaStream_t s);
+                            long step0, long n_steps, int capturing, cudaStream_t s);
 
 }  // namespace lr

@@ -583,7 +583,8 @@ struct lr_sparse {
   int fp32;   // 1: FP32_G64 state arithmetic
   int fused;  // 1: the fused persistent kernel (FP32_G64), 0: the launches per RK4 stage
   int gram_tc;   // fused: 1 when the Gram matrix is formed on the tensor cores (rank padded to 20)
-  int wide;    // fused: 1 when the whole-chip launches are faster than the teams
+  int wide;    // fused: 1 when the whole-chip launches are faster than the teams (which a capture takes
+               // all the same), 2: in a capture too
   int n_cta;   // fused: persistent CTAs (n_team teams of team_c)
   int n_team, team_c;   // fused: teams (one trajectory at a time each), CTAs per team
   size_t o_fsc;   // fused: per-CTA stage buffers
@@ -988,7 +989,7 @@ extern "C" lr_status lr_sparse_create(const lr_sparse_model* m, int n_traj, int 
       fused_teams(s, sms);
       s->wide = !getenv("LR_SPARSE_FUSED") && !getenv("LR_SPARSE_C") && !getenv("LR_SPARSE_SPLIT") && !gram_env &&
                 wide_is_faster(s, sms);
-      if (const char* we = getenv("LR_SPARSE_WIDE")) s->wide = atoi(we) != 0;
+      if (const char* we = getenv("LR_SPARSE_WIDE")) s->wide = atoi(we) ? 2 : 0;
     } else {
       cudaGetLastError();
     }
@@ -1142,7 +1143,11 @@ extern "C" lr_status lr_sparse_integrate(lr_sparse* s, double dt, long n_steps, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const SpDev d = dev(s);
   const SpParams p = params(s);
-  if (s->fused && !s->wide) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return cuda_fail(s, cudaGetLastError());
+  // a capture holds the fused kernel: the launches are 21 nodes a step
+  const bool wide = s->wide == 2 || (s->wide && cap == cudaStreamCaptureStatusNone);
+  if (s->fused && !wide) {
     const SfSmem L = sf_smem(s->M, s->K, s->gram_tc);
     cudaError_t e0 = raise_fused_smem(L.total);
     if (e0 != cudaSuccess) return cuda_fail(s, e0);
@@ -1237,6 +1242,10 @@ extern "C" lr_status lr_sparse_integrate(lr_sparse* s, double dt, long n_steps, 
       if (e1 != cudaSuccess) return cuda_fail(s, e1);
     }
   } else if (s->fp32) {
+    if (s->fused) {   // the fused kernel keeps Z_n alone
+      const cudaError_t e1 = cudaMemcpyAsync(d.Zs, d.Z, state_bytes(s), cudaMemcpyDeviceToDevice, st);
+      if (e1 != cudaSuccess) return cuda_fail(s, e1);
+    }
     launch_step_kernels<float2>(s, d, p, s->step, n_steps, dt, st);
   } else {
     launch_step_kernels<double2>(s, d, p, s->step, n_steps, dt, st);
