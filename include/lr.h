@@ -38,7 +38,10 @@
  * by lr_destroy. The library never allocates device memory: every device
  * buffer lives in one caller-owned workspace (e.g. a torch tensor's storage)
  * bound with lr_bind_workspace, which must stay alive and unmodified while
- * the context uses it. Host buffers passed to the calls are owned by the
+ * the context uses it. (Long runs of small batches are CUDA graphs, whose nodes the
+ * driver holds: a context keeps at most four, without memory for one the same
+ * kernels are launched one by one, and lr_destroy, which frees them, may
+ * wait for the device.) Host buffers passed to the calls are owned by the
  * caller and only read/written during the call.
  *
  * Errors: every call returns an lr_status; nothing crosses the ABI as an
@@ -118,10 +121,11 @@ typedef enum { LR_PREC_FP64 = 0, LR_PREC_FP32_G64 = 1, LR_PREC_FP32 = 2, LR_PREC
 /* PLAIN: straightforward HBM-resident kernels, several launches per RK4
  * stage (the reference GPU path). FUSED: one persistent launch per
  * integrate call, state resident on chip; batches far smaller than the GPU
- * (FP64, FP32_G64) run the wide schedule instead, four launches per RK4 stage
- * over the whole chip in the same arithmetic, where that is faster for one
- * context at a time. LR_FUSED_WIDE = 0 / 1 at lr_create forces either: 0 is the faster
- * one for several such contexts on streams of their own. AUTO picks FUSED when supported,
+ * (FP64, FP32_G64) run the wide schedule instead, four kernels per RK4 stage
+ * over the whole chip in the same arithmetic, where that is faster: as launches up to
+ * 62 steps, beyond that as one device-side loop (a CUDA graph that the context keeps; a
+ * call of any length only enqueues it, and runs of several contexts on streams
+ * of their own overlap). LR_FUSED_WIDE = 0 / 1 at lr_create forces either. AUTO picks FUSED when supported,
  * except for FP64 contexts whose fused plan needs teams of more than two CTAs
  * per trajectory (batches far smaller than the GPU), which run PLAIN. */
 typedef enum { LR_ENGINE_AUTO = 0, LR_ENGINE_PLAIN = 1, LR_ENGINE_FUSED = 2 } lr_engine;
@@ -568,9 +572,9 @@ lr_status lr_sparse_loss(lr_sparse* s, double eta, double kappa, double gamma, d
  * lr_sparse_integrate; the stage input, the operator images and the RK4
  * accumulator in a per-team L2-resident region; the Gram matrix in
  * double-word FP32 and its inverse in double-word FP32; batches far smaller
- * than the GPU run the launches of lr_sparse_create in the same arithmetic
- * where that is faster, except under stream capture; LR_SPARSE_WIDE = 0 / 1
- * forces either), 0 for the launches per RK4 stage described at lr_sparse_create (FP64 contexts, or FP32_G64 with the environment variable
+ * than the GPU run the kernels of lr_sparse_create in the same arithmetic
+ * where that is faster (from 50 steps as one device-side loop), except under
+ * stream capture; LR_SPARSE_WIDE = 0 / 1 forces either), 0 for the launches per RK4 stage described at lr_sparse_create (FP64 contexts, or FP32_G64 with the environment variable
  * LR_SPARSE_FUSED=0 at lr_sparse_create). *team (may be NULL) = the CTAs
  * (one thread-block cluster) that share each trajectory's rows: 1 when the
  * batch has at least as many trajectories as the GPU has SMs (each CTA then

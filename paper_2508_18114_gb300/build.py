@@ -19,6 +19,11 @@ BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr"]
+RDC = ("lr_loop.cu",)   # uses the device runtime library (cudadevrt)
+
+
+def _flags(src: str):
+    return FLAGS + (["-rdc=true"] if os.path.basename(src) in RDC else [])
 
 
 def nvcc() -> str:
@@ -34,7 +39,7 @@ def sources():
 
 def _compile(src: str, extra) -> str:
     obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
-    cmd = [nvcc(), *ARCH, *FLAGS, *extra, "-c", src, "-o", obj]
+    cmd = [nvcc(), *ARCH, *_flags(src), *extra, "-c", src, "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
@@ -47,7 +52,7 @@ def build(verbose: bool = False, extra=()) -> str:
     with cf.ThreadPoolExecutor(max_workers=min(len(srcs), os.cpu_count() or 4)) as ex:
         objs = list(ex.map(lambda s: _compile(s, list(extra)), srcs))
     tmp = OUT + ".tmp"
-    cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs, "-lcudart"]
+    cmd = [nvcc(), *ARCH, "-Xcompiler", "-fPIC", "-shared", "-o", tmp, *objs, "-lcudart", "-lcudadevrt"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("link failed:\n%s\n%s" % (r.stdout, r.stderr))
@@ -62,7 +67,7 @@ def ptxas_report() -> str:
     os.makedirs(BUILD, exist_ok=True)
     out = []
     for src in sources():
-        cmd = [nvcc(), *ARCH, *FLAGS, "-Xptxas", "-v", "-c", src, "-o", os.devnull]
+        cmd = [nvcc(), *ARCH, *_flags(src), "-Xptxas", "-v", "-c", src, "-o", os.devnull]
         r = subprocess.run(cmd, capture_output=True, text=True)
         out.append(r.stderr)
     return "\n".join(out)

@@ -20,6 +20,7 @@ struct lr_ctx {
   lr_options opt{};
   lr_engine engine = LR_ENGINE_PLAIN;
   std::vector<TrajDev> traj;
+  lr::LoopCache loops;
   std::vector<PulseDev> pulses;
   int nt_max = 0, max_N = 0, max_M = 0, max_nblk = 0;
   long n_rec = 0;
@@ -472,7 +473,7 @@ lr_status lr_integrate(lr_ctx* c, double dt, long n_steps, void* stream) {
   if (c->engine == LR_ENGINE_PLAIN)
     e = lr::plain_integrate(p, rp, c->max_nblk, c->max_N, c->step, n_steps, s);
   else
-    e = lr::fused_integrate(c->fused, p, rp, c->opt.precision, c->step, n_steps, cap != cudaStreamCaptureStatusNone, s);
+    e = lr::fused_integrate(c->fused, p, rp, c->opt.precision, c->step, n_steps, cap != cudaStreamCaptureStatusNone, c->loops, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "integrate launch");
   c->step += n_steps;
   e = lr::launch_eps_a(p, rp, n_steps, s);

@@ -146,7 +146,10 @@ double assign_teams(const std::vector<double>& t, int n, std::vector<int>* order
 // Measured, teams / wide: N = 2000, M = 20, 1 candidate 62 / 47, 2 candidates 62 / 61;
 // N = 480, M = 32 (two modes) 202 / 62, 8 candidates 203 / 114; N = 8000, M = 32 269 /
 // 148; N = 2000, M = 10 32 / 35; N = 40, M = 4 10 / 28. The line lies at 0.9, where no
-// measured batch lost more than 1%.
+// measured batch lost more than 1%. Both sides launched from the host; in the device loop
+// of a long run the wide schedule takes less (N = 2000, M = 20: 38), and contexts side by side
+// on streams of their own too (teams / wide, us a stage of all: 2 contexts 63 / 46, 4
+// contexts 63 / 57, 8 contexts 123 / 119).
 bool wide_is_faster(const std::vector<TrajDev>& traj, const FusedPlan& plan) {
   double wide = 0.0;
   std::vector<double> team;
@@ -164,7 +167,7 @@ bool wide_is_faster(const std::vector<TrajDev>& traj, const FusedPlan& plan) {
 
 // Wide schedule: two stage buffers and the accumulator, X_k, partial sums, from `off`.
 struct WideLayout {
-  size_t za, zb, acc, x, part, total;
+  size_t za, zb, acc, x, part, loop, total;
 };
 WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
   auto take = [&](size_t bytes) {
@@ -178,6 +181,7 @@ WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
   L.acc = take(plan.es * (size_t)plan.tot);
   L.x = take(sizeof(double2) * 2 * LR_MAX_RANK * LR_MAX_RANK * n_traj);
   L.part = take(sizeof(double) * plan.part);
+  L.loop = take(3 * sizeof(long long));
   L.total = off;
   return L;
 }
@@ -373,7 +377,7 @@ cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratc
 }
 
 cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunParams& rp, lr_precision prec,
-                            long step0, long n_steps, int capturing, cudaStream_t s) {
+                            long step0, long n_steps, int capturing, LoopCache& loops, cudaStream_t s) {
   // a capture holds the teams' one kernel: the wide schedule is 16 nodes a step
   if (plan.wide == 2 || (plan.wide && !capturing)) {
     const WideLayout L = wide_layout(plan, rp.n_traj, order_bytes(rp.n_traj));
@@ -384,7 +388,8 @@ cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunPa
     q.acc = sc + L.acc;
     q.X = reinterpret_cast<double2*>(sc + L.x);
     q.part = reinterpret_cast<double*>(sc + L.part);
-    return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, prec != LR_PREC_FP64, s);
+    return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, prec != LR_PREC_FP64,
+                          LoopRef{&loops, capturing ? nullptr : reinterpret_cast<long long*>(sc + L.loop)}, s);
   }
   const size_t es = prec == LR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const SmemLayout L = layout(plan.R, plan.Mp, plan.zs_smem, es, plan.tc, plan.gram_mode == 2);

@@ -46,6 +46,6 @@ size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj);
 // makes no host-to-device copy and can be captured in a CUDA graph.
 cudaError_t fused_prepare(const FusedPlan& plan, lr_precision prec, void* scratch, int n_traj);
 cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunParams& rp, lr_precision prec,
-                            long step0, long n_steps, int capturing, cudaStream_t s);
+                            long step0, long n_steps, int capturing, LoopCache& loops, cudaStream_t s);
 
 }  // namespace lr

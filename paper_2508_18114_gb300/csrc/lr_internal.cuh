@@ -256,6 +256,42 @@ cudaError_t launch_convert(const void* src, void* dst, long long n, int to_fp32,
 cudaError_t launch_diagnostics(const DevPtrs& p, const RunParams& rp, long n_valid, double* purity, double* eig,
                                cudaStream_t s);
 
+// lr_loop.cu: steps of a context as one graph launch. The body enqueues `per` steps; they
+// run for c[0] = first, first + per, .. below first + n. They read their number from c[0]
+// and the steps of the whole call from c[2].
+struct LoopCount {
+  long long first, n, call;
+};
+// A context's loops: the graph of a body is kept, for at most LOOP_KEPT (dt, tau, counter)
+// at a time, because destroying one waits for the device. One context is not used by two
+// threads, and launches of one graph run one after the other on any streams.
+constexpr int LOOP_KEPT = 4;
+struct LoopCache {
+  struct Entry {
+    double dt, tau;
+    const long long* c;
+    cudaGraphExec_t exec;
+  } e[LOOP_KEPT];
+  int n = 0, next = 0;
+  LoopCache() = default;
+  LoopCache(const LoopCache&) = delete;
+  ~LoopCache();
+};
+struct LoopRef {   // a context's loops and the counter (3 x 8 bytes) in its workspace; c null (a capture): host launches
+  LoopCache* cache;
+  long long* c;
+};
+// Nothing is enqueued on s unless cudaSuccess is returned.
+cudaError_t device_loop_run(LoopRef loop, double dt, double tau, LoopCount count, long per,
+                            cudaError_t (*body)(void*, cudaStream_t), void* arg, cudaStream_t s);
+template <typename F>
+cudaError_t device_loop(LoopRef loop, double dt, double tau, LoopCount count, long per, F body, cudaStream_t s) {
+  return device_loop_run(loop, dt, tau, count, per,
+                         [](void* f, cudaStream_t st) { return (*static_cast<F*>(f))(st); }, &body, s);
+}
+// Launches from which a run is a device loop: about the depth of the launch queue.
+constexpr long LOOP_LAUNCHES = 1000;
+
 // lr_plain.cu
 int plain_rows_per_block();
 size_t plain_partial_doubles(int M);
@@ -265,7 +301,7 @@ cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk,
 // Its kernels as the wide schedule of the fused engine: n_steps from the device's step
 // counter p.dstep; p.Za, p.Zb, p.acc, p.X and p.part in its scratch.
 cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, int fp32,
-                           cudaStream_t s);
+                           LoopRef loop, cudaStream_t s);
 // single kernels of the plain engine (used by the adjoint's recomputation)
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const double2* zin, cudaStream_t s);
 void plain_gram_launch(const DevPtrs& p, const RunParams& rp, int max_nblk, const float2* zin, cudaStream_t s);

@@ -104,6 +104,11 @@ size_t plain_partial_doubles(int M) { return pstride(M); }
 struct StepRef {
   const long long* dstep = nullptr;
   long k = 0, n = 0;
+  const long long* loop = nullptr;   // device loop: k counts from loop[0], and n is loop[2]
+  __device__ __forceinline__ long at() const { return loop ? (long)loop[0] + k : k; }
+  __device__ __forceinline__ bool fits(long max_steps) const {
+    return *dstep >= 0 && *dstep + (loop ? (long)loop[2] : n) <= max_steps;
+  }
 };
 
 template <typename T2>
@@ -208,7 +213,7 @@ __global__ void __launch_bounds__(PT) plain_gram(const TrajDev* __restrict__ tra
       out[2 * e + 1] = (double)im;
     }
   }
-  if (with_obs && sr.dstep) with_obs = (*sr.dstep + sr.k) % pop_every == 0;
+  if (with_obs && sr.dstep) with_obs = (*sr.dstep + sr.at()) % pop_every == 0;
   if (with_obs) {
     for (int i = threadIdx.x; i < PR; i += blockDim.x) {
       double w = 0.0;
@@ -283,12 +288,11 @@ template <typename A>
 __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, double2* __restrict__ Gi, long step, int stage,
                                                   int record, int do_solve, double t, StepRef sr) {
   if (sr.dstep) {
-    const long s0 = (long)*sr.dstep;
-    if (s0 < 0 || s0 + sr.n > rp.max_steps) {   // every launch of the schedule leaves
+    if (!sr.fits(rp.max_steps)) {   // every launch of the schedule leaves
       if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_error(p.err, DEV_CAPACITY);
       return;
     }
-    step = s0 + sr.k;
+    step = (long)*sr.dstep + sr.at();
     record = stage == 0 && step % rp.pop_every == 0;
     t = __dadd_rn(__dmul_rn((double)step, rp.dt), t);   // as the host forms it
   }
@@ -406,7 +410,7 @@ __global__ void __launch_bounds__(RT) plain_rhs(DevPtrs p, RunParams rp, const T
                                                 const double* __restrict__ ctab, int cstride, StepRef ref,
                                                 const __grid_constant__
                                                 typename Weight<typename real_of<T2>::type>::Tab sq) {
-  if (ref.dstep && (*ref.dstep < 0 || *ref.dstep + ref.n > rp.max_steps)) return;
+  if (ref.dstep && !ref.fits(rp.max_steps)) return;
   using T = typename real_of<T2>::type;
   constexpr bool f32 = sizeof(T) == 4;
   const int tj = blockIdx.y;
@@ -637,8 +641,11 @@ cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk,
 
 // The wide schedule of the fused engine: the step counter on the device, for the
 // complex64 state the double-word Gram and M x M phase. The buffers of p are the caller's.
+constexpr long LOOP_STEPS = 4;   // steps in the body of a device loop
+
 template <typename T2>
-static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, cudaStream_t s) {
+static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, LoopRef loop,
+                          cudaStream_t s) {
   // the team kernel's arithmetic and limits of a pivot: one context refuses the same
   // states whichever schedule it runs
   using A = typename std::conditional<sizeof(T2) == sizeof(float2), DwArith, F64Arith>::type;
@@ -646,24 +653,43 @@ static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, i
               reinterpret_cast<T2*>(p.Za)};
   const dim3 ggrid(max_nblk, rp.n_traj);
   const double c[4] = {0.0, 0.5 * rp.dt, 0.5 * rp.dt, rp.dt};
-  for (long k = 0; k <= n_steps; ++k) {
-    const StepRef ref{p.dstep, k, n_steps};
-    for (int stage = 0; stage < (k < n_steps ? 4 : 1); ++stage) {
-      const int solve = k < n_steps;
-      plain_gram<T2><<<ggrid, PT, 0, s>>>(p.traj, Z[stage], p.part, stage == 0, ref, rp.pop_every, sq_table());
-      plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 ? LR_MAX_NT + 1 : 0, s);
-      plain_solve<A><<<dim3(solve_blocks(rp, solve), rp.n_traj), ST, 0, s>>>(p, rp, nullptr, 0, stage, 0, solve, c[stage],
-                                                                             ref);
-      if (solve) rhs_launch(p, rp, max_N, Z[stage], stage < 3 ? Z[stage + 1] : nullptr, stage, nullptr, 0, ref, s);
+  // step k, or step lp[0] + k of a device loop; the last one records only
+  auto step = [&](long k, const long long* lp, bool last, cudaStream_t st) {
+    const StepRef ref{p.dstep, k, n_steps, lp};
+    for (int stage = 0; stage < (last ? 1 : 4); ++stage) {
+      plain_gram<T2><<<ggrid, PT, 0, st>>>(p.traj, Z[stage], p.part, stage == 0, ref, rp.pop_every, sq_table());
+      plain_reduce_launch(p.traj, rp.n_traj, LR_MAX_RANK, p.part, 6, stage == 0 ? LR_MAX_NT + 1 : 0, st);
+      plain_solve<A><<<dim3(solve_blocks(rp, !last), rp.n_traj), ST, 0, st>>>(p, rp, nullptr, 0, stage, 0, !last, c[stage],
+                                                                              ref);
+      if (!last) rhs_launch(p, rp, max_N, Z[stage], stage < 3 ? Z[stage + 1] : nullptr, stage, nullptr, 0, ref, st);
     }
-    const cudaError_t e = cudaGetLastError();
+    return cudaGetLastError();
+  };
+  long k = 0;
+  if (loop.c && 16 * n_steps >= LOOP_LAUNCHES) {
+    const long n = n_steps - n_steps % LOOP_STEPS;
+    const cudaError_t e = device_loop(loop, rp.dt, rp.tau, LoopCount{0, n, n_steps}, LOOP_STEPS, [&](cudaStream_t st) {
+      for (long i = 0; i < LOOP_STEPS; ++i) {
+        const cudaError_t ei = step(i, loop.c, false, st);
+        if (ei != cudaSuccess) return ei;
+      }
+      return cudaSuccess;
+    }, s);
+    if (e == cudaSuccess)
+      k = n;
+    else
+      cudaGetLastError();   // no memory for the graph, say: the same launches from the host
+  }
+  for (; k <= n_steps; ++k) {
+    const cudaError_t e = step(k, nullptr, k == n_steps, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 cudaError_t wide_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, int fp32,
-                           cudaStream_t s) {
-  return fp32 ? wide_t<float2>(p, rp, max_nblk, max_N, n_steps, s) : wide_t<double2>(p, rp, max_nblk, max_N, n_steps, s);
+                           LoopRef loop, cudaStream_t s) {
+  return fp32 ? wide_t<float2>(p, rp, max_nblk, max_N, n_steps, loop, s)
+              : wide_t<double2>(p, rp, max_nblk, max_N, n_steps, loop, s);
 }
 
 }  // namespace lr

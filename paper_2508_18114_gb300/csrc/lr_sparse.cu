@@ -106,9 +106,17 @@ struct SpParams {
   double wd, tau;
   long max_steps, n_rec;
   int pop_every;
+  const long long* base;   // device loop: the first step of this round of its body (null: none)
 };
 
 enum : int { MODE_SOLVE = 1, MODE_OBS = 2, MODE_BETA = 4 };
+
+// Stage 0 of a recording step records the populations, photons and trace too.
+__device__ __forceinline__ int record_mode(const SpParams& p, int mode, long& step) {
+  if (!(mode & MODE_BETA)) return mode;
+  if (p.base) step += (long)*p.base;
+  return step % p.pop_every == 0 ? mode | MODE_OBS : mode;
+}
 
 template <typename T2> __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
   return mk2<T2>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -140,6 +148,7 @@ __device__ __forceinline__ void dw_acc(DWs& s, float a, float b) {
 // stage times t, t + dt/2, t + dt/2, t + dt of CHI_STEPS steps (one thread per
 // factor: ~10 us of FP64 latency, whatever their number).
 __global__ void __launch_bounds__(64) sp_chi(SpDev d, SpParams p, long step, double dt) {
+  if (p.base) step += (long)*p.base;
   const int tj = blockIdx.x, c = threadIdx.x;
   if (c >= 4 * NCH) return;
   const int stage = c / NCH, ch = c - stage * NCH;
@@ -254,7 +263,8 @@ constexpr int ACC_MAX = (1 + LR_SPARSE_MAX_JUMPS) * LR_MAX_RANK * LR_MAX_RANK / 
 
 // NACC: accumulators per thread, >= (M (M + 1) / 2 + K M^2) / SP_T (4, 8 or ACC_MAX)
 template <typename T2, int NACC>
-__global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode) {
+__global__ void __launch_bounds__(SP_T) sp_gram(SpDev d, SpParams p, int mode, long step) {
+  mode = record_mode(p, mode, step);
   using T = typename Scalar<T2>::type;
   constexpr int R = rows_per_block<T2>();
   __shared__ T2 sZ[R][LR_MAX_RANK], sY[LR_SPARSE_MAX_JUMPS + 1][R][LR_MAX_RANK];
@@ -412,6 +422,7 @@ __global__ void __launch_bounds__(SP_T) sp_reduce(SpDev d, SpParams p, int lo, i
 // plain_solve, the same phase of the bare-mode engine).
 template <typename A>
 __global__ void __launch_bounds__(ST) sp_solve(SpDev d, SpParams p, long step, int mode) {
+  mode = record_mode(p, mode, step);
   __shared__ typename A::C Gs[LR_MAX_RANK * (LR_MAX_RANK + 1)];
   __shared__ short2 tri[LR_MAX_RANK * (LR_MAX_RANK + 1) / 2];
   __shared__ MmShared<A> mm;
@@ -590,6 +601,8 @@ struct lr_sparse {
   size_t o_fsc;   // fused: per-CTA stage buffers
   size_t o_fvala, o_fdiag;   // fused: values of A without its static diagonal, and that diagonal (hi + lo)
   size_t o_fflag;   // fused: [T] hand-over flags of the split schedule
+  size_t o_loop;    // fused: step counter of a device loop
+  lr::LoopCache loops;
   long nnz, max_steps, n_rec, step;
   double dt;   // RK4 step of the run (0 before the first integrate)
   int pop_every;
@@ -663,6 +676,7 @@ void layout(lr_sparse* s) {
     const size_t Mp = (size_t)(s->M + 3) / 4 * 4;
     s->o_fsc = take((size_t)s->n_team * (3 + s->K) * s->N * Mp * sizeof(float2));
     s->o_fflag = take((size_t)s->T * sizeof(int));
+    s->o_loop = take(3 * sizeof(long long));
   }
   s->total = o;
 }
@@ -766,7 +780,8 @@ void fused_teams(lr_sparse* s, int sms) {
 //   wide:  26 + 0.75 M + 4.3e-6 x T N M (M + 11).
 // Measured, teams / wide: N = 2000, M = 20, 1 pulse 57 / 48, 2 pulses 57 / 56, 4 pulses
 // 114 / 74, 8 pulses 153 / 110, 20 pulses 168 / 224; N = 3600, M = 32 174 / 96; N = 120,
-// M = 4 16 / 29. The line lies at 0.9: no measured batch above it was slower wide.
+// M = 4 16 / 29. The line lies at 0.9: no measured batch above it was slower wide. Both sides
+// launched from the host; in the device loop of a long run one pulse takes 36.
 bool wide_is_faster(const lr_sparse* s, int sms) {
   if (s->T >= sms) return false;   // one CTA per trajectory fills the chip
   const double w = s->M * (s->M + 11.0);
@@ -810,56 +825,73 @@ size_t state_bytes(const lr_sparse* s) {
 }
 
 template <typename T2>
-void launch_gram(const lr_sparse* s, const SpDev& d, const SpParams& p, int mode, cudaStream_t st) {
+void launch_gram(const lr_sparse* s, const SpDev& d, const SpParams& p, int mode, long step, cudaStream_t st) {
   const dim3 gg((unsigned)s->nblk, (unsigned)s->T);
   const int per = (s->M * (s->M + 1) / 2 + s->K * s->M * s->M + SP_T - 1) / SP_T;
   if (per <= 4)
-    sp_gram<T2, 4><<<gg, SP_T, 0, st>>>(d, p, mode);
+    sp_gram<T2, 4><<<gg, SP_T, 0, st>>>(d, p, mode, step);
   else if (per <= 8)
-    sp_gram<T2, 8><<<gg, SP_T, 0, st>>>(d, p, mode);
+    sp_gram<T2, 8><<<gg, SP_T, 0, st>>>(d, p, mode, step);
   else
-    sp_gram<T2, ACC_MAX><<<gg, SP_T, 0, st>>>(d, p, mode);
+    sp_gram<T2, ACC_MAX><<<gg, SP_T, 0, st>>>(d, p, mode, step);
 }
 
 template <typename T2>
 void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, long step0, long n_steps, double dt,
-                         cudaStream_t st) {
+                         LoopRef loop, cudaStream_t st) {
   const unsigned ab = (unsigned)(((long long)s->N * ((s->M + 3) / 4) + AT - 1) / AT);
   const int rb = SP_T / s->M;
   const dim3 gu((unsigned)((s->N + rb - 1) / rb), (unsigned)s->T);
   const int n2 = 2 * (1 + s->K) * s->M * s->M, no = n2 + 4 + s->n_levels;
   // a trajectory's share of two blocks per SM, at most eight
   const unsigned sb = (unsigned)std::max(1, std::min(8, 304 / s->T));
-  auto reduce = [&](int lo, int hi) { sp_reduce<<<dim3((hi - lo + 31) / 32, s->T), SP_T, 0, st>>>(d, p, lo, hi); };
   // the M x M phase: that of the fused kernel where these launches stand in for it, else FP64
-  auto solve = [&](unsigned blocks, long step, int mode) {
+  auto solve = [&](const SpParams& p, unsigned blocks, long step, int mode, cudaStream_t st) {
     if (s->wide)
       sp_solve<DwArith><<<dim3(blocks, s->T), ST, 0, st>>>(d, p, step, mode);
     else
       sp_solve<WidePivot><<<dim3(blocks, s->T), ST, 0, st>>>(d, p, step, mode);
   };
-  for (long i = 0; i <= n_steps; ++i) {
-    const long step = step0 + i;
-    const bool rec = step % s->pop_every == 0;
+  auto reduce = [&](const SpParams& p, int lo, int hi, cudaStream_t st) {
+    sp_reduce<<<dim3((hi - lo + 31) / 32, s->T), SP_T, 0, st>>>(d, p, lo, hi);
+  };
+  // step step0 + i, or *p.base + i of a device loop; i counts from a table of channel
+  // factors; the last one records only
+  auto one = [&](const SpParams& p, long i, bool last, cudaStream_t st) {
+    const long step = p.base ? i : step0 + i;
     const int c4 = 4 * (int)(i % CHI_STEPS);
     if (c4 == 0) sp_chi<<<dim3(s->T, CHI_STEPS), 64, 0, st>>>(d, p, step, dt);
-    if (i == n_steps) {   // observation of the final state
-      const int mode = MODE_BETA | (rec ? MODE_OBS : 0);
+    if (last) {
       sp_apply<T2><<<dim3(ab, s->T), AT, 0, st>>>(d, p, c4, 1);
-      launch_gram<T2>(s, d, p, mode, st);
-      reduce(n2, no);
-      solve(1, step, mode);
-      break;
+      launch_gram<T2>(s, d, p, MODE_BETA, step, st);
+      reduce(p, n2, no, st);
+      solve(p, 1, step, MODE_BETA, st);
+      return;
     }
     for (int stg = 0; stg < 4; ++stg) {
-      const int mode = MODE_SOLVE | (stg == 0 ? MODE_BETA | (rec ? MODE_OBS : 0) : 0);
+      const int mode = MODE_SOLVE | (stg == 0 ? MODE_BETA : 0);
       sp_apply<T2><<<dim3(ab, s->T, s->K + (stg == 0 ? 2 : 1)), AT, 0, st>>>(d, p, c4 + stg, 0);
-      launch_gram<T2>(s, d, p, mode, st);
-      reduce(0, stg == 0 ? no : n2);
-      solve(sb, step, mode);
+      launch_gram<T2>(s, d, p, mode, step, st);
+      reduce(p, 0, stg == 0 ? no : n2, st);
+      solve(p, sb, step, mode, st);
       sp_update<T2><<<gu, SP_T, 0, st>>>(d, p, stg, dt);
     }
+  };
+  long i = 0;
+  if (loop.c && 20 * n_steps >= LOOP_LAUNCHES) {
+    const long n = n_steps - n_steps % CHI_STEPS;
+    SpParams q = p;
+    q.base = loop.c;
+    const cudaError_t e = device_loop(loop, dt, p.tau, LoopCount{step0, n, n_steps}, CHI_STEPS, [&](cudaStream_t c) {
+      for (long k = 0; k < CHI_STEPS; ++k) one(q, k, false, c);
+      return cudaGetLastError();
+    }, st);
+    if (e == cudaSuccess)
+      i = n;
+    else
+      cudaGetLastError();   // no memory for the graph, say: the same launches from the host
   }
+  for (; i <= n_steps; ++i) one(p, i, i == n_steps, st);
 }
 
 SpParams params(const lr_sparse* s) {
@@ -878,6 +910,7 @@ SpParams params(const lr_sparse* s) {
   p.max_steps = s->max_steps;
   p.n_rec = s->n_rec;
   p.pop_every = s->pop_every;
+  p.base = nullptr;
   return p;
 }
 
@@ -1147,6 +1180,8 @@ extern "C" lr_status lr_sparse_integrate(lr_sparse* s, double dt, long n_steps, 
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return cuda_fail(s, cudaGetLastError());
   // a capture holds the fused kernel: the launches are 21 nodes a step
   const bool wide = s->wide == 2 || (s->wide && cap == cudaStreamCaptureStatusNone);
+  const bool may_loop = s->fused && cap == cudaStreamCaptureStatusNone;
+  const LoopRef loop{&s->loops, may_loop ? reinterpret_cast<long long*>(s->ws + s->o_loop) : nullptr};
   if (s->fused && !wide) {
     const SfSmem L = sf_smem(s->M, s->K, s->gram_tc);
     cudaError_t e0 = raise_fused_smem(L.total);
@@ -1246,9 +1281,9 @@ extern "C" lr_status lr_sparse_integrate(lr_sparse* s, double dt, long n_steps, 
       const cudaError_t e1 = cudaMemcpyAsync(d.Zs, d.Z, state_bytes(s), cudaMemcpyDeviceToDevice, st);
       if (e1 != cudaSuccess) return cuda_fail(s, e1);
     }
-    launch_step_kernels<float2>(s, d, p, s->step, n_steps, dt, st);
+    launch_step_kernels<float2>(s, d, p, s->step, n_steps, dt, loop, st);
   } else {
-    launch_step_kernels<double2>(s, d, p, s->step, n_steps, dt, st);
+    launch_step_kernels<double2>(s, d, p, s->step, n_steps, dt, loop, st);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(s, e);
