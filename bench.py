@@ -17,6 +17,7 @@ pass of the whole hot path. Inputs are seeded synthetic workloads
 from __future__ import annotations
 
 import argparse
+import contextlib
 import json
 import math
 import os
@@ -229,7 +230,40 @@ def oracle_sample(wl, n_steps, candidates=(0,)):
     return ntraj * n_steps / dt, dt, ntraj
 
 
-def full_pulse_error(wl, info, dev):
+class plan_of:
+    """The environment in which a batch of another size takes the launch plan of a timed
+    one: the wide schedule, or the teams that ``env`` names."""
+
+    def __init__(self, var, wide, env):
+        self.env = {var: "1"} if wide else dict(env, **{var: "0"})
+
+    def __enter__(self):
+        self.saved = {k: os.environ.get(k) for k in self.env}
+        os.environ.update(self.env)
+
+    def __exit__(self, *exc):
+        for k, v in self.saved.items():
+            if v is None:
+                os.environ.pop(k, None)
+            else:
+                os.environ[k] = v
+
+
+def fused_plan(info, wide, prec):
+    env = {"LR_FUSED_C": str(info.team_size)}
+    if prec == "fp32_g64":
+        env.update({"LR_FUSED_ZS": "smem" if info.stage_in_smem else "global",
+                    "LR_FUSED_TC": str(info.tensor_passes), "LR_FUSED_GRAM": "tc" if info.gram_tc else "dw"})
+    return plan_of("LR_FUSED_WIDE", wide, env)
+
+
+def plan_text(info, wide):
+    return "wide schedule" if wide else ("team %d, stage state %s, tensor passes %d, gram on tensor cores %d"
+                                         % (info.team_size, "shared memory" if info.stage_in_smem else "L2",
+                                            info.tensor_passes, info.gram_tc))
+
+
+def full_pulse_error(wl, info, wide, dev):
     """Errors of the timed launch plan over the whole pulse against the FP64
     oracle's full-pulse values (tests/golden/full_pulse_c4.txt, written by the
     oracle-only script beside it): the golden candidates of this workload run
@@ -243,13 +277,10 @@ def full_pulse_error(wl, info, dev):
     gold = full_pulse.load("c4")
     cands = sorted(gold["cands"])
     sub = [wl.candidates[c] for c in cands]
-    saved = {k: os.environ.get(k) for k in ("LR_FUSED_C", "LR_FUSED_ZS", "LR_FUSED_TC", "LR_FUSED_GRAM")}
-    os.environ.update({"LR_FUSED_C": str(info.team_size), "LR_FUSED_ZS": "smem" if info.stage_in_smem else "global",
-                       "LR_FUSED_TC": str(info.tensor_passes), "LR_FUSED_GRAM": "tc" if info.gram_tc else "dw"})
-    try:
+    with fused_plan(info, wide, "fp32_g64"):
         b = LowRankBatch([c.model for c in sub], [c.M for c in sub], precision="fp32_g64", engine="fused",
                          max_steps=wl.n_steps, pop_every=gold["rec_every"], eta=wl.eta, device=dev)
-        q = b.query()
+        q, qw = b.query(), b.wide
         b.set_pulse([(c.pulse.kind, c.pulse.p) for c in sub], wl.tau)
         b.set_initial(wl.init_seed, wl.eps)
         t0 = time.perf_counter()
@@ -258,18 +289,10 @@ def full_pulse_error(wl, info, dev):
         ion, _ = b.loss()
         sec = time.perf_counter() - t0
         b.close()
-    finally:
-        for k, v in saved.items():
-            if v is None:
-                os.environ.pop(k, None)
-            else:
-                os.environ[k] = v
     obs["pop_every"] = gold["rec_every"]
     e = full_pulse.errors(gold, obs, cands, eps_a=obs["eps_a"], ion=ion)
-    e.update({"sample": "candidates %s of this workload, g and e, all %d RK4 steps (tau = %g ns), plan: team %d, "
-                        "stage state %s, tensor passes %d (%.1f s)"
-                        % (cands, wl.n_steps, wl.tau, q.team_size, "shared memory" if q.stage_in_smem else "L2",
-                           q.tensor_passes, sec),
+    e.update({"sample": "candidates %s of this workload, g and e, all %d RK4 steps (tau = %g ns), plan: %s (%.1f s)"
+                        % (cands, wl.n_steps, wl.tau, plan_text(q, qw), sec),
               "eps_a": [float(x) for x in obs["eps_a"]],
               "eps_a_oracle": [gold["cands"][c]["eps_a"] for c in cands]})
     return e
@@ -381,8 +404,10 @@ def run_ours(args):
         b.integrate(wl.dt, chunk)
     b.sync()
     # the fused engine's integrate is timed as a captured CUDA graph, replayed
-    # once per bench step (each replay continues the pulse run)
-    graph = b.capture_integrate(wl.dt, chunk) if b.engine == "fused" and not args.no_graph else None
+    # once per bench step (each replay continues the pulse run); a batch of the wide
+    # schedule by direct calls (a capture would record the teams)
+    wide = b.wide
+    graph = b.capture_integrate(wl.dt, chunk) if b.engine == "fused" and not wide and not args.no_graph else None
     sampler = ClockSampler(local)
     if dist:
         dist.barrier()
@@ -428,13 +453,13 @@ def run_ours(args):
     # Those captures predate the 32-byte stage-state accesses of the current kernel, so the
     # line's traffic is null and the last capture's figure is reported beside it.
     traffic, traffic_last = None, None
-    if (wl.name == "c4" and prec == "fp32_g64" and engine == "fused" and info.team_size == 2
+    if (wl.name == "c4" and prec == "fp32_g64" and engine == "fused" and not wide and info.team_size == 2
             and not info.stage_in_smem and info.tensor_passes == 0):
         per = TRAFFIC_GRAM_TC if info.gram_tc else 2.532e6
         traffic_last = per * ntraj * chunk if per else None
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic, "traffic_last_capture": traffic_last,
-                "kernel": "integrate (%s engine)" % engine,
+                "kernel": "integrate (wide schedule)" if wide else "integrate (%s engine)" % engine,
                 "peak_source": "%s pipe: 152 SMs x %d FMA/clk x 2 x %.0f MHz sampled SM clock (unit counts)"
                                % (pipe, FP64_FMA_PER_CLK if prec == "fp64" else FP32_FMA_PER_CLK, mhz),
                 "flops_per_step": fl}
@@ -443,10 +468,11 @@ def run_ours(args):
     roofline["frac_of_measured"] = achieved / pm if pm else None
     roofline["peak_measured_source"] = ("lr_measure_peak: %s chains, 8 CTAs x 256 threads per SM, CUDA events, "
                                         "after the timed region" % ("DFMA" if prec == "fp64" else "FFMA"))
-    # kernels per bench step: the integrator's (plain: 3 per RK4 stage pair and
-    # records; fused: one persistent launch), the eps_a epilogue and the step advance
-    if engine == "plain":
-        launches = (16 * chunk + 3) + 2
+    # kernels per bench step: the integrator's (plain and wide: 4 per RK4 stage and 3 for the
+    # last record, from 63 steps wide also the loop's, one per 4 steps; fused: one
+    # persistent launch), the eps_a epilogue and the step advance
+    if engine == "plain" or wide:
+        launches = (16 * chunk + 3) + 2 + (1 + chunk // 4 if wide and 16 * chunk >= 1000 else 0)
     else:
         launches = 3
     launches *= args.steps
@@ -502,7 +528,7 @@ def run_ours(args):
     err = None
     full = None
     if rank == 0 and not args.no_full_pulse and wl.name == "c4" and prec == "fp32_g64" and engine == "fused":
-        full = full_pulse_error(wl, info, dev)
+        full = full_pulse_error(wl, info, wide, dev)
     if rank == 0 and not args.no_cpu_baseline:
         from oracle import parallel
         ns = args.cpu_steps or default_cpu_steps(wl)
@@ -511,18 +537,18 @@ def run_ours(args):
         dt_cpu = time.perf_counter() - t0
         cpu = {"value": 2 * ns / dt_cpu, "unit": "traj*steps/s", "cores": 2, "kind": "oracle",
                "sample": "%d RK4 steps of the g and e trajectories of candidate 0 (%.1f s)" % (ns, dt_cpu)}
-        # accuracy of this path on the same sample, against the FP64 oracle
-        bq = LowRankBatch([cands[0].model], [cands[0].M], precision=prec, engine=args.engine, max_steps=ns,
-                          pop_every=ns, eta=wl.eta, device=dev, frame=wl.frame)
+        # accuracy of the timed plan on the same sample, against the FP64 oracle
+        with fused_plan(info, wide, prec) if engine == "fused" else contextlib.nullcontext():
+            bq = LowRankBatch([cands[0].model], [cands[0].M], precision=prec, engine=engine, max_steps=ns,
+                              pop_every=ns, eta=wl.eta, device=dev, frame=wl.frame)
         bq.set_pulse([(cands[0].pulse.kind, cands[0].pulse.p)], wl.tau)
         bq.set_initial(wl.init_seed, wl.eps)
         bq.integrate(wl.dt, ns)
         og = bq.observables()
-        qinfo = bq.query()
+        qplan = plan_text(bq.query(), bq.wide) if engine == "fused" else "%s engine" % engine
         bq.close()
         bo = ora["beta"]
-        err = {"sample": "candidate 0, g and e, %d RK4 steps (team %d, tensor passes %d, gram on tensor cores %d)"
-                         % (ns, qinfo.team_size, qinfo.tensor_passes, qinfo.gram_tc),
+        err = {"sample": "candidate 0, g and e, %d RK4 steps (%s)" % (ns, qplan),
                "beta_rel": float(np.abs(og["beta"] - bo).max() / np.abs(bo).max()),
                "pops_abs": float(max(np.abs(og["pops"][j][:, :ora["pops"][j].shape[1]] - ora["pops"][j]).max()
                                      for j in range(2))),
@@ -531,9 +557,10 @@ def run_ours(args):
     if rank == 0:
         desc = workload_desc(wl, prec)
         desc.update({"parallelism": "dp%d (independent replicas)" % world, "engine": engine,
-                     "team_size": info.team_size, "stage_state": "shared memory" if info.stage_in_smem else "L2",
-                     "projection": ("tcgen05 TF32 x%d" % info.tensor_passes) if info.tensor_passes else "CUDA cores",
-                     "gram": ("tcgen05 bf16 slices (exact), double-word sums" if info.gram_tc else
+                     "schedule": "wide" if wide else "teams" if engine == "fused" else None,
+                     "team_size": 0 if wide else info.team_size, "stage_state": "shared memory" if info.stage_in_smem and not wide else "L2",
+                     "projection": ("tcgen05 TF32 x%d" % info.tensor_passes) if info.tensor_passes and not wide else "CUDA cores",
+                     "gram": ("tcgen05 bf16 slices (exact), double-word sums" if info.gram_tc and not wide else
                               "double-word FP32 on the CUDA cores" if prec in ("fp32_g64", "tf32_g64") else prec),
                      "chunk_rk4_steps": chunk,
                      "launch": "CUDA graph replay" if graph is not None else "direct lr_integrate",
@@ -542,7 +569,7 @@ def run_ours(args):
             "metric": "traj_steps_per_s", "value": value, "unit": "traj*steps/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": DTYPE_GRAM_TC if info.gram_tc else DTYPE_LABEL[prec],
+            "dtype": DTYPE_GRAM_TC if info.gram_tc and not wide else DTYPE_LABEL[prec],
             "data": "synthetic (seeded pulses and initial states)", "config": desc,
             "pulse_evals_per_s": value / (2 * spp),
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
@@ -682,11 +709,13 @@ def run_paper(args):
     peak = SMS * fma_clk * 2 * mhz * 1e6 / 1e12
     achieved = fl / (ms * 1e-3 / args.steps) / 1e12
     team = b.team
-    split = b.fused and team == 1 and T > torch.cuda.get_device_properties(dev).multi_processor_count \
+    wide = b.wide
+    fused = b.fused and not wide
+    split = fused and team == 1 and T > torch.cuda.get_device_properties(dev).multi_processor_count \
         and os.environ.get("LR_SPARSE_SPLIT", "1") != "0"
     kname = (("sf_kernel (fused persistent sparse kernel, one launch per integrate; %s)"
               % ("equal spans of trajectory-steps per CTA" if split else "%d CTA(s) per trajectory" % team))
-             if b.fused else "integrate (sparse engine, 5 launches per RK4 stage)")
+             if fused else "integrate (sparse engine, 5 kernels per RK4 stage)")
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": None, "kernel": kname,
                 "peak_source": "%s FMA pipe: 152 SMs x %d FMA/clk x 2 x %.0f MHz sampled SM clock (unit counts)"
@@ -696,8 +725,10 @@ def run_paper(args):
     roofline["frac_of_measured"] = achieved / pm if pm else None
     # fused: one integrate launch and sp_loss per bench step; launch path: per RK4 step
     # 4 x (apply, gram, reduce, solve, update), sp_chi every eight steps, the closing
-    # observation pass apply, gram, reduce, solve, then sp_loss
-    launches = (2 if b.fused else 20 * chunk + chunk // 8 + 1 + 4 + 1) * args.steps
+    # observation pass apply, gram, reduce, solve, then sp_loss; wide from 50 steps also the
+    # loop's, one per eight steps
+    launches = (2 if fused else 20 * chunk + chunk // 8 + 1 + 4 + 1
+                + (1 + chunk // 8 if wide and 20 * chunk >= 1000 else 0)) * args.steps
 
     e2e = None
     if not args.no_e2e:
@@ -724,12 +755,14 @@ def run_paper(args):
         v, dt_cpu, ora = paper_oracle_sample(wl, model_o, ns, traj=1, dt=dt)
         cpu = {"value": v, "unit": "traj*steps/s", "cores": 1, "kind": "oracle",
                "sample": "%d RK4 steps of trajectory 1 (candidate 0, |e>) (%.1f s)" % (ns, dt_cpu)}
-        bq = sparse.SparseBatch(model, wl.M, pulses[:2], wl.tau, ns, pop_every=ns, device=dev, precision=prec)
+        with (plan_of("LR_SPARSE_WIDE", wide, {"LR_SPARSE_C": str(team)}) if b.fused else contextlib.nullcontext()):
+            bq = sparse.SparseBatch(model, wl.M, pulses[:2], wl.tau, ns, pop_every=ns, device=dev, precision=prec)
         bq.set_initial([0, 1], wl.init_seed, wl.eps)
         bq.integrate(dt, ns)
         og = bq.observables()
         bo = ora["beta"]
-        err = {"sample": "candidate 0, |e>, %d RK4 steps" % ns,
+        err = {"sample": "candidate 0, |e>, %d RK4 steps (%s)"
+                         % (ns, "wide schedule" if bq.wide else "team %d" % bq.team if bq.fused else "launches"),
                "beta_rel": float(np.abs(og["beta"][1] - bo).max() / np.abs(bo).max()),
                "pops_abs": float(np.abs(og["pops"][1] - ora["pops"]).max())}
         del bq
@@ -739,7 +772,7 @@ def run_paper(args):
             "metric": "traj_steps_per_s", "value": value, "unit": "traj*steps/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f64" if prec == "fp64" else (DTYPE_GRAM_TC if b.fused and b.gram_tc else
+            "dtype": "f64" if prec == "fp64" else (DTYPE_GRAM_TC if fused and b.gram_tc else
                                                    ("f32 bulk; double-word f32 (~2^-48) Gram, G^-1 "
                                                     "and X_k; f64 signal") if b.fused else
                                                    "f32 bulk; double-word f32 (~2^-48) Gram; f64 G^-1, "
@@ -751,11 +784,12 @@ def run_paper(args):
                                       else "frame of the drive, counter-rotating terms kept", model["N"],
                                       "x".join(map(str, wl.dims)), wl.M, dt, wl.tau, prec),
                        "trajectories": T, "N": model["N"], "M": wl.M, "nnz": int(model["nnz"]),
-                       "engine": "sparse (fused persistent kernel)" if b.fused else "sparse (five launches per stage)",
-                       "gram": ("tcgen05 bf16 slices (exact), double-word sums" if b.fused and b.gram_tc else
+                       "engine": "sparse (fused persistent kernel)" if fused else "sparse (five kernels per stage)",
+                       "gram": ("tcgen05 bf16 slices (exact), double-word sums" if fused and b.gram_tc else
                                 "double-word FP32 on the CUDA cores" if prec != "fp64" else "f64"),
                        "schedule": (("equal spans of the batch's trajectory-steps, one per CTA" if split else
-                                     "teams of %d CTA(s), one trajectory at a time" % team) if b.fused else None),
+                                     "teams of %d CTA(s), one trajectory at a time" % team) if fused else
+                                    "wide" if wide else None),
                        "chunk_rk4_steps": chunk,
                        "parallelism": "dp%d (independent replicas)" % world,
                        "l2": "flushed (256 MiB write) between timed steps"},

@@ -366,6 +366,10 @@ lr_status lr_backward(lr_ctx* ctx, void* dev_ws, size_t ws_bytes, const double* 
                       int ckpt_every, void* stream);
 
 lr_status lr_query(const lr_ctx* ctx, lr_info* info);
+/* *wide = 1 when direct lr_integrate calls of a FUSED context run the wide schedule (see
+ * lr_engine); team_size .. gram_tc of lr_info then describe the teams that a stream
+ * capture records. 0 otherwise. */
+lr_status lr_query_schedule(const lr_ctx* ctx, int* wide);
 
 /* No-allocation entry point (the paper has no counterpart; this is a
  * deployment convenience).
@@ -586,6 +590,10 @@ lr_status lr_sparse_loss(lr_sparse* s, double eta, double kappa, double gamma, d
  * lr_sparse_create, rank padded to 20), 0 for the double-word CUDA-core
  * sums (the default). */
 lr_status lr_sparse_query(const lr_sparse* s, int* fused, int* team, int* gram_tc);
+/* *wide = 1 when lr_sparse_integrate of a fused context runs the kernels of
+ * lr_sparse_create over the whole chip (*team and *gram_tc of lr_sparse_query then
+ * describe the kernel that a stream capture records), 0 otherwise. */
+lr_status lr_sparse_query_schedule(const lr_sparse* s, int* wide);
 const char* lr_sparse_last_error(const lr_sparse* s);
 void lr_sparse_destroy(lr_sparse* s);
 

@@ -632,6 +632,12 @@ lr_status lr_backward(lr_ctx* c, void* dev_ws, size_t ws_bytes, const double* d_
   return check_device_error(c);
 }
 
+lr_status lr_query_schedule(const lr_ctx* c, int* wide) {
+  if (!c || !wide) return LR_ERR_ARG;
+  *wide = c->engine == LR_ENGINE_FUSED && c->fused.wide;
+  return LR_OK;
+}
+
 lr_status lr_query(const lr_ctx* c, lr_info* info) {
   if (!c || !info) return LR_ERR_ARG;
   info->n_cand = c->n_cand;

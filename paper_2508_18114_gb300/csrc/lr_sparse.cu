@@ -1351,6 +1351,12 @@ extern "C" lr_status lr_sparse_query(const lr_sparse* s, int* fused, int* team, 
   return LR_OK;
 }
 
+extern "C" lr_status lr_sparse_query_schedule(const lr_sparse* s, int* wide) {
+  if (!s || !wide) return LR_ERR_ARG;
+  *wide = s->fused && s->wide;
+  return LR_OK;
+}
+
 extern "C" const char* lr_sparse_last_error(const lr_sparse* s) { return s ? s->msg.c_str() : "null context"; }
 
 extern "C" void lr_sparse_destroy(lr_sparse* s) { delete s; }

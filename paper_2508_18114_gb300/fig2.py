@@ -126,12 +126,13 @@ def run(steps=80000, dt=5e-4, M=20, every=100, amp_mhz=150.0, dims=(100, 4, 5), 
                                        device=device)
                 b.set_initial(lvs, seed, eps)
                 _, sec = timed(lambda: b.integrate(h, n))
-                runs[name] = (b.observables(), sec, b.team if b.fused else 0)
+                runs[name] = (b.observables(), sec, ("wide schedule" if b.wide else "fused, %d CTA(s) per trajectory" % b.team) if b.fused else
+                              "five kernels per stage")
                 del b
-            o, sec, team = runs["together"]
+            o, sec, engine = runs["together"]
             key = "lra_%s%s" % (prec, sfx)
             out["runs"][key] = {
-                "engine": ("fused, %d CTA(s) per trajectory" % team) if team else "four launches per stage",
+                "engine": engine,
                 "seconds_g_and_e_together": sec,
                 "seconds_per_trajectory_alone": [runs["g"][1], runs["e"][1]] if "g" in runs else None,
                 "eps_a": assignment_error(o["beta"][0], o["beta"][1], h, P["kappa"], P["gamma"])}

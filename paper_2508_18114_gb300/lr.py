@@ -42,7 +42,7 @@ EXPORTS = (
     "lr_sparse_destroy", "lr_grow_rank", "lr_measure_peak", "lr_sparse_query",
     "lr_full_create", "lr_full_workspace_size", "lr_full_bind_workspace", "lr_full_set_initial",
     "lr_full_set_state", "lr_full_set_state_lowrank", "lr_full_get_state", "lr_full_integrate", "lr_full_observables", "lr_full_last_error",
-    "lr_full_destroy", "lr_assignment_shots",
+    "lr_full_destroy", "lr_assignment_shots", "lr_query_schedule", "lr_sparse_query_schedule",
 )
 
 
@@ -101,6 +101,8 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.lr_observables.argtypes = [vp, vp, vp, vp, vp, vp, vp]
     lib.lr_sync.argtypes = [vp, vp]
     lib.lr_query.argtypes = [vp, C.POINTER(lr_info)]
+    lib.lr_query_schedule.argtypes = [vp, C.POINTER(C.c_int)]
+    lib.lr_sparse_query_schedule.argtypes = [vp, C.POINTER(C.c_int)]
     lib.lr_status_string.argtypes = [i]
     lib.lr_status_string.restype = C.c_char_p
     lib.lr_last_error.argtypes = [vp]
@@ -263,6 +265,14 @@ class LowRankBatch:
     @property
     def engine(self) -> str:
         return ENGINE_NAME[self.query().engine]
+
+    @property
+    def wide(self) -> bool:
+        """True when integrate() runs the wide schedule in place of the teams that
+        query() describes (and capture_integrate() records)."""
+        w = C.c_int()
+        self._check(self._lib.lr_query_schedule(self._h, C.byref(w)))
+        return bool(w.value)
 
     @property
     def n_traj(self) -> int:

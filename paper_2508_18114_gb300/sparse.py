@@ -105,10 +105,19 @@ class SparseBatch:
 
     @property
     def fused(self) -> bool:
-        """True when the context runs the fused persistent kernel."""
+        """True when the context has the fused persistent kernel (which a small batch
+        does not run: see ``wide``)."""
         f = C.c_int()
         self._check(self._lib.lr_sparse_query(self._h, C.byref(f), None, None))
         return bool(f.value)
+
+    @property
+    def wide(self) -> bool:
+        """True when integrate() of a fused context runs the kernels over the whole chip
+        in place of the fused kernel."""
+        w = C.c_int()
+        self._check(self._lib.lr_sparse_query_schedule(self._h, C.byref(w)))
+        return bool(w.value)
 
     @property
     def gram_tc(self) -> bool:
@@ -119,7 +128,7 @@ class SparseBatch:
 
     @property
     def team(self) -> int:
-        """CTAs per trajectory of the fused kernel (0: the four-launch path)."""
+        """CTAs per trajectory of the fused kernel (0: a context without it)."""
         f, t = C.c_int(), C.c_int()
         self._check(self._lib.lr_sparse_query(self._h, C.byref(f), C.byref(t), None))
         return t.value
