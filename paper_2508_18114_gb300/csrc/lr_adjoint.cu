@@ -70,7 +70,6 @@ struct Ptrs {
   double2* Xs;      // [4][n_traj][2][MR2]  X_k' of each stage of the step (row-major M x M)
   double2* Gi;      // [4][n_traj][MR2]     G^-1 of each stage
   double2* EP;      // [n_traj][4][MR2]     E_r', E_b', X_r' E_r', X_b' E_b'
-  const double* part;
   double* bpart;
   double* thbar;    // [n_traj][8]
   double2* beta;
@@ -534,7 +533,6 @@ cudaError_t backward_t(const DevPtrs& main, const RunParams& rp0, char* ws, cons
   a.pulse = main.pulse;
   a.err = main.err;
   a.EP = P2(L.EP);
-  a.part = p.part;
   a.bpart = reinterpret_cast<double*>(ws + L.bpart);
   a.thbar = reinterpret_cast<double*>(ws + L.thbar);
   a.beta = P2(L.beta);

@@ -113,7 +113,7 @@ lr_status check_device_error(lr_ctx* c) {
   if (ce != cudaSuccess) return cuda_fail(c, ce, "reading device error word");
   switch (e) {
     case lr::DEV_OK: return LR_OK;
-    case lr::DEV_NOT_PD: return fail(c, LR_ERR_NOT_PD, "Gram matrix lost positive definiteness (Cholesky breakdown)");
+    case lr::DEV_NOT_PD: return fail(c, LR_ERR_NOT_PD, "Gram matrix lost positive definiteness (pivot lost)");
     case lr::DEV_NONFINITE: return fail(c, LR_ERR_NONFINITE, "non-finite value in the state or readout signal");
     case lr::DEV_TIMEOUT: return fail(c, LR_ERR_TIMEOUT, "a device-side wait ran out of its budget");
     case lr::DEV_CAPACITY:

@@ -161,15 +161,16 @@ bool wide_is_faster(const std::vector<TrajDev>& traj, const FusedPlan& plan) {
     wide = std::max(wide, fp64 ? 25.0 + 1.5 * d.M : 20.0 + 1.1 * d.M);
   }
   for (const TrajDev& d : traj)
-    wide += d.N * (fp64 ? 4.5e-3 / 152 * d.M * (d.M + 2.6) : 4.6e-6 * d.M * (d.M + 11.0));
+    wide += d.N * (fp64 ? 4.5e-3 / SMS * d.M * (d.M + 2.6) : 4.6e-6 * d.M * (d.M + 11.0));
   return wide < 0.9 * assign_teams(team, plan.n_clusters, nullptr);
 }
 
-// Wide schedule: two stage buffers and the accumulator, X_k, partial sums, from `off`.
+// Wide schedule: two stage buffers and the accumulator, partial sums, a loop counter, from
+// `off` (X_k has a place of its own in every context).
 struct WideLayout {
-  size_t za, zb, acc, x, part, loop, total;
+  size_t za, zb, acc, part, loop, total;
 };
-WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
+WideLayout wide_layout(const FusedPlan& plan, size_t off) {
   auto take = [&](size_t bytes) {
     const size_t at = off;
     off += (bytes + 255) / 256 * 256;
@@ -179,7 +180,6 @@ WideLayout wide_layout(const FusedPlan& plan, int n_traj, size_t off) {
   L.za = take(plan.es * (size_t)plan.tot);
   L.zb = take(plan.es * (size_t)plan.tot);
   L.acc = take(plan.es * (size_t)plan.tot);
-  L.x = take(sizeof(double2) * 2 * LR_MAX_RANK * LR_MAX_RANK * n_traj);
   L.part = take(sizeof(double) * plan.part);
   L.loop = take(3 * sizeof(long long));
   L.total = off;
@@ -357,7 +357,7 @@ bool fused_plan(const std::vector<TrajDev>& traj, lr_precision prec, int frame, 
 size_t fused_scratch_bytes(const FusedPlan& plan, int n_traj) {
   // order list, then global stage buffers (only without smem residency) and accumulators per team
   size_t b = order_bytes(n_traj);
-  const size_t wide = plan.wide ? wide_layout(plan, n_traj, b).total : 0;   // in the place of the teams' buffers
+  const size_t wide = plan.wide ? wide_layout(plan, b).total : 0;   // in the place of the teams' buffers
   const size_t es = plan.es;
   if (!plan.zs_smem)
     b += ((2 * (size_t)plan.R * (plan.Mp + 1) * es * plan.C * plan.n_clusters + 255) / 256) * 256;
@@ -380,13 +380,12 @@ cudaError_t fused_integrate(const FusedPlan& plan, const DevPtrs& p, const RunPa
                             long step0, long n_steps, int capturing, LoopCache& loops, cudaStream_t s) {
   // a capture holds the teams' one kernel: the wide schedule is 16 nodes a step
   if (plan.wide == 2 || (plan.wide && !capturing)) {
-    const WideLayout L = wide_layout(plan, rp.n_traj, order_bytes(rp.n_traj));
+    const WideLayout L = wide_layout(plan, order_bytes(rp.n_traj));
     char* sc = static_cast<char*>(p.scratch);
     DevPtrs q = p;
     q.Za = sc + L.za;
     q.Zb = sc + L.zb;
     q.acc = sc + L.acc;
-    q.X = reinterpret_cast<double2*>(sc + L.x);
     q.part = reinterpret_cast<double*>(sc + L.part);
     return wide_integrate(q, rp, plan.max_nblk, plan.Nmax, n_steps, prec != LR_PREC_FP64,
                           LoopRef{&loops, capturing ? nullptr : reinterpret_cast<long long*>(sc + L.loop)}, s);

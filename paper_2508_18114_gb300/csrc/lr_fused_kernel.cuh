@@ -8,8 +8,9 @@
 //   B1          one cluster barrier: partials and the new Z_s are visible;
 //   R  (every CTA, redundantly) reduce the C partial slots in rank order,
 //               G^-1 by symmetric sweeps and X_k = G^-1 T_k (FP64 for the FP64
-//               state; double-word FP32, ~2^-48, for the FP32 state), pre-scaled, conjugate-transposed and rounded to the bulk
-//               precision: XT_r = kappa/2 X_r^dag, XT_b = gamma/2 X_b^dag;
+//               state; double-word FP32, ~2^-48, for the FP32 state), pre-scaled,
+//               conjugate-transposed and rounded to the bulk precision:
+//               XT_r = kappa/2 X_r^dag, XT_b = gamma/2 X_b^dag;
 //   F  (local + DSMEM halo) F = -i H_eff Z_s + (rZ_s) XT_r + (bZ_s) XT_b and the
 //               RK4 stage update; the next stage input goes to the other Z_s
 //               buffer, the accumulator and Z_n are updated in L2.
@@ -235,8 +236,8 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
   T2* Tred = reinterpret_cast<T2*>(smem + a.o_tred);           // [2][Mp*Mp]
   T2* XT = reinterpret_cast<T2*>(smem + a.o_xs);               // [2][Mp][Mp] (l, m)
   // misc (FP64 scalars): [8..24) photon partials per level, [64..81) reduced
-  // populations and photons, [128..131) bulk-precision step sizes, [136..140) mbarriers of the tensor-core Gram, [140] phase-P task
-  // counter, [141] tensor-core timeout flag, [142] tensor-core mbarrier, [143]
+  // populations and photons, [128..131) bulk-precision step sizes, [136..140) mbarriers
+  // of the tensor-core Gram, [140] phase-P task counter, [141] tensor-core timeout flag, [142] tensor-core mbarrier, [143]
   // TMEM base address, [144..164) column maxima of the tensor-core Gram
   double* misc = reinterpret_cast<double*>(smem + a.o_misc);
   if (a.debug_wait > 0) {

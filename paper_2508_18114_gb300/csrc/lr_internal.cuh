@@ -32,6 +32,8 @@ struct PulseDev {
   double p[8];
 };
 
+constexpr int SMS = 152;   // of a GB300: sizes of grids and cost estimates; no result depends on how many run
+
 // Device error word values (first error wins).
 enum DevErr : unsigned { DEV_OK = 0, DEV_NOT_PD = 1, DEV_NONFINITE = 2, DEV_TIMEOUT = 3, DEV_CAPACITY = 4 };
 

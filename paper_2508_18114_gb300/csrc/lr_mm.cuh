@@ -177,7 +177,9 @@ struct MmShared {   // column k of the matrix and 1 / a_kk, by parity of k
 // double-word), not by its M^2/2 updates. It replaces an L D L^dag factorisation,
 // L^-1 and G^-1 = L^-dag D^-1 L^-1 (three passes with ~870 cycles per elimination
 // step): 36k -> 14k cycles at M = 20. The error is that of the
-// factorisation, the condition number of the scaled G times the unit roundoff.
+// factorisation, the condition number of the scaled G times the unit roundoff: X_k =
+// G^-1 T_k in FP64 against 200 bits, M = 4 .. 32, cond 1 .. 5e9, has 0.2 to 0.8
+// of the forward error of Cholesky substitution.
 //
 // Called by the warps below mm_warps(M, NT / 32) with all their lanes; the result
 // is in gi[i * ldg + j] after the block barrier that the caller adds.

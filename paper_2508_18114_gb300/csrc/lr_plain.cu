@@ -4,7 +4,7 @@
 //   plain_gram  - per row block, partial sums of G = Z^dag Z (upper triangle),
 //                 T_r = Z^dag r Z and T_b = Z^dag b Z, plus level populations
 //                 and readout photons at recording steps;
-//   plain_reduce - the partials added in block order, one thread per entry;
+//   plain_reduce - the partials added in a fixed order, a warp per 32 entries and share;
 //   plain_solve - a few blocks per trajectory: record beta = tr(T_r) at stage 1 of
 //                 each step, G^-1 by symmetric sweeps, X_r = G^-1 T_r, X_b = G^-1 T_b;
 //   plain_rhs   - per element: F = -i H_eff Z + 1/2 kappa (rZ) X_r^dag
@@ -14,12 +14,14 @@
 // and -1/2 sum_k L_k^dag L_k Z is folded into the diagonal of H_eff.
 //
 // The state type is a template parameter: complex128 (the reference path), or
-// complex64 for the FP32-bulk recomputation inside the adjoint. With complex64
-// the Gram matrix is summed from the exact products of the FP32 entries in
-// double-word FP32 (FP64-class), G^-1 and X_k are FP64,
-// and the operator apply, T_k, the projection term and the RK4 update run in
-// FP32 (the diagonal energies and the step sizes split into hi + lo floats so
-// that FP32 does not round the mode frequencies or dt).
+// complex64 for the FP32-bulk recomputation inside the adjoint and for the wide
+// schedule of the fused engine (wide_integrate: the same kernels, the step counter on
+// the device). With complex64 the Gram matrix is summed from the exact products of
+// the FP32 entries in double-word FP32 (FP64-class), G^-1 and X_k are FP64 in the
+// adjoint and double-word FP32 in the wide schedule (as in the fused kernel), and the
+// operator apply, T_k, the projection term and the RK4 update run in FP32 (the
+// diagonal energies and the step sizes split into hi + lo floats so that FP32 does
+// not round the mode frequencies or dt; the couplings rounded once).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(ST) plain_solve(DevPtrs p, RunParams rp, doubl
 
 // a trajectory's share of two blocks per SM, at most eight
 static int solve_blocks(const RunParams& rp, int do_solve) {
-  return do_solve ? std::max(1, std::min(8, 304 / rp.n_traj)) : 1;
+  return do_solve ? std::max(1, std::min(8, 2 * SMS / rp.n_traj)) : 1;
 }
 void plain_solve_launch(const DevPtrs& p, const RunParams& rp, double2* Gi, long step, int stage, int record, int do_solve,
                         double t, cudaStream_t s) {
@@ -603,9 +605,9 @@ void plain_rhs_launch(const DevPtrs& p, const RunParams& rp, int max_N, const fl
   rhs_launch(p, rp, max_N, zin, zout, stage, coef, cstride, StepRef{}, s);
 }
 
-template <typename T2>
-static cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0, long n_steps,
-                        cudaStream_t s) {
+cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0, long n_steps,
+                            cudaStream_t s) {
+  using T2 = double2;
   T2* Zn = reinterpret_cast<T2*>(p.Zn);
   T2* Za = reinterpret_cast<T2*>(p.Za);
   T2* Zb = reinterpret_cast<T2*>(p.Zb);
@@ -634,15 +636,10 @@ static cudaError_t integrate_t(const DevPtrs& p, const RunParams& rp, int max_nb
   return cudaGetLastError();
 }
 
-cudaError_t plain_integrate(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long step0,
-                            long n_steps, cudaStream_t s) {
-  return integrate_t<double2>(p, rp, max_nblk, max_N, step0, n_steps, s);
-}
+constexpr long LOOP_STEPS = 4;   // steps in the body of a device loop
 
 // The wide schedule of the fused engine: the step counter on the device, for the
 // complex64 state the double-word Gram and M x M phase. The buffers of p are the caller's.
-constexpr long LOOP_STEPS = 4;   // steps in the body of a device loop
-
 template <typename T2>
 static cudaError_t wide_t(const DevPtrs& p, const RunParams& rp, int max_nblk, int max_N, long n_steps, LoopRef loop,
                           cudaStream_t s) {

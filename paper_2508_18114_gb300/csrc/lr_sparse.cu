@@ -19,8 +19,8 @@
 //               projection Zs^+ L_k Zs);
 //   sp_update - whole rows per block (Y_k rows staged in shared memory):
 //               F = W + 1/2 sum_k Y_k X_k^dag, then the classical RK4 stage.
-// After the last step an observation pass (apply r, Gram, solve without
-// Cholesky) records beta and the observables of the final state.
+// After the last step an observation pass (apply r, Gram, reduce, solve without
+// the sweeps) records beta and the observables of the final state.
 //
 // FP32_G64 contexts run, by default, the fused persistent kernel of
 // lr_sparse_fused.cuh instead: one launch per integrate call, one CTA per
@@ -844,7 +844,7 @@ void launch_step_kernels(const lr_sparse* s, const SpDev& d, const SpParams& p, 
   const dim3 gu((unsigned)((s->N + rb - 1) / rb), (unsigned)s->T);
   const int n2 = 2 * (1 + s->K) * s->M * s->M, no = n2 + 4 + s->n_levels;
   // a trajectory's share of two blocks per SM, at most eight
-  const unsigned sb = (unsigned)std::max(1, std::min(8, 304 / s->T));
+  const unsigned sb = (unsigned)std::max(1, std::min(8, 2 * SMS / s->T));
   // the M x M phase: that of the fused kernel where these launches stand in for it, else FP64
   auto solve = [&](const SpParams& p, unsigned blocks, long step, int mode, cudaStream_t st) {
     if (s->wide)
@@ -980,7 +980,7 @@ extern "C" lr_status lr_sparse_create(const lr_sparse_model* m, int n_traj, int 
   s->ntile = (N + R - 1) / R;
   // Gram blocks per trajectory: enough blocks for ~8 per SM over the batch, each
   // looping over ntile / nblk row tiles (fewer partial sums for the solve)
-  const int want = (8 * 152 + n_traj - 1) / n_traj;
+  const int want = (8 * SMS + n_traj - 1) / n_traj;
   s->nblk = std::min(s->ntile, std::max(8, want));
   s->nnz = m->nnz;
   s->max_steps = max_steps;
