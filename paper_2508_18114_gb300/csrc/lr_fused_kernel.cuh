@@ -1022,8 +1022,10 @@ __global__ void __launch_bounds__(NTH, 1) fused_kernel(const Args a) {
               g[u] = Ar::zero();
               if (e < M * (M + 1) / 2) {
                 const int i = tri[e].x, j = tri[e].y, o = j * Mp + i;
-                // the partials in rank order, two loads in flight (four, unrolled, made the
-                // 512 trajectories of N = 2000, M = 20 1.5% slower: instruction cache)
+                // the partials in rank order, two loads in flight. Four, unrolled, made the 512
+                // trajectories of N = 2000, M = 20 1.5% slower (instruction cache); eight for
+                // teams of more than two give small batches on ten or more CTAs back the
+                // 0.3 us a stage that the exact sums cost, and take 3 us from others
                 typename Ar::Sum sum;
 #pragma unroll 1
                 for (int r0 = 0; r0 < C; r0 += 2) {

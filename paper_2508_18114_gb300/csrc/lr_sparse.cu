@@ -106,7 +106,7 @@ struct SpParams {
   double wd, tau;
   long max_steps, n_rec;
   int pop_every;
-  const long long* base;   // device loop: the first step of this round of its body (null: none)
+  const long long* base;   // device loop: the first step of this pass of its body (null: none)
 };
 
 enum : int { MODE_SOLVE = 1, MODE_OBS = 2, MODE_BETA = 4 };
